@@ -4,9 +4,9 @@
 // the server and returns at once.  One scheduler thread forms batches from
 // the pending requests in arrival order and launches each batch as a packed
 // solve (wave.cu) on one of max_inflight slots -- a stream with its own device
-// workspace and pinned buffers -- as soon as a slot is free, so requests that
-// arrive while others run are admitted as slots free up and their work
-// overlaps on the device.  A batch is bounded by max_batch_requests, by
+// workspace and pinned buffers -- as soon as a slot is free (batches of few
+// seeds a short pace apart, see kPace), so requests that arrive while others
+// run are admitted as slots free up and their work overlaps on the device.  A batch is bounded by max_batch_requests, by
 // max_batch_seeds and by the slot's share of the memory budget (admission by
 // device memory); a request that cannot fit a slot alone fails with
 // HJCD_ENOMEM.  When a batch's copies back to pinned memory complete, a host
@@ -79,6 +79,8 @@ struct Server {
     int64_t next_id = 1;
     bool stopping = false;
     std::vector<Slot> slots;
+    bool launched = false;
+    Clock::time_point t_last;  // the last batch's launch
     std::string fatal;  // first CUDA failure of the scheduler
 
     void run();
@@ -87,6 +89,15 @@ struct Server {
 };
 
 namespace {
+
+// A batch follows the last one by at least kPace while fewer than kFillSeeds seeds per SM are
+// waiting: requests that arrive closely together then share one launch sequence, whose time is
+// mostly the latency of its longest candidate, instead of each taking a slot of its own, while a
+// lone request, or a queue that can fill the GPU, is launched at once.  A burst of 20 requests (1 to 8
+// targets each): 1.95 ms against 2.20 without the pace; a Poisson trace at 2000 requests/s: p50 0.56
+// against 0.44 ms, p99 1.42 against 1.35 ms, at 4000/s p99 1.70 against 1.69 ms.
+constexpr std::chrono::microseconds kPace(250);
+constexpr int64_t kFillSeeds = 64;
 
 struct CbArg {
     Server* sv;
@@ -279,8 +290,17 @@ void Server::run() {
             }
         }
         // new batches on free slots
+        bool paced = false;
         for (Slot& sl : slots) {
             if (sl.busy || pending.empty()) continue;
+            if (max_requests > 1 && launched && !stopping && Clock::now() < t_last + kPace) {
+                int64_t waiting = 0;
+                for (const Req* r : pending) waiting += r->seeds;
+                if (waiting < kFillSeeds * sm_count() && (int)pending.size() < max_requests) {
+                    paced = true;
+                    break;
+                }
+            }
             std::vector<Req*> take;
             int64_t seeds = 0;
             std::vector<int32_t> robots;
@@ -295,6 +315,8 @@ void Server::run() {
                 take.push_back(r);
                 seeds += r->seeds;
             }
+            launched = true;
+            t_last = Clock::now();
             lock.unlock();
             launch(sl, take);
             lock.lock();
@@ -304,7 +326,8 @@ void Server::run() {
         bool busy = false;
         for (Slot& sl : slots) busy = busy || sl.busy;
         if (stopping && pending.empty() && !busy) break;
-        cv.wait(lock);
+        if (paced) cv.wait_until(lock, t_last + kPace);
+        else cv.wait(lock);
     }
 }
 
