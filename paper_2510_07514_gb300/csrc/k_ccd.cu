@@ -128,27 +128,40 @@ __device__ __forceinline__ float2 quat_angle2(float2 w, float2 vv) {
 // (cos, sin of x/2).  The only differences are those that form the residual's own components, as
 // in the direct evaluation, and the squares are summed, so the closed form is as accurate (a float32
 // emulation against the float64 method agrees to 2e-7 on Panda).
-__device__ __forceinline__ CcdTrials ccd_joint_trials(const V3 pj, const V3 z, float thj, float lo, float hi,
-                                                      const V3 Ep, const V3 pt, const Q4 qerr, float nqw,
-                                                      float dphi, float pe2, float inv_p2, float inv_o2) {
-    CcdTrials o;
+// The position step needs the end effector only: it and the joint's geometry come first
+// (CcdGeom), so that a caller can let them overlap the error quaternion's chain.
+struct CcdGeom {
+    float nup2, nvp2, nu2, ez, cs, sn, d;
+};
+__device__ __forceinline__ CcdGeom ccd_joint_geom(const V3 pj, const V3 z, const V3 Ep, const V3 pt, float pe2) {
+    CcdGeom g;
     const V3 u = Ep - pj;
     const V3 v = pt - pj;
     const float uz = dot(u, z), vz = dot(v, z);
     const V3 up = fma3(-uz, z, u);
     const V3 vp = fma3(-vz, z, v);
-    const float nup2 = dot(up, up), nvp2 = dot(vp, vp);
-    const float nu2 = fmaf(uz, uz, nup2), nv2 = fmaf(vz, vz, nvp2);
+    g.nup2 = dot(up, up);
+    g.nvp2 = dot(vp, vp);
+    g.nu2 = fmaf(uz, uz, g.nup2);
+    const float nv2 = fmaf(vz, vz, g.nvp2);
     const V3 zxu = cross(z, up);
-    const float ez = vz - uz;
+    g.ez = vz - uz;
+
+    // Eq. theta_proj, signed about the axis: atan2(z.(up x vp), up.vp) = atan2(zxu.vp, up.vp)
+    g.cs = dot(up, vp);
+    g.sn = dot(zxu, vp);
+    const bool deg = g.nu2 < 1e-24f || nv2 < 1e-24f || g.nup2 <= pe2 * g.nu2 || g.nvp2 <= pe2 * nv2;
+    g.d = deg ? 0.0f : atan2_all(g.sn, g.cs);
+    return g;
+}
+
+__device__ __forceinline__ CcdTrials ccd_joint_trials(const CcdGeom& g, const V3 z, float thj, float lo, float hi,
+                                                      const Q4 qerr, float nqw, float dphi, float inv_p2, float inv_o2) {
+    CcdTrials o;
+    const float nup2 = g.nup2, nvp2 = g.nvp2, nu2 = g.nu2, ez = g.ez, cs = g.cs, sn = g.sn, d = g.d;
     const float az = dot(qerr.v, z);
     const V3 qp = fma3(-az, z, qerr.v);
     const float qp2 = dot(qp, qp);
-
-    // Eq. theta_proj, signed about the axis: atan2(z.(up x vp), up.vp) = atan2(zxu.vp, up.vp)
-    const float cs = dot(up, vp), sn = dot(zxu, vp);
-    const bool deg = nu2 < 1e-24f || nv2 < 1e-24f || nup2 <= pe2 * nu2 || nvp2 <= pe2 * nv2;
-    const float d = deg ? 0.0f : atan2_all(sn, cs);
     // Eq. ori_update: delta(k) sgn(a.z) phi
     const float dq = (az > 0.0f) ? dphi : ((az < 0.0f) ? -dphi : 0.0f);
 
@@ -191,6 +204,32 @@ __device__ __forceinline__ CcdTrials ccd_joint_trials(const V3 pj, const V3 z, f
     o.rq = ang.y;
     o.so = sc.y;
     return o;
+}
+
+// Acceptance of theta_hat (reading: an improvement above gamma in position or in orientation):
+// its residual is the end effector at Ep and the error quaternion turned by da about the distal
+// chosen joint (origin Pa, axis Za) first, then by db about the proximal one; ep0 and eo are the
+// current errors.
+__device__ __forceinline__ bool ccd_accept_pos(float gamma, const V3 Ep, const V3 pt, float ep0, const V3 Pa, const V3 Za,
+                                               float da, const V3 Pb, const V3 Zb, float db) {
+    float sa_, ca_, sb_, cb_;
+    __sincosf(0.5f * da, &sa_, &ca_);
+    __sincosf(0.5f * db, &sb_, &cb_);
+    V3 x = Pa + rotate_half(Za, sa_, ca_, Ep - Pa);
+    x = Pb + rotate_half(Zb, sb_, cb_, x - Pb);
+    const V3 e1 = pt - x;
+    const float ep1 = sqrt_approx(dot(e1, e1));
+    return ep0 - ep1 > gamma;
+}
+__device__ __forceinline__ bool ccd_accept_ori(float gamma, const Q4 qerr, float eo, const V3 Za, float da, const V3 Zb,
+                                               float db) {
+    float sa_, ca_, sb_, cb_;
+    __sincosf(0.5f * da, &sa_, &ca_);
+    __sincosf(0.5f * db, &sb_, &cb_);
+    Q4 q1 = qmul(qerr, Q4{ca_, (-sa_) * Za});
+    q1 = qmul(q1, Q4{cb_, (-sb_) * Zb});
+    const float eo1 = quat_angle(q1.w, dot(q1.v, q1.v));
+    return eo - eo1 > gamma;
 }
 
 // One iteration of a candidate: kinematics with frames into the column, the
@@ -269,8 +308,8 @@ __device__ __forceinline__ int ccd_step(const RobotParams* rob, const RobotParam
         const float2 pa = col.a(j), pb = col.b(j), za = col.c(j);
         const V3 pj = v3(pa.x, pa.y, pb.x);
         const V3 z = v3(za.x, za.y, col.zz(j));
-        const CcdTrials tr =
-            ccd_joint_trials(pj, z, pb.y, R.lim[j].x, R.lim[j].y, E.p, pt, qerr, nqw, dphi, pe2, inv_p2, inv_o2);
+        const CcdTrials tr = ccd_joint_trials(ccd_joint_geom(pj, z, E.p, pt, pe2), z, pb.y, R.lim[j].x, R.lim[j].y, qerr,
+                                              nqw, dphi, inv_p2, inv_o2);
         if (tr.sp < best_p * one_m_tie) {  // joint 0 against +inf
             best_p = tr.sp;
             jp = j;
@@ -304,18 +343,9 @@ __device__ __forceinline__ int ccd_step(const RobotParams* rob, const RobotParam
     col.frame(p_hi ? jp : jo, Pa, Za);  // the distal joint
     col.frame(p_hi ? jo : jp, Pb, Zb);
     const float da = p_hi ? aP : aO, db = p_hi ? aO : aP;
-    float sa_, ca_, sb_, cb_;
-    __sincosf(0.5f * da, &sa_, &ca_);
-    __sincosf(0.5f * db, &sb_, &cb_);
-    V3 x = Pa + rotate_half(Za, sa_, ca_, E.p - Pa);
-    x = Pb + rotate_half(Zb, sb_, cb_, x - Pb);
-    Q4 q1 = qmul(qerr, Q4{ca_, (-sa_) * Za});
-    q1 = qmul(q1, Q4{cb_, (-sb_) * Zb});
-    const V3 e1 = pt - x;
-    const float ep1 = sqrt_approx(dot(e1, e1));
-    const float eo1 = quat_angle(q1.w, dot(q1.v, q1.v));
-    // acceptance (reading: an improvement above gamma in position or in orientation)
-    const bool acc = (ep0 - ep1 > P.cd_gamma_pos) || (eo - eo1 > P.cd_gamma_ori);
+    const bool acc_p = ccd_accept_pos(P.cd_gamma_pos, E.p, pt, ep0, Pa, Za, da, Pb, Zb, db);
+    const bool acc_o = ccd_accept_ori(P.cd_gamma_ori, qerr, eo, Za, da, Zb, db);
+    const bool acc = acc_p || acc_o;
 
     if (TRACE && kk == 0) {
         if (A.tr.jp) A.tr.jp[c] = jp;
@@ -501,6 +531,345 @@ __global__ void __launch_bounds__(TH, HJCD_CCD_THREADS_PER_SM / TH) k_ccd(const 
     }
 }
 
+// ----------------------------------------------------------------------------
+// PO-CCD with a candidate's work spread over a CTA, for batches too small to fill the GPU with one
+// thread per candidate: there the time is the latency of one candidate's chain of iterations, and a
+// thread that walks all of its joints one after another makes that chain long (a lone warp issues
+// an instruction every four cycles or so, whatever the instruction).  A CTA takes 16 candidates;
+// lanes l and l + 16 of every warp belong to candidate l, and the warps share its joints,
+// exchanging through shared memory with five barriers per iteration:
+//   1. warps 0 and 1, one half warp per row: the x, y and z rows of the kinematics chain, which never
+//      meet (a frame's row is updated from the same row only), from the joints' sines and cosines
+//   2. the last warp: flange pose, error quaternion, break test; beside it the other warps: their
+//      joints' geometry and position step, which need the end effector only
+//   3. those warps: the trials of their joints, the position trial in the lower half warp and the
+//      orientation trial in the upper one
+//   4. warps 0 and 1: greedy choice, acceptance by the position and by the orientation; beside them
+//      the others draw the perturbation that the lanes about to reject will need
+//   5. every half warp: the accepted update or the perturbation of its joints, their sines and cosines
+// The arithmetic is ccd_step's, operation by operation, so the results are its bits.  Bound by
+// latency: about 3000 cycles per iteration on Panda (kinematics rows 500, residual 890, trials 460,
+// choice and acceptance 550, update 450, the barriers the rest).  One target of 1000 seeds: 55 us for
+// at most 32 iterations, where k_ccd takes 125 us.
+constexpr int kCoopCands = 16;     // candidates per CTA
+constexpr int kCoopMaxWarps = 16;  // joint warps and the residual's
+
+struct CoopCol {  // [joint][candidate] fields, nl joints in the layout
+    int nl;
+    float4* q;     // [candidate]: error quaternion
+    float4* pick;  // [candidate]: chosen joints (jp | jo << 8), their steps, accepted by the position
+    float2* tr;    // [joint][lane]: score and step of the position (lower half) and orientation trials
+    float2* fr;    // [row][joint][candidate]: component `row` of the joint's origin and of its axis
+    float2* e;     // [row][candidate]: that component of the last frame's first two axes
+    float2* er;    // [candidate]: angle of the error quaternion, position error (0, -1: done)
+    float2* cs;    // cosine and sine of the joint angle
+    float *th, *nz;  // joint angle, normal draw
+    int* acc_o;      // [candidate]: accepted by the orientation
+    __device__ __forceinline__ void frame(int j, int l, V3& p, V3& z) const {
+        const float2 a = fr[j * kCoopCands + l], b = fr[(nl + j) * kCoopCands + l], c = fr[(2 * nl + j) * kCoopCands + l];
+        p = v3(a.x, b.x, c.x);
+        z = v3(a.y, b.y, c.y);
+    }
+};
+__host__ __device__ constexpr size_t coop_ccd_bytes(int n) {
+    return (size_t)kCoopCands * (sizeof(float4) * 2 + sizeof(float2) * (2 * n + 3 * n + 3 + 1 + n) + sizeof(float) * (2 * n + 1) +
+                                 sizeof(int));
+}
+__device__ __forceinline__ CoopCol coop_col(void* base, int nl) {
+    CoopCol C;
+    C.nl = nl;
+    C.q = reinterpret_cast<float4*>(base);
+    C.pick = C.q + kCoopCands;
+    C.tr = reinterpret_cast<float2*>(C.pick + kCoopCands);
+    C.fr = C.tr + 2 * kCoopCands * nl;
+    C.e = C.fr + kCoopCands * 3 * nl;
+    C.er = C.e + kCoopCands * 3;
+    C.cs = C.er + kCoopCands;
+    C.th = reinterpret_cast<float*>(C.cs + kCoopCands * nl);
+    C.nz = C.th + kCoopCands * nl;
+    C.acc_o = reinterpret_cast<int*>(C.nz + kCoopCands * (nl + 1));  // nz: one row more, an odd chain's last pair
+    return C;
+}
+
+// One row of the kinematics chain (fk_step's operations on that row): component `row` of every
+// joint's origin and axis, and of the last frame's other axes
+template <int N>
+__device__ __forceinline__ void coop_fk_row(const CoopCol& C, const RobotParams& R, int n, int row, int l) {
+    float c0 = row == 0 ? 1.0f : 0.0f, c1 = row == 1 ? 1.0f : 0.0f, c2 = row == 2 ? 1.0f : 0.0f, p = 0.0f;
+    float2* const fr = C.fr + row * C.nl * kCoopCands + l;
+    const float2* const csl = C.cs + l;
+    auto step = [&](int j) {
+        const float4 g = R.dh[j];
+        const float2 cs = csl[j * kCoopCands];
+        const float b1 = fmaf(g.x, c1, g.y * c2);
+        const float b2 = fmaf(g.x, c2, (-g.y) * c1);
+        p = fmaf(g.w, b2, fmaf(g.z, c0, p));
+        const float n0 = fmaf(cs.x, c0, cs.y * b1);
+        c1 = fmaf(cs.x, b1, (-cs.y) * c0);
+        c0 = n0;
+        c2 = b2;
+        fr[j * kCoopCands] = make_float2(p, c2);
+    };
+    if (N) {
+#pragma unroll
+        for (int j = 0; j < N; ++j) step(j);
+    } else {
+#pragma unroll 4
+        for (int j = 0; j < n; ++j) step(j);
+    }
+    C.e[row * kCoopCands + l] = make_float2(c0, c1);
+}
+
+// One trial of a joint: ccd_joint_trials' operations on one half of its pairs, for the step x
+__device__ __forceinline__ float2 ccd_joint_trial(const CcdGeom& g, float az, float qp2, float x, float thj, float lo,
+                                                  float hi, float qw, float inv_p2, float inv_o2) {
+    const float st = __fadd_rn(clampf(__fadd_rn(thj, x), lo, hi), -thj);
+    float sh, ch;
+    __sincosf(__fmul_rn(0.5f, st), &sh, &ch);
+    const float m2sh = __fmul_rn(-2.0f, sh);
+    const float msn = __fmul_rn(m2sh, ch);
+    const float cst = fmaf(m2sh, sh, 1.0f);
+    // both forms of the position residual (ccd_joint_trials says when the first is taken)
+    const float ra = fmaf(2.0f, fmaf(msn, g.sn, __fmul_rn(cst, -g.cs)), fmaf(g.ez, g.ez, g.nvp2 + g.nup2));
+    const float ex = fmaf(cst, -g.nup2, g.cs), ey = fmaf(msn, g.nup2, g.sn);
+    const float rb = fmaf(fmaf(ex, ex, __fmul_rn(ey, ey)), __fdividef(1.0f, g.nup2), __fmul_rn(g.ez, g.ez));
+    const float r2 = g.nup2 <= 1e-6f * g.nu2 ? ra : rb;
+    const float w = fmaf(qw, ch, __fmul_rn(sh, az));
+    const float tz = fmaf(ch, az, __fmul_rn(sh, -qw));
+    const float vv = fmaf(tz, tz, qp2);
+    // quat_angle2
+    const float ay = sqrt_approx(vv), ax = fabsf(w);
+    const float t = __fdividef(fminf(ax, ay), fmaxf(fmaxf(ax, ay), 1e-30f));
+    const float s = __fmul_rn(t, t);
+    float p = fmaf(-4.166443301e-03f, s, 2.232482877e-02f);
+    p = fmaf(p, s, -5.666722692e-02f);
+    p = fmaf(p, s, 9.704074739e-02f);
+    p = fmaf(p, s, -1.393516270e-01f);
+    p = fmaf(p, s, 1.995220255e-01f);
+    p = fmaf(p, s, -3.333036250e-01f);
+    p = fmaf(p, s, 9.999994549e-01f);
+    const float ang = ay > ax ? fmaf(__fmul_rn(-2.0f, t), p, 2.0f * 1.57079632679489662f) : __fmul_rn(__fmul_rn(2.0f, t), p);
+    return make_float2(fmaf(r2, inv_p2, __fmul_rn(__fmul_rn(ang, ang), inv_o2)), st);
+}
+
+// RED as for k_ccd; N > 0: the launch's one robot has N joints (unrolled loops); N = 0: any robots
+template <bool RED, int N>
+__global__ void __launch_bounds__(kCoopMaxWarps * 32, 1) k_ccd_coop(const CcdArgs A) {
+    extern __shared__ __align__(16) float sm[];
+    __shared__ long long s_base;
+    const RobotParams* rob = stage_robots(sm, A.rs);
+    const int WJ = ((int)blockDim.x >> 5) - 1;  // the warps that share the joints
+    const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
+    const int l = lane & (kCoopCands - 1), half = lane >> 4;
+    const CoopCol C = coop_col(reinterpret_cast<char*>(sm) + robots_smem_bytes(A.rs.n), N ? N : A.rs.n_max);
+    const hjcd_params& P = A.P;
+    const float pe2 = P.proj_eps * P.proj_eps;
+    const float one_m_tie = 1.0f - P.cd_tie;
+    unsigned long long n_it = 0, n_cand = 0;
+    auto sincos_of = [&](const RobotParams& R, int j, float th) {
+        float s, c;
+        if (RED) sincos_red(th + R.off[j], &s, &c);
+        else __sincosf(th, &s, &c);
+        return make_float2(c, s);
+    };
+
+    for (int64_t g = blockIdx.x;; g += gridDim.x) {
+        __syncthreads();  // the last group's state is no longer read
+        int64_t base = kCoopCands * g;
+        if (A.queue) {
+            if (threadIdx.x == 0) s_base = (long long)atomicAdd(A.queue, (unsigned long long)kCoopCands);
+            __syncthreads();
+            base = s_base;
+        }
+        if (base >= A.C) break;
+        const int64_t c = base + l;
+        int32_t t = 0, s = 0;
+        bool have = c < A.C;
+        if (have) have = A.map.lookup_search(c, t, s);
+        s += A.seed_base;
+        const TargetDesc T = A.tg[have ? t : 0];
+        const RobotParams& R = N ? rob[0] : rob[have ? T.robot : 0];
+        const int n = N ? N : R.n;  // (a lane without a candidate runs along on a robot's joints, unread)
+        const V3 pt = v3(T.p[0], T.p[1], T.p[2]);
+        const int cap = A.n_iters >= 0 ? A.n_iters : T.cd_iters;
+        const float inv_p2 = 1.0f / (T.eps_pos * T.eps_pos), inv_o2 = 1.0f / (T.eps_ori * T.eps_ori);
+        const bool valid = have && T.eps_pos > 0.0f;
+        bool alive = valid;
+        int iters = cap;              // the residual warp's
+        float ep2 = 0.0f, eo = 0.0f;  // the residual warp's
+        float delta_k = P.cd_delta0 * powf(P.cd_rho, (float)A.k0);
+
+        // seeds (or the caller's joint vectors), their sines and cosines
+        for (int j = 2 * warp + half; j < n; j += 2 * (WJ + 1)) {
+            float th = 0.0f;
+            if (have && A.th_in) {
+                th = A.th_in[j * A.ld + c];
+            } else if (have) {
+                const uint4 w = rnd_block(T, (uint32_t)s, kPhaseSeed, 0, (uint32_t)(j >> 2));
+                th = fmaf(u01(word(w, j & 3)), R.lim[j].y - R.lim[j].x, R.lim[j].x);
+            }
+            C.th[j * kCoopCands + l] = th;
+            C.cs[j * kCoopCands + l] = sincos_of(R, j, th);
+        }
+        __syncthreads();
+
+        for (int kk = 0;; ++kk) {
+            // 1. kinematics rows
+            if (2 * warp + half < 3) coop_fk_row<N>(C, R, n, 2 * warp + half, l);
+            __syncthreads();
+
+            // 2. residual and break test; beside it the joints' geometry.  (A candidate that is done
+            // keeps its errors and runs along: its trials are not read.)
+            Frame F;
+            {
+                const float2 r0 = C.e[l], r1 = C.e[kCoopCands + l], r2 = C.e[2 * kCoopCands + l];
+                F.c0 = v3(r0.x, r1.x, r2.x);
+                F.c1 = v3(r0.y, r1.y, r2.y);
+                C.frame(n - 1, l, F.p, F.c2);
+            }
+            const Frame E = fk_flange(R, F);
+            int j = min(warp, n - 1);
+            V3 pj{}, z{};
+            CcdGeom g0{};
+            if (warp == WJ) {
+                const Q4 qe = quat_error(T, quat_from_frame(E));
+                const V3 e = pt - E.p;
+                if (alive) {
+                    ep2 = dot(e, e);
+                    eo = quat_angle(qe.w, dot(qe.v, qe.v));
+                    if (kk > 0 && ep2 < P.cd_eps_pos2 && eo * eo < P.cd_eps_ori2) {
+                        iters = kk;
+                        alive = false;
+                    } else if (kk == cap) {
+                        alive = false;
+                    }
+                    if (half == 0) {
+                        C.q[l] = make_float4(qe.w, qe.v.x, qe.v.y, qe.v.z);
+                        C.er[l] = make_float2(eo, alive ? sqrt_approx(ep2) : -1.0f);
+                        if (alive) ++n_it;
+                    }
+                }
+            } else {
+                C.frame(j, l, pj, z);
+                g0 = ccd_joint_geom(pj, z, E.p, pt, pe2);
+            }
+            if (!__syncthreads_or(warp == WJ && alive)) break;
+
+            // 3. trials
+            const float4 q4 = C.q[l];
+            const Q4 qerr{q4.x, v3(q4.y, q4.z, q4.w)};
+            const float2 er = C.er[l];  // eo, ep
+            if (warp != WJ) {
+                alive = alive && er.y >= 0.0f;
+                const float dphi = delta_k * er.x;
+                for (;;) {
+                    const float az = dot(qerr.v, z);
+                    const V3 qp = fma3(-az, z, qerr.v);
+                    // Eq. theta_proj; Eq. ori_update
+                    const float x = half == 0 ? g0.d : ((az > 0.0f) ? dphi : ((az < 0.0f) ? -dphi : 0.0f));
+                    const float2 tr = ccd_joint_trial(g0, az, dot(qp, qp), x, C.th[j * kCoopCands + l], R.lim[j].x,
+                                                      R.lim[j].y, qerr.w, inv_p2, inv_o2);
+                    if (warp < n) C.tr[j * 32 + lane] = tr;
+                    j += WJ;
+                    if (j >= n) break;
+                    C.frame(j, l, pj, z);
+                    g0 = ccd_joint_geom(pj, z, E.p, pt, pe2);
+                }
+            }
+            __syncthreads();
+
+            // 4. greedy choice and acceptance; the perturbation's draws
+            if (warp < 2) {
+                float best = __int_as_float(0x7f800000), d = 0.0f;  // of this half's kind of trial
+                int jb = 0;
+                auto scan = [&](int j) {
+                    const float2 v = C.tr[j * 32 + lane];
+                    const bool w = v.x < best * one_m_tie;
+                    best = w ? v.x : best;
+                    jb = w ? j : jb;
+                    d = w ? v.y : d;
+                };
+                if (N) {
+#pragma unroll
+                    for (int j = 0; j < N; ++j) scan(j);
+                } else {
+#pragma unroll 4
+                    for (int j = 0; j < n; ++j) scan(j);
+                }
+                const int j2 = __shfl_xor_sync(0xffffffffu, jb, 16);
+                const float d2 = __shfl_xor_sync(0xffffffffu, d, 16);
+                const int jp = half ? j2 : jb, jo = half ? jb : j2;
+                float aP = half ? d2 : d, aO = half ? d : d2;
+                if (jp == jo) {  // the larger step
+                    if (fabsf(aP) >= fabsf(aO)) aO = 0.0f;
+                    else aP = 0.0f;
+                }
+                const bool p_hi = jp > jo;
+                V3 Pa, Za, Pb, Zb;
+                C.frame(p_hi ? jp : jo, l, Pa, Za);
+                C.frame(p_hi ? jo : jp, l, Pb, Zb);
+                const float da = p_hi ? aP : aO, db = p_hi ? aO : aP;
+                if (warp == 0) {
+                    const bool acc = ccd_accept_pos(P.cd_gamma_pos, E.p, pt, er.y, Pa, Za, da, Pb, Zb, db);
+                    C.pick[l] = make_float4(__int_as_float(jp | jo << 8), aP, aO, acc ? 1.0f : 0.0f);
+                } else {
+                    C.acc_o[l] = ccd_accept_ori(P.cd_gamma_ori, qerr, er.x, Za, da, Zb, db);
+                }
+            } else if (alive) {
+                for (int q = 2 * (warp - 2) + half; 2 * q < n; q += 2 * (WJ - 1)) {
+                    const float2 zz = normal_pair(T, (uint32_t)s, kPhaseCd, (uint32_t)(A.k0 + kk), q);
+                    C.nz[2 * q * kCoopCands + l] = zz.x;
+                    C.nz[(2 * q + 1) * kCoopCands + l] = zz.y;
+                }
+            }
+            __syncthreads();
+
+            // 5. the accepted steps, or theta + N(0, sigma^2 I) (clamped as in ccd_step); the sines and
+            // cosines of the next pass
+            {
+                const float4 pk = C.pick[l];
+                const bool acc = pk.w != 0.0f || C.acc_o[l] != 0;
+                const int jp = __float_as_int(pk.x) & 255, jo = __float_as_int(pk.x) >> 8;
+                for (int i = 2 * warp + half; i < n; i += 2 * (WJ + 1)) {
+                    const float th = C.th[i * kCoopCands + l], nz = C.nz[i * kCoopCands + l];
+                    const float lo = R.lim[i].x, hi = R.lim[i].y;
+                    const float t1 = i == jp ? clampf(th + pk.y, lo, hi) : th;
+                    const float t2 = i == jo ? clampf(t1 + pk.z, lo, hi) : t1;
+                    const float tn = acc ? t2 : clampf(fmaf(P.cd_sigma, nz, th), lo, hi);
+                    if (alive) {
+                        C.th[i * kCoopCands + l] = tn;
+                        C.cs[i * kCoopCands + l] = sincos_of(R, i, tn);
+                    }
+                }
+            }
+            delta_k *= P.cd_rho;
+            __syncthreads();
+        }
+
+        if (have && A.th_out)
+            for (int i = 2 * warp + half; i < n; i += 2 * (WJ + 1)) A.th_out[i * A.ld + c] = C.th[i * kCoopCands + l];
+        if (warp == WJ && have && half == 0) {
+            ++n_cand;
+            const float ep = sqrtf(ep2);
+            if (A.score) {
+                const float a = ep / T.eps_pos, b = eo / T.eps_ori;
+                A.score[c] = valid ? fmaf(a, a, b * b) : __int_as_float(0x7f800000);
+            }
+            if (A.perr) A.perr[c] = ep;
+            if (A.oerr) A.oerr[c] = eo;
+            if (A.iters) A.iters[c] = iters;
+        }
+    }
+    if (A.cnt && warp == WJ) {
+        n_it = warp_sum(n_it);
+        n_cand = warp_sum(n_cand);
+        if (lane == 0) {
+            atomicAdd(&A.cnt->v[0], n_it);
+            atomicAdd(&A.cnt->v[5], n_cand);
+        }
+    }
+}
+
 // cd_variant = 2, the target-wide break: one CTA per target runs all of its
 // seeds in lock-step, iteration by iteration, and stops every seed once any
 // seed passes the coarse test.  Pass kk tests each seed's state after kk
@@ -620,6 +989,25 @@ void launch_ccd_t(const CcdArgs& A, cudaStream_t st) {
     k_ccd<TRACE, TH, RED><<<g, TH, smem, st>>>(A);
 }
 
+template <bool RED, int N>
+void launch_ccd_coop_n(const CcdArgs& A, int warps, cudaStream_t st) {
+    const size_t smem = robots_smem_bytes(A.rs.n) + coop_ccd_bytes(A.rs.n_max);
+    static SmemLimit lim;
+    allow_dyn_smem(k_ccd_coop<RED, N>, lim, robots_smem_bytes(kMaxLaunchRobots) + coop_ccd_bytes(kMaxDof));
+    int per_sm = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ccd_coop<RED, N>, 32 * warps, smem);
+    const int g = (int)std::min<int64_t>((A.C + kCoopCands - 1) / kCoopCands, (int64_t)sm_count() * std::max(per_sm, 1));
+    k_ccd_coop<RED, N><<<g, 32 * warps, smem, st>>>(A);
+}
+
+template <bool RED>
+void launch_ccd_coop(const CcdArgs& A, int warps, cudaStream_t st) {
+    const int n = A.rs.n == 1 ? A.rs.n_max : 0;
+    if (n == 6) launch_ccd_coop_n<RED, 6>(A, warps, st);
+    else if (n == 7) launch_ccd_coop_n<RED, 7>(A, warps, st);
+    else launch_ccd_coop_n<RED, 0>(A, warps, st);
+}
+
 template <bool TRACE, bool RED>
 void launch_ccd_b(const CcdArgs& A, cudaStream_t st) {
     if (A.block == 64) launch_ccd_t<TRACE, 64, RED>(A, st);
@@ -639,6 +1027,20 @@ void launch_ccd(const CcdArgs& A, bool trace, cudaStream_t st) {
                        robots_smem_bytes(kMaxLaunchRobots) +
                            sizeof(float) * (kColWordsPerJoint * kMaxDof + kSlotWords) * 128);
         k_ccd_lock<128><<<A.map.T, 128, smem, st>>>(A);
+        return;
+    }
+    const bool whole = !trace && A.P.cd_variant == 0 && !A.list_in && A.seg_begin == 0 && A.seg_end == 0;
+    // Up to 64 candidates per SM (two resident CTAs of 16 on every SM, twice) the spread kernel's
+    // shorter iterations win; past that its extra work does.  Phase time, spread / one thread per candidate, us (7, 20, 24
+    // joints): 1000 candidates 55 / 125, 91 / 267, 106 / 311; 4000: 59 / 125, 118 / 269, 135 / 313;
+    // 8000: 109 / 126, 224 / 269, 258 / 313; 16000: 198 / 126, 400 / 272, 464 / 314.  Eight warps (the
+    // residual's and seven joint warps), twelve for a long chain while a CTA has its SM to itself
+    // (20 joints, 1000 candidates: 99 with eight).
+    const int64_t sms = sm_count();
+    if (whole && A.C <= sms * 4 * kCoopCands) {
+        const int warps = A.rs.n_max > 8 && A.C <= sms * kCoopCands ? 12 : 8;
+        if (A.in_limits && A.rs.plain) launch_ccd_coop<false>(A, warps, st);
+        else launch_ccd_coop<true>(A, warps, st);
         return;
     }
     if (trace) launch_ccd_b<true, true>(A, st);

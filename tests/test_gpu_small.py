@@ -1,0 +1,115 @@
+"""Small batches: the PO-CCD and PJ-IK kernels that spread a candidate's work over a CTA.
+
+They run the one-thread-per-candidate kernels' operations in the same order, so a candidate's
+results must be the same bits whether its batch is small (spread kernels) or large.  Sizes: one
+candidate, the edges of a CTA's 16, more CTAs than fit at once; chains of one joint up to the
+longest, joint tables with and without offsets.
+"""
+import numpy as np
+import pytest
+import torch
+
+from paper_2510_07514_gb300 import api, build, hjcd, inputs
+
+pytestmark = pytest.mark.gpu
+
+BIG = 24000  # candidates: more than the spread kernels take (64 per SM)
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    build.build()
+    c = api.Context(0)
+    yield c
+    c.close()
+
+
+def _robot(which):
+    if which == "offsets":  # joint offsets, limits past pi, a rotated flange
+        r = inputs.panda()
+        r.theta_off = np.linspace(-0.7, 0.9, 7)
+        r.lo, r.hi = r.lo - 1.0, r.hi + 1.5
+        c, s = np.cos(0.4), np.sin(0.4)
+        r.flange = r.flange @ np.array([[c, 0, s, 0], [0, 1, 0, 0], [-s, 0, c, 0], [0, 0, 0, 1.0]])
+        return r
+    if which.startswith("planar"):
+        return inputs.planar([0.3] * int(which[6:]))
+    if which.startswith("random"):
+        return inputs.cfg3_chains()[int(which[6:])]
+    return inputs.dof_scaling_robot(int(which[5:]))
+
+
+def _case(ctx, which, seed):
+    rob = _robot(which)
+    rid = ctx.add_robot(rob)
+    rng = np.random.default_rng(seed)
+    T = 24
+    tg = ctx.fk(rid, torch.as_tensor(inputs.joint_samples(rng, rob, T).T.copy(), dtype=torch.float32, device="cuda"))
+    tgt = torch.as_tensor(np.arange(BIG) * T // BIG, dtype=torch.int32, device="cuda")
+    cand = torch.as_tensor(np.arange(BIG) % 1000, dtype=torch.int32, device="cuda")
+    th = torch.as_tensor(inputs.joint_samples(rng, rob, BIG).T.copy(), dtype=torch.float32, device="cuda")
+    return rob, rid, tg, tgt, cand, th
+
+
+def _run(ctx, stage, rob, rid, tg, tgt, cand, th, params, sl):
+    """The stage on candidates sl: theta, score, errors, iterations (rows of the slice)."""
+    tgt, cand, th = tgt[sl].contiguous(), cand[sl].contiguous(), th[:, sl].clone(memory_format=torch.contiguous_format)
+    C = tgt.numel()
+    sc, pe, oe = (torch.empty(C, device="cuda") for _ in range(3))
+    it = torch.empty(C, dtype=torch.int32, device="cuda")
+    if stage == "ccd":
+        hjcd.hjcd_po_ccd(ctx.h, rid, tg.shape[0], tg, 1e-3, 1e-2, 77, params, C, tgt, cand, th, th, C, 0, params.cd_max_iters,
+                         sc, pe, oe, it)
+    else:
+        hjcd.hjcd_pjik(ctx.h, rid, tg.shape[0], tg, 1e-3, 1e-2, 77, params, C, tgt, cand, th, C, 0, params.lm_max_iters, sc, pe,
+                       oe, it)
+    torch.cuda.synchronize()
+    return [x.cpu().numpy() for x in (th, sc, pe, oe, it)]
+
+
+@pytest.mark.parametrize("stage", ["ccd", "lm"])
+@pytest.mark.parametrize("which", ["planar1", "planar2", "planar3", "random0", "chain7", "offsets", "random5", "chain24"])
+def test_small_batches_give_the_bits_of_large_ones(ctx, stage, which):
+    case = _case(ctx, which, 11)
+    for over in ({}, dict(lm_A=0, cd_max_iters=1, lm_max_iters=1), dict(lm_A=6, lm_lambda=1e-6, lm_trust_R=2.0)):
+        params = api.make_params(**over)
+        big = _run(ctx, stage, *case, params, slice(0, BIG))
+        for a, b in ((0, 1), (5, 20), (16, 32), (40, 57), (100, 101 + 2432), (0, 9728)):
+            small = _run(ctx, stage, *case, params, slice(a, b))
+            for x, y in zip(small, big):
+                np.testing.assert_array_equal(x.view(np.uint32), np.ascontiguousarray(y[..., a:b]).view(np.uint32))
+
+
+@pytest.mark.parametrize("which,seeds", [("random0", 997), ("chain7", 1000), ("chain12", 333), ("random5", 500)])
+def test_small_solves_give_the_rows_of_large_ones(ctx, which, seeds):
+    rob = _robot(which)
+    rid = ctx.add_robot(rob)
+    T = 10500 // seeds + 1
+    th = torch.as_tensor(inputs.joint_samples(np.random.default_rng(3), rob, T).T.copy(), dtype=torch.float32, device="cuda")
+    tg = ctx.fk(rid, th)
+    big = ctx.solve(rid, -1, tg, seeds, 16, 5, rob.n)
+    for t in (1, 3):
+        small = ctx.solve(rid, -1, tg[:t].contiguous(), seeds, 16, 5, rob.n)
+        for x, y in zip(small, big):
+            assert torch.equal(x.view(torch.int32), y[:t].view(torch.int32))
+
+
+def test_a_small_mixed_batch_gives_each_request_its_bits(ctx):
+    """Robots of different joint counts in one small batch (CTAs that straddle requests) against
+    each request in a batch of its own robot too large for the spread kernels."""
+    rng = np.random.default_rng(8)
+    items, big = [], []
+    for which in ("random0", "chain24", "chain7", "planar2"):
+        rob = _robot(which)
+        rid = ctx.add_robot(rob)
+        th = torch.as_tensor(inputs.joint_samples(rng, rob, 40).T.copy(), dtype=torch.float32, device="cuda")
+        tg = ctx.fk(rid, th)
+        items.append(ctx.batch_item(rid, -1, tg[:3].contiguous(), 301, 8, 21, rob.n))
+        big.append(ctx.solve(rid, -1, tg, 301, 8, 21, rob.n))
+    ctx.solve_batch([it for it, _ in items])
+    torch.cuda.synchronize()
+    for (_, got), ref in zip(items, big):
+        for x, y in zip(got, ref):
+            assert torch.equal(x.view(torch.int32), y[:3].view(torch.int32))
