@@ -211,9 +211,9 @@ void hjcd_graph_destroy(hjcd_graph* graph);
 /* ---- launch configuration and autotuning --------------------------------------- */
 
 /* Candidates per CTA of the PO-CCD kernel (64, 128 or 256; default 64) and
- * warps per CTA of the PJ-IK kernel (2, 4 or 8; default 8; a PJ-IK launch of
- * at most 64 candidates per SM always takes 2) for every later launch of the
- * context.  Results do not depend on them. */
+ * warps per CTA of the PJ-IK kernel (2, 4 or 8; default 8) for every later
+ * launch of the context; launches of at most 64 candidates per SM take kernels
+ * of their own, which have a fixed configuration.  Results do not depend on them. */
 hjcd_status hjcd_set_launch_config(hjcd_ctx* ctx, int32_t ccd_block, int32_t lm_warps);
 
 typedef struct hjcd_tune_report {
@@ -271,8 +271,10 @@ hjcd_status hjcd_solve_from_topk(hjcd_ctx* ctx, int32_t robot_id, int32_t scene_
  * paper has no serving layer).  One scheduler thread packs the pending
  * requests, in arrival order, into batches (one launch per phase, as
  * hjcd_solve_batch) and runs each batch on one of max_inflight streams as
- * soon as one is free: requests arriving while others run are admitted as
- * streams and memory free up, and their work overlaps on the device.  A
+ * soon as one is free (small batches at least a quarter of a millisecond after
+ * the last, unless max_batch_requests is 1): requests arriving while others
+ * run are admitted as streams and memory free up, and their work overlaps on
+ * the device.  A
  * batch holds at most max_batch_requests requests, max_batch_seeds PO-CCD
  * seeds and memory_budget / max_inflight bytes of device workspace; a request
  * that does not fit that share alone fails with HJCD_ENOMEM.  Zero fields take

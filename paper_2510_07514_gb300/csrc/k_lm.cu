@@ -236,6 +236,13 @@ __device__ __forceinline__ LmCta<WARPS> lm_cta(float* f) {
     return LmCta<WARPS>{reinterpret_cast<unsigned*>(b), b + WARPS, b + WARPS + WARPS * 32, b + WARPS + 2 * WARPS * 32};
 }
 
+// 1/2 |W r|^2 of a residual r = (e, om)
+__device__ __forceinline__ float weighted_cost(const float (&w)[6], const V3 e, const V3 om) {
+    const float e0 = w[0] * e.x, e1 = w[1] * e.y, e2 = w[2] * e.z;
+    const float e3 = w[3] * om.x, e4 = w[4] * om.y, e5 = w[5] * om.z;
+    return 0.5f * fmaf(e0, e0, fmaf(e1, e1, fmaf(e2, e2, fmaf(e3, e3, fmaf(e4, e4, e5 * e5)))));
+}
+
 // weighted cost 1/2 |W r|^2 at the trial point clamp(theta + alpha dir) of lane s
 // (the kinematics passes, the 6 x 6 solve and the trial spreading each exist
 // once in the kernel, called from every branch that needs them, which keeps
@@ -254,10 +261,8 @@ __device__ __noinline__ float trial_cost(const RobotParams* rob, const TargetDes
     }
     const Frame E = fk_flange(R, F);
     const V3 w = quat_log(quat_error(T, quat_from_frame(E)));
-    const float e0 = S.W(0, s) * (T.p[0] - E.p.x), e1 = S.W(1, s) * (T.p[1] - E.p.y);
-    const float e2 = S.W(2, s) * (T.p[2] - E.p.z), e3 = S.W(3, s) * w.x, e4 = S.W(4, s) * w.y;
-    const float e5 = S.W(5, s) * w.z;
-    return 0.5f * fmaf(e0, e0, fmaf(e1, e1, fmaf(e2, e2, fmaf(e3, e3, fmaf(e4, e4, e5 * e5)))));
+    const float w6[6] = {S.W(0, s), S.W(1, s), S.W(2, s), S.W(3, s), S.W(4, s), S.W(5, s)};
+    return weighted_cost(w6, v3(T.p[0] - E.p.x, T.p[1] - E.p.y, T.p[2] - E.p.z), w);
 }
 
 // theta <- clamp(theta + alpha dir) for lane s (the trial point the cost was taken at)
@@ -278,26 +283,58 @@ __device__ __forceinline__ void trial_item(int i, int A, const float* alphas, in
     *alpha = i < A ? alphas[i + 1] : 1.0f;
 }
 
-// Weighted cost of lane l's configuration with its single coordinate turned by x (the end
-// effector rotated by x about the joint's axis; see the mapping notes above).
-__device__ __noinline__ float coord_cost(const LmW S, int l, float x) {
+// Weighted cost of a configuration (position error e0, error quaternion q) with its single
+// coordinate (axis z, position Jacobian column v) turned by x: the end effector rotated by x about
+// the joint's axis (see the mapping notes above).
+__device__ __forceinline__ float coord_cost_at(const float (&w6)[6], const V3 z, const V3 v, const V3 e0, const Q4 q,
+                                               float x) {
     float sh, ch;
     sincos_red(0.5f * x, &sh, &ch);
-    const V3 z = v3(S.sc_z(0, l), S.sc_z(1, l), S.sc_z(2, l));
-    const V3 v = v3(S.sc_v(0, l), S.sc_v(1, l), S.sc_v(2, l));
     const V3 up = cross(v, z);  // component of p_ee - p_j normal to the axis
     const float a = 2.0f * sh * sh, b = 2.0f * sh * ch;  // 1 - cos x, sin x
-    const V3 e = fma3(a, up, fma3(-b, v, v3(S.e(0, l), S.e(1, l), S.e(2, l))));
-    const Q4 q{S.qe(0, l), v3(S.qe(1, l), S.qe(2, l), S.qe(3, l))};
+    const V3 e = fma3(a, up, fma3(-b, v, e0));
     Q4 q2{fmaf(q.w, ch, sh * dot(q.v, z)), fma3(ch, q.v, (-sh) * fma3(q.w, z, cross(q.v, z)))};
     if (q2.w < 0.0f) {
         q2.w = -q2.w;
         q2.v = (-1.0f) * q2.v;
     }
-    const V3 w = quat_log(q2);
-    const float e0 = S.W(0, l) * e.x, e1 = S.W(1, l) * e.y, e2 = S.W(2, l) * e.z;
-    const float e3 = S.W(3, l) * w.x, e4 = S.W(4, l) * w.y, e5 = S.W(5, l) * w.z;
-    return 0.5f * fmaf(e0, e0, fmaf(e1, e1, fmaf(e2, e2, fmaf(e3, e3, fmaf(e4, e4, e5 * e5)))));
+    return weighted_cost(w6, e, quat_log(q2));
+}
+__device__ __noinline__ float coord_cost(const LmW S, int l, float x) {
+    const float w6[6] = {S.W(0, l), S.W(1, l), S.W(2, l), S.W(3, l), S.W(4, l), S.W(5, l)};
+    return coord_cost_at(w6, v3(S.sc_z(0, l), S.sc_z(1, l), S.sc_z(2, l)), v3(S.sc_v(0, l), S.sc_v(1, l), S.sc_v(2, l)),
+                         v3(S.e(0, l), S.e(1, l), S.e(2, l)), Q4{S.qe(0, l), v3(S.qe(1, l), S.qe(2, l), S.qe(3, l))}, x);
+}
+
+// One joint's terms of |d_gn|^2 and, for the segment from d_gn to the Cauchy point ac g, of
+// |d_cp - d_gn|^2 and 2 d_gn.(d_cp - d_gn)
+__device__ __forceinline__ void dogleg_terms(float dgn, float g, float ac, float& ngn2, float& qa, float& qb) {
+    const float di = fmaf(ac, g, -dgn);
+    ngn2 = fmaf(dgn, dgn, ngn2);
+    qa = fmaf(di, di, qa);
+    qb = fmaf(2.0f * dgn, di, qb);
+}
+
+// The dogleg step wgn d_gn + wgd g inside the radius Rt (ngd2 = |d_cp|^2)
+__device__ __forceinline__ void dogleg_weights(float ngn2, float ngd2, float qa, float qb, float ac, float Rt, float& wgn,
+                                               float& wgd) {
+    const float R2 = Rt * Rt;
+    wgn = 1.0f;
+    wgd = 0.0f;
+    if (ngn2 <= R2) {
+        wgn = 1.0f;
+        wgd = 0.0f;
+    } else if (ngd2 >= R2) {
+        wgn = 0.0f;
+        wgd = ngd2 > 0.0f ? Rt * rsqrtf(ngd2) * ac : 0.0f;
+    } else {
+        // the point of the segment from the Gauss-Newton step to the Cauchy point on the boundary
+        const float qc = ngn2 - R2;
+        const float disc = fmaxf(fmaf(qb, qb, -4.0f * qa * qc), 0.0f);
+        const float tau = (2.0f * qc) / (sqrtf(disc) - qb);  // smaller root, stable form (qb < 0 here)
+        wgn = 1.0f - tau;
+        wgd = tau * ac;
+    }
 }
 
 // The dogleg step of Eq. dogleg and the single-coordinate step of Eq. single-coord for lane l,
@@ -347,7 +384,7 @@ __device__ __noinline__ void dogleg_prepare(const LmW S, int l, int n, float Rt,
         jgjg = fmaf(Jg[r], Jg[r], jgjg);
     }
     const float ac = jgjg > 0.0f ? __fdividef(gg, jgjg) : 0.0f;
-    const float ngd2 = ac * ac * gg, R2 = Rt * Rt;
+    const float ngd2 = ac * ac * gg;
     // |d_gn|^2 and, for the segment from d_gn to the Cauchy point, |d_cp - d_gn|^2 and 2 d_gn.(d_cp - d_gn)
     float ngn2 = 0.0f, qa = 0.0f, qb = 0.0f;
 #pragma unroll 1
@@ -359,26 +396,10 @@ __device__ __noinline__ void dogleg_prepare(const LmW S, int l, int n, float Rt,
             dgn = fmaf(col[r], y2[r], dgn);
             g = fmaf(col[r], b[r], g);
         }
-        const float di = fmaf(ac, g, -dgn);
-        ngn2 = fmaf(dgn, dgn, ngn2);
-        qa = fmaf(di, di, qa);
-        qb = fmaf(2.0f * dgn, di, qb);
+        dogleg_terms(dgn, g, ac, ngn2, qa, qb);
     }
-    float wgn = 1.0f, wgd = 0.0f;  // step = wgn * dgn + wgd * g
-    if (ngn2 <= R2) {
-        wgn = 1.0f;
-        wgd = 0.0f;
-    } else if (ngd2 >= R2) {
-        wgn = 0.0f;
-        wgd = ngd2 > 0.0f ? Rt * rsqrtf(ngd2) * ac : 0.0f;
-    } else {
-        // the point of the segment from the Gauss-Newton step to the Cauchy point on the boundary
-        const float qc = ngn2 - R2;
-        const float disc = fmaxf(fmaf(qb, qb, -4.0f * qa * qc), 0.0f);
-        const float tau = (2.0f * qc) / (sqrtf(disc) - qb);  // smaller root, stable form (qb < 0 here)
-        wgn = 1.0f - tau;
-        wgd = tau * ac;
-    }
+    float wgn, wgd;
+    dogleg_weights(ngn2, ngd2, qa, qb, ac, Rt, wgn, wgd);
     // the step, and the single coordinate: the joint with the largest |g_i| (the first of
     // equals), a 1-D Gauss-Newton step on it clamped to R
     int is = 0;
@@ -724,6 +745,447 @@ __global__ void __launch_bounds__(WARPS * 32, 16 / WARPS) k_lm(const LmArgs A) {
     }
 }
 
+// ----------------------------------------------------------------------------
+// PJ-IK with a candidate's work spread over a CTA, for batches too small to fill the GPU with one
+// lane per candidate: there the time is the latency of one candidate's chain of iterations.  A CTA
+// takes 16 candidates; a half warp (a unit) works on one part of all of them at a time -- a row of a
+// kinematics chain, a joint's column, an entry of a normal matrix, a trial -- and the units exchange
+// through shared memory.  Every trial of Alg. 4 is taken at once (the line search, the dogleg step,
+// the single coordinate), and so is the set-up of the dogleg step beside that of the LM step: with
+// 16 candidates some full step nearly always fails, and the units would idle otherwise.  The
+// perturbation's draws are made beside the factorisations.  Each quantity is formed by k_lm's
+// operations in their order (the sums over the joints and over the rows as well), so the results
+// are its bits.  Bound by latency: thirteen exchanges per iteration, the residuals (a lone warp's
+// chain of about 150 dependent instructions) and the 6 x 6 solve the longest stages.  One Panda
+// target of 1000 seeds: 74 us for at most 20 iterations, where k_lm takes 172 us.
+constexpr int kCoopCands = 16;    // candidates per CTA
+constexpr int kCoopLmWarps = 16;  // most warps per CTA
+constexpr int kCoopMaxA = 6;      // deepest line search taken here
+
+// Shared state [field][candidate], pointers at this thread's candidate; nl joints in the layout.
+struct LmC {
+    int nl;
+    float4* e4;  // [set][row]: that row of the last frame (its axes c0, c1, c2 and origin); set 0 the
+                 // configuration, 1 + i trial i
+    float2* c2;  // [set][joint]: cosine and sine of the joint's angle
+    float* f;
+    __device__ __forceinline__ float4& e(int set, int row) const { return e4[(set * 3 + row) * kCoopCands]; }
+    __device__ __forceinline__ float2& cs(int set, int j) const { return c2[(set * nl + j) * kCoopCands]; }
+    __device__ __forceinline__ float& at(int i) const { return f[i * kCoopCands]; }
+    __device__ __forceinline__ float& th(int j) const { return at(j); }
+    __device__ __forceinline__ float& st(int j) const { return at(nl + j); }       // LM step
+    __device__ __forceinline__ float& dgn(int j) const { return at(2 * nl + j); }  // Gauss-Newton step
+    __device__ __forceinline__ float& g(int j) const { return at(3 * nl + j); }    // gradient
+    __device__ __forceinline__ float& dd(int j) const { return at(4 * nl + j); }   // squared column norm
+    __device__ __forceinline__ float& jc(int r, int j) const { return at((5 + r) * nl + j); }   // J, then W J
+    __device__ __forceinline__ float& sc(int r, int j) const { return at((11 + r) * nl + j); }  // W J S
+    __device__ __forceinline__ float& fr(int r, int j) const { return at((17 + r) * nl + j); }  // joint origin, axis
+    __device__ __forceinline__ float& nz(int j) const { return at(23 * nl + j); }  // normal draws, nl + 1 rows
+    __device__ __forceinline__ float& s(int i) const { return at(24 * nl + 1 + i); }
+    __device__ __forceinline__ int& si(int i) const { return reinterpret_cast<int&>(s(i)); }
+};
+// scalars of LmC::s: M of the LM step and of the Gauss-Newton step, their solutions, W, W r, the
+// error, the error quaternion, the single coordinate's axis, column, joint and step, ...
+enum { kM = 0, kM0 = 21, kY = 42, kY2 = 48, kW = 54, kB = 60, kE = 66, kQ = 72, kSz = 76, kSv = 79, kSj = 82, kSstep = 83,
+       kCost = 84, kAc = 85, kNgd2 = 86, kWgn = 87, kWgd = 88, kStat = 89, kMask = 90, kLmCScalars = 91 };
+__host__ __device__ constexpr size_t coop_lm_bytes(int n, int A) {
+    return sizeof(float) * kCoopCands * ((size_t)12 * (A + 3) + (size_t)2 * (A + 3) * n + 24 * n + 1 + kLmCScalars);
+}
+
+// One row of a kinematics chain (fk_step's operations on that row) from the sines and cosines of
+// `set`; with FRAMES every joint's origin and axis go to C.fr
+template <int N, bool FRAMES>
+__device__ __forceinline__ void lmc_fk_row(const LmC& C, const RobotParams& R, int n_, int set, int row) {
+    const int n = N ? N : n_;
+    float c0 = row == 0 ? 1.0f : 0.0f, c1 = row == 1 ? 1.0f : 0.0f, c2 = row == 2 ? 1.0f : 0.0f, p = 0.0f;
+    auto step = [&](int j) {
+        const float4 g = R.dh[j];
+        const float2 cs = C.cs(set, j);
+        const float b1 = fmaf(g.x, c1, g.y * c2);
+        const float b2 = fmaf(g.x, c2, (-g.y) * c1);
+        p = fmaf(g.w, b2, fmaf(g.z, c0, p));
+        const float n0 = fmaf(cs.x, c0, cs.y * b1);
+        c1 = fmaf(cs.x, b1, (-cs.y) * c0);
+        c0 = n0;
+        c2 = b2;
+        if (FRAMES) {
+            C.fr(row, j) = p;
+            C.fr(3 + row, j) = c2;
+        }
+    };
+    if (N) {
+#pragma unroll
+        for (int j = 0; j < N; ++j) step(j);
+    } else {
+#pragma unroll 4
+        for (int j = 0; j < n; ++j) step(j);
+    }
+    C.e(set, row) = make_float4(c0, c1, c2, p);
+}
+// flange frame of a set
+__device__ __forceinline__ Frame lmc_flange(const LmC& C, const RobotParams& R, int set) {
+    const float4 a = C.e(set, 0), b = C.e(set, 1), c = C.e(set, 2);
+    return fk_flange(R, Frame{v3(a.x, b.x, c.x), v3(a.y, b.y, c.y), v3(a.z, b.z, c.z), v3(a.w, b.w, c.w)});
+}
+
+// row and column of entry q of a packed lower triangle
+__device__ __constant__ int8_t kTriRow[21] = {0, 1, 1, 2, 2, 2, 3, 3, 3, 3, 4, 4, 4, 4, 4, 5, 5, 5, 5, 5, 5};
+__device__ __constant__ int8_t kTriCol[21] = {0, 0, 1, 0, 1, 2, 0, 1, 2, 3, 0, 1, 2, 3, 4, 0, 1, 2, 3, 4, 5};
+
+// RED as for k_lm; N > 0: the launch's one robot has N joints (unrolled loops); N = 0: any robots
+template <bool RED, int N>
+__global__ void __launch_bounds__(kCoopLmWarps * 32, 1) k_lm_coop(const LmArgs A) {
+    extern __shared__ __align__(16) float smem_f[];
+    __shared__ float alphas[kCoopMaxA + 1];
+    if (threadIdx.x == 0) ls_alphas(alphas, A.P.lm_A, A.P.lm_beta);  // visible after the staging barrier
+    const RobotParams* rob = stage_robots(smem_f, A.rs);
+    const hjcd_params& P = A.P;
+    const float Rt = P.lm_trust_R;
+    const int lsA = P.lm_A, nt = lsA + 2;  // kinematics trials: the full step, the line search, the dogleg
+    const int nl = N ? N : A.rs.n_max;
+    const int W = (int)blockDim.x >> 5, U = 2 * W;
+    const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
+    const int l = lane & (kCoopCands - 1), half = lane >> 4, u = 2 * warp + half;
+    LmC C;
+    C.nl = nl;
+    C.e4 = reinterpret_cast<float4*>(reinterpret_cast<char*>(smem_f) + robots_smem_bytes(A.rs.n)) + l;
+    C.c2 = reinterpret_cast<float2*>(C.e4 - l + 3 * (nt + 1) * kCoopCands) + l;
+    C.f = reinterpret_cast<float*>(C.c2 - l + (nt + 1) * nl * kCoopCands) + l;
+    unsigned long long n_it = 0, n_fk = 0, n_sc = 0;
+    auto sincos_of = [&](const RobotParams& R, int j, float th) {
+        float sn, cn;
+        if (RED) sincos_red(th + R.off[j], &sn, &cn);
+        else __sincosf(th, &sn, &cn);
+        return make_float2(cn, sn);
+    };
+
+    for (int64_t base = kCoopCands * (int64_t)blockIdx.x; base < A.C; base += kCoopCands * (int64_t)gridDim.x) {
+        __syncthreads();  // the last group's state is no longer read
+        const int64_t c = base + l;
+        int32_t t = 0, s = 0;
+        bool have = c < A.C;
+        if (have) have = A.map.lookup(c, t, s);
+        const TargetDesc T = A.tg[have ? t : 0];
+        const RobotParams& R = N ? rob[0] : rob[have ? T.robot : 0];
+        const int n = N ? N : R.n;  // (a lane without a candidate runs along on a robot's joints, unread)
+        const int cap = A.n_iters >= 0 ? A.n_iters : T.lm_iters;
+        bool alive = have && T.eps_pos > 0.0f;
+        if (have && !alive && u == 0) {  // invalid target: no iterations, infinite score
+            if (A.score) A.score[c] = __int_as_float(0x7f800000);
+            if (A.perr) A.perr[c] = 0.0f;
+            if (A.oerr) A.oerr[c] = 0.0f;
+            if (A.iters) A.iters[c] = cap;
+        }
+        const bool mine = alive;
+        for (int j = u; j < n; j += U) {
+            const float th = mine ? A.th[j * A.ld + c] : 0.0f;
+            C.th(j) = th;
+            C.cs(0, j) = sincos_of(R, j, th);
+        }
+        if (u == 0) C.si(kStat) = 0;
+        __syncthreads();
+
+        for (int kk = 0;; ++kk) {
+            // kinematics with frames
+            if (u < 3) lmc_fk_row<N, true>(C, R, n, 0, u);
+            __syncthreads();
+
+            // the last warp: residual and break; the others: Jacobian columns z_i x (P_ee - P_i), z_i
+            {
+                const Frame E = lmc_flange(C, R, 0);
+                if (warp == W - 1) {
+                    const Q4 qerr = quat_error(T, quat_from_frame(E));
+                    const V3 om = quat_log(qerr);
+                    const V3 epv = v3(T.p[0], T.p[1], T.p[2]) - E.p;
+                    const float ep = sqrt_approx(dot(epv, epv)), eo = sqrt_approx(dot(om, om));
+                    if (alive && half == 0) {
+                        ++n_fk;
+                        if ((kk > 0 && ep < T.eps_pos && eo < T.eps_ori) || kk == cap) {
+                            if (A.score) {
+                                const float a = ep / T.eps_pos, bb = eo / T.eps_ori;
+                                A.score[c] = fmaf(a, a, bb * bb);
+                            }
+                            if (A.perr) A.perr[c] = ep;
+                            if (A.oerr) A.oerr[c] = eo;
+                            if (A.iters) A.iters[c] = kk;
+                            C.si(kStat) = 1;
+                        }
+                        C.s(kE) = epv.x;
+                        C.s(kE + 1) = epv.y;
+                        C.s(kE + 2) = epv.z;
+                        C.s(kE + 3) = om.x;
+                        C.s(kE + 4) = om.y;
+                        C.s(kE + 5) = om.z;
+                        C.s(kQ) = qerr.w;
+                        C.s(kQ + 1) = qerr.v.x;
+                        C.s(kQ + 2) = qerr.v.y;
+                        C.s(kQ + 3) = qerr.v.z;
+                    }
+                } else {
+                    for (int j = u; j < n; j += U - 2) {
+                        const V3 Zi = v3(C.fr(3, j), C.fr(4, j), C.fr(5, j));
+                        const V3 jp = cross(Zi, E.p - v3(C.fr(0, j), C.fr(1, j), C.fr(2, j)));
+                        C.jc(0, j) = jp.x;
+                        C.jc(1, j) = jp.y;
+                        C.jc(2, j) = jp.z;
+                        C.jc(3, j) = Zi.x;
+                        C.jc(4, j) = Zi.y;
+                        C.jc(5, j) = Zi.z;
+                    }
+                }
+            }
+            __syncthreads();
+            alive = alive && C.si(kStat) == 0;
+
+            // row norms, W and W r
+            if (u < 6) {
+                float rn = 0.0f;
+#pragma unroll 4
+                for (int j = 0; j < n; ++j) {
+                    const float v = C.jc(u, j);
+                    rn = fmaf(v, v, rn);
+                }
+                const float wo = __fdividef(T.eps_pos, T.eps_ori);
+                const float w = (u < 3 ? 1.0f : wo) * rsqrtf(fmaxf(rn, 1e-12f));  // c / max(|row|, 1e-6)
+                C.s(kW + u) = w;
+                C.s(kB + u) = w * C.s(kE + u);
+            }
+            if (!__syncthreads_or(alive)) break;
+
+            // weighted columns and those scaled to unit length; the last warp: the cost
+            if (warp == W - 1) {
+                float cost0 = 0.0f;
+#pragma unroll
+                for (int r = 0; r < 6; ++r) cost0 = fmaf(C.s(kB + r), C.s(kB + r), cost0);
+                if (half == 0) {
+                    C.s(kCost) = 0.5f * cost0;
+                    C.si(kMask) = 0;
+                }
+            } else {
+                for (int j = u; j < n; j += U - 2) {
+                    float col[6], dd = 1e-9f;
+#pragma unroll
+                    for (int r = 0; r < 6; ++r) {
+                        col[r] = C.jc(r, j) * C.s(kW + r);
+                        dd = fmaf(col[r], col[r], dd);
+                        C.jc(r, j) = col[r];
+                    }
+                    const float rs = rsqrtf(dd);
+                    C.dd(j) = dd;
+#pragma unroll
+                    for (int r = 0; r < 6; ++r) C.sc(r, j) = col[r] * rs;
+                }
+            }
+            __syncthreads();
+
+            // the normal matrices: entry q of the scaled columns' (LM), of the columns' (Gauss-Newton)
+            for (int q = u; q < 42; q += U) {
+                const int k = q < 21 ? q : q - 21;
+                const float* a = q < 21 ? &C.sc(kTriRow[k], 0) : &C.jc(kTriRow[k], 0);
+                const float* b = q < 21 ? &C.sc(kTriCol[k], 0) : &C.jc(kTriCol[k], 0);
+                float m = 0.0f;
+#pragma unroll 4
+                for (int j = 0; j < n; ++j) m = fmaf(a[j * kCoopCands], b[j * kCoopCands], m);
+                C.s(kM + q) = m;
+            }
+            __syncthreads();
+
+            // factorisations and solutions, the LM system in the lower half of warp 0 and the
+            // Gauss-Newton system in the upper one; the other warps draw the perturbation
+            if (warp == 0) {
+                const int m0 = half ? kM0 : kM;
+                const float reg = half ? P.lm_gn_reg : P.lm_lambda;
+                float M[21], inv[6], b[6], y[6];
+#pragma unroll
+                for (int q = 0; q < 21; ++q) M[q] = C.s(m0 + q);
+#pragma unroll
+                for (int r = 0; r < 6; ++r) {
+                    b[r] = C.s(kB + r);
+                    M[tri(r, r)] += reg;
+                }
+                chol6(M, inv);
+                chol6_solve(M, inv, b, y);
+#pragma unroll
+                for (int r = 0; r < 6; ++r) C.s((half ? kY2 : kY) + r) = y[r];
+            } else if (warp == 1) {
+                // J g = M0 W r, the Cauchy point
+                float Jg[6], gg = 0.0f, jgjg = 0.0f;
+#pragma unroll
+                for (int r = 0; r < 6; ++r) {
+                    float a = 0.0f;
+#pragma unroll
+                    for (int q = 0; q < 6; ++q) a = fmaf(C.s(kM0 + (r >= q ? tri(r, q) : tri(q, r))), C.s(kB + q), a);
+                    Jg[r] = a;
+                }
+#pragma unroll
+                for (int r = 0; r < 6; ++r) {
+                    gg = fmaf(C.s(kB + r), Jg[r], gg);
+                    jgjg = fmaf(Jg[r], Jg[r], jgjg);
+                }
+                const float ac = jgjg > 0.0f ? __fdividef(gg, jgjg) : 0.0f;
+                C.s(kAc) = ac;
+                C.s(kNgd2) = ac * ac * gg;
+            } else if (alive) {
+                for (int q = u - 4; 2 * q < n; q += U - 4) {
+                    const float2 z = normal_pair(T, (uint32_t)s, kPhaseLm, (uint32_t)A.k0 + (uint32_t)kk, q);
+                    C.nz(2 * q) = z.x;
+                    C.nz(2 * q + 1) = z.y;
+                }
+            }
+            __syncthreads();
+
+            // each joint's LM step, Gauss-Newton step and gradient
+            for (int j = u; j < n; j += U) {
+                float a = 0.0f, dgn = 0.0f, g = 0.0f;
+#pragma unroll
+                for (int r = 0; r < 6; ++r) {
+                    const float v = C.jc(r, j);
+                    a = fmaf(v, C.s(kY + r), a);
+                    dgn = fmaf(v, C.s(kY2 + r), dgn);
+                    g = fmaf(v, C.s(kB + r), g);
+                }
+                C.st(j) = clampf(__fdividef(a, C.dd(j)), -Rt, Rt);  // trust region
+                C.dgn(j) = dgn;
+                C.g(j) = g;
+            }
+            __syncthreads();
+
+            // the dogleg's weights; the single coordinate
+            if (warp == 0) {
+                const float ac = C.s(kAc);
+                float ngn2 = 0.0f, qa = 0.0f, qb = 0.0f;
+#pragma unroll 4
+                for (int j = 0; j < n; ++j) dogleg_terms(C.dgn(j), C.g(j), ac, ngn2, qa, qb);
+                float wgn, wgd;
+                dogleg_weights(ngn2, C.s(kNgd2), qa, qb, ac, Rt, wgn, wgd);
+                C.s(kWgn) = wgn;
+                C.s(kWgd) = wgd;
+            } else if (warp == 1) {
+                int is = 0;
+                float gbest = -1.0f;
+#pragma unroll 4
+                for (int j = 0; j < n; ++j) {
+                    const float g = fabsf(C.g(j));
+                    if (g > gbest) {
+                        gbest = g;
+                        is = j;
+                    }
+                }
+                float cn = 0.0f, col[6];
+#pragma unroll
+                for (int r = 0; r < 6; ++r) {
+                    col[r] = C.jc(r, is);
+                    cn = fmaf(col[r], col[r], cn);
+                }
+                C.si(kSj) = is;
+                C.s(kSstep) = cn > 0.0f ? clampf(__fdividef(C.g(is), cn), -Rt, Rt) : 0.0f;
+#pragma unroll
+                for (int r = 0; r < 3; ++r) {
+                    C.s(kSv + r) = __fdividef(col[r], C.s(kW + r));
+                    C.s(kSz + r) = __fdividef(col[3 + r], C.s(kW + 3 + r));
+                }
+            }
+            __syncthreads();
+
+            // sines and cosines of the trials' angles
+            for (int w = u; w < nt * n; w += U) {
+                const int i = N ? w / (N ? N : 1) : w / n, j = w - i * n;
+                const float dir = i <= lsA ? C.st(j) : fmaf(C.s(kWgn), C.dgn(j), C.s(kWgd) * C.g(j));
+                const float al = i <= lsA ? alphas[i] : 1.0f;
+                C.cs(1 + i, j) = sincos_of(R, j, clampf(fmaf(al, dir, C.th(j)), R.lim[j].x, R.lim[j].y));
+            }
+            __syncthreads();
+
+            // the trials' kinematics rows
+            for (int w = u; w < 3 * nt; w += U) lmc_fk_row<N, false>(C, R, n, 1 + w / 3, w % 3);
+            __syncthreads();
+
+            // the trials' costs (first the warps with kinematics trials, then those with the single
+            // coordinate's); bit i of the mask: trial i lowered the cost, in the order of Alg. 4
+            {
+                const int kw = (nt + 1) / 2, items = kw + (lsA + 2) / 2;  // warps' worth of either
+                for (int w = warp; w < items; w += W) {
+                    const bool kin = w < kw;
+                    const int i = 2 * (kin ? w : w - kw) + half;
+                    if (i >= (kin ? nt : lsA + 1)) continue;
+                    const float w6[6] = {C.s(kW), C.s(kW + 1), C.s(kW + 2), C.s(kW + 3), C.s(kW + 4), C.s(kW + 5)};
+                    float cost;
+                    if (kin) {
+                        const Frame E = lmc_flange(C, R, 1 + i);
+                        const V3 om = quat_log(quat_error(T, quat_from_frame(E)));
+                        cost = weighted_cost(w6, v3(T.p[0], T.p[1], T.p[2]) - E.p, om);
+                    } else {
+                        const int j = C.si(kSj);
+                        const float th0 = C.th(j);
+                        const float thj = clampf(fmaf(alphas[i], C.s(kSstep), th0), R.lim[j].x, R.lim[j].y);
+                        cost = coord_cost_at(w6, v3(C.s(kSz), C.s(kSz + 1), C.s(kSz + 2)),
+                                             v3(C.s(kSv), C.s(kSv + 1), C.s(kSv + 2)), v3(C.s(kE), C.s(kE + 1), C.s(kE + 2)),
+                                             Q4{C.s(kQ), v3(C.s(kQ + 1), C.s(kQ + 2), C.s(kQ + 3))}, thj - th0);
+                    }
+                    if (cost < C.s(kCost)) atomicOr(&C.si(kMask), 1 << (kin ? i : nt + i));
+                }
+            }
+            __syncthreads();
+
+            // the first success in the order of Alg. 4, else the perturbation
+            if (alive) {
+                const int pick = __ffs(C.si(kMask)) - 1;
+                for (int j = u; j < n; j += U) {
+                    const float lo = R.lim[j].x, hi = R.lim[j].y;
+                    float th = C.th(j);
+                    if (pick < 0) {
+                        th = clampf(fmaf(P.lm_sigma, C.nz(j), th), lo, hi);
+                    } else if (pick < nt) {
+                        const float dir = pick <= lsA ? C.st(j) : fmaf(C.s(kWgn), C.dgn(j), C.s(kWgd) * C.g(j));
+                        th = clampf(fmaf(pick <= lsA ? alphas[pick] : 1.0f, dir, th), lo, hi);
+                    } else if (j == C.si(kSj)) {
+                        th = clampf(fmaf(alphas[pick - nt], C.s(kSstep), th), lo, hi);
+                    }
+                    C.th(j) = th;
+                    C.cs(0, j) = sincos_of(R, j, th);
+                }
+                if (u == 0) {  // the passes and trials the sequential method evaluates
+                    ++n_it;
+                    n_fk += pick >= 0 && pick < nt ? pick + 1 : nt;
+                    if (pick < 0 || pick >= nt) n_sc += pick < 0 ? lsA + 1 : pick - nt + 1;
+                }
+            }
+            __syncthreads();
+        }
+        if (mine)
+            for (int j = u; j < n; j += U) A.th[j * A.ld + c] = C.th(j);
+    }
+    if (A.cnt) {
+        n_it = warp_sum(n_it);
+        n_fk = warp_sum(n_fk);
+        n_sc = warp_sum(n_sc);
+        if (lane == 0 && (warp == 0 || warp == W - 1)) {
+            atomicAdd(&A.cnt->v[1], n_it);
+            atomicAdd(&A.cnt->v[2], n_fk);
+            atomicAdd(&A.cnt->v[7], n_sc);
+        }
+    }
+}
+
+template <bool RED, int N>
+void launch_lm_coop_n(const LmArgs& A, int warps, cudaStream_t st) {
+    const size_t smem = robots_smem_bytes(A.rs.n) + coop_lm_bytes(A.rs.n_max, A.P.lm_A);
+    static SmemLimit lim;
+    allow_dyn_smem(k_lm_coop<RED, N>, lim, robots_smem_bytes(kMaxLaunchRobots) + coop_lm_bytes(N ? N : kMaxDof, kCoopMaxA));
+    int per_sm = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lm_coop<RED, N>, 32 * warps, smem);
+    const int g = (int)std::min<int64_t>((A.C + kCoopCands - 1) / kCoopCands, (int64_t)sm_count() * std::max(per_sm, 1));
+    k_lm_coop<RED, N><<<g, 32 * warps, smem, st>>>(A);
+}
+
+template <bool RED>
+void launch_lm_coop(const LmArgs& A, int warps, cudaStream_t st) {
+    const int n = A.rs.n == 1 ? A.rs.n_max : 0;
+    if (n == 6) launch_lm_coop_n<RED, 6>(A, warps, st);
+    else if (n == 7) launch_lm_coop_n<RED, 7>(A, warps, st);
+    else launch_lm_coop_n<RED, 0>(A, warps, st);
+}
+
 template <bool TRACE, int WARPS, bool RED>
 void launch_lm_t(const LmArgs& A, cudaStream_t st) {
     const size_t smem = robots_smem_bytes(A.rs.n) +
@@ -762,6 +1224,18 @@ void launch_lm_w(const LmArgs& A, cudaStream_t st) {
 
 void launch_lm(const LmArgs& A, bool trace, cudaStream_t st) {
     if (A.C <= 0) return;
+    // Up to 64 candidates per SM (two resident CTAs of 16 on every SM, twice) the spread kernel's
+    // shorter iterations win; past that its extra work does.  Phase time of the polish, spread /
+    // one lane per candidate, us (7, 20, 24 joints): 1000 candidates 74 / 172, 123 / 328, 137 / 360;
+    // 4000: 86 / 200, 168 / 346, 182 / 356; 8000: 166 / 221, 322 / 346, 338 / 356; 16000: 311 / 240,
+    // 594 / 395, 616 / 363.  Twelve warps while a CTA has its SM to itself (8: 76, 139, 150), eight
+    // (two CTAs per SM) beyond.
+    if (!trace && A.P.lm_A <= kCoopMaxA && A.C <= (int64_t)sm_count() * 4 * kCoopCands) {
+        const int warps = A.C <= (int64_t)sm_count() * kCoopCands ? 12 : 8;
+        if (A.in_limits && A.rs.plain) launch_lm_coop<false>(A, warps, st);
+        else launch_lm_coop<true>(A, warps, st);
+        return;
+    }
     if (trace) launch_lm_w<true, true>(A, st);
     else if (A.in_limits && A.rs.plain) launch_lm_w<false, false>(A, st);
     else launch_lm_w<false, true>(A, st);
