@@ -513,41 +513,131 @@ inline int grid_for(int64_t items, int per_block, int per_sm = 64) {
 }
 
 // ----------------------------------------------------------------------------
-// per-target selection: 64-bit keys (score bits << 32 | index) sorted in
-// shared memory by a bitonic network; non-negative scores order like their
-// IEEE bit patterns, the index in the low word breaks ties toward the lower
-// candidate, and invalid entries get the all-ones key and sort last.
+// per-target selection.  A candidate's key is 32 bits (a non-negative score orders like its IEEE
+// bit pattern; ties go to the lower candidate) and the order of the first `want` of a target's M
+// keys is found by one bucket pass in shared memory: the keys' range is cut into up to kMaxBins
+// equal bins, the candidates are gathered by bin, and a candidate's rank is its bin's start plus
+// its rank among the few that share the bin.  The work is linear while the bins are short (a
+// whole sort of 1024 keys took 55 barriers, this takes eight); keys that crowd one bin cost
+// their square, which only equal scores reach.
 
-constexpr uint64_t kNoKey = ~0ull;
+constexpr uint32_t kNoKey32 = 0xffffffffu;  // never ranked
+constexpr int kMaxBins = 2048;
 
-__device__ __forceinline__ uint64_t score_key(float s, uint32_t idx) {
-    if (!(s == s)) return kNoKey;  // NaN
-    const uint32_t bits = __float_as_uint(s + 0.0f);  // -0 -> +0
-    return ((uint64_t)bits << 32) | idx;
+__device__ __forceinline__ uint32_t score_bits(float s) {
+    return __float_as_uint(s + 0.0f);  // -0 -> +0
 }
 
-__device__ __forceinline__ void bitonic_sort(uint64_t* keys, int N) {
-    for (int size = 2; size <= N; size <<= 1) {
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int i = threadIdx.x; i < (N >> 1); i += blockDim.x) {
-                const int lo = 2 * i - (i & (stride - 1));
-                const int hi = lo + stride;
-                const bool up = (lo & size) == 0;
-                const uint64_t a = keys[lo], b = keys[hi];
-                if ((a > b) == up) {
-                    keys[lo] = b;
-                    keys[hi] = a;
-                }
-            }
-            __syncthreads();
+// bins of a pass over M keys
+__host__ __device__ __forceinline__ int bucket_bins(int M) {
+    int bins = 32;
+    while (bins < M && bins < kMaxBins) bins <<= 1;
+    return bins;
+}
+// Shared memory of the bucket pass for up to M keys.
+__host__ __device__ __forceinline__ size_t bucket_smem_bytes(int M) {
+    const size_t m = M > 0 ? M : 1;
+    return sizeof(uint32_t) * (m + bucket_bins((int)m) + 36) + sizeof(uint16_t) * 2 * ((m + 1) / 2 * 2);
+}
+struct Bucket {
+    int bins;
+    uint32_t* key;    // [M]: written by the caller
+    uint32_t* bin;    // [bins]
+    uint32_t* tmp;    // [36]
+    uint16_t* slot;   // [M]
+    uint16_t* order;  // [M]: the candidates of the first `want` ranks
+};
+__device__ __forceinline__ Bucket bucket_of(void* smem, int M) {
+    Bucket B;
+    B.bins = bucket_bins(M);
+    B.key = reinterpret_cast<uint32_t*>(smem);
+    B.bin = B.key + M;
+    B.tmp = B.bin + B.bins;
+    B.slot = reinterpret_cast<uint16_t*>(B.tmp + 36);
+    B.order = B.slot + (M + 1) / 2 * 2;
+    return B;
+}
+
+// B.order[r] for r < min(want, returned) from B.key[0, M) (visible to the whole CTA when it is
+// called); returns the number of keys other than kNoKey32.  All threads of the CTA take part
+// (a multiple of 32, at most 1024); ends with a barrier.
+__device__ __forceinline__ int bucket_order(const Bucket& B, int M, int want) {
+    const int tid = threadIdx.x, nth = blockDim.x, lane = tid & 31, warp = tid >> 5;
+    const int bins = B.bins;
+    // range and number of the keys
+    uint32_t lo = kNoKey32, hi = 0;
+    int cnt = 0;
+    for (int i = tid; i < M; i += nth) {
+        const uint32_t k = B.key[i];
+        if (k != kNoKey32) {
+            lo = min(lo, k);
+            hi = max(hi, k);
+            ++cnt;
         }
     }
-}
-
-__device__ __forceinline__ int pow2_at_least(int m) {
-    int N = 1;
-    while (N < m) N <<= 1;
-    return N;
+    for (int i = tid; i < bins; i += nth) B.bin[i] = 0;
+    if (tid < 3) B.tmp[32 + tid] = tid == 0 ? kNoKey32 : 0u;
+    __syncthreads();
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    if (lane == 0 && cnt) {
+        atomicMin(&B.tmp[32], lo);
+        atomicMax(&B.tmp[33], hi);
+        atomicAdd(&B.tmp[34], (uint32_t)cnt);
+    }
+    __syncthreads();
+    lo = B.tmp[32];
+    hi = B.tmp[33];
+    const int valid = (int)B.tmp[34];
+    const int span = valid ? 32 - __clz(hi - lo) : 0;  // bits of the range
+    const int shift = max(0, span - (31 - __clz(bins)));
+    // bin sizes, their starts (an exclusive scan: a run of bins per thread)
+    for (int i = tid; i < M; i += nth) {
+        const uint32_t k = B.key[i];
+        if (k != kNoKey32) atomicAdd(&B.bin[(k - lo) >> shift], 1u);
+    }
+    __syncthreads();
+    const int per = (bins + nth - 1) / nth, b0 = min(bins, tid * per), b1 = min(bins, b0 + per);
+    uint32_t sum = 0;
+    for (int i = b0; i < b1; ++i) sum += B.bin[i];
+    uint32_t inc = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += v;
+    }
+    if (lane == 31) B.tmp[warp] = inc;
+    __syncthreads();
+    uint32_t at = inc - sum;
+    for (int w = 0; w < warp; ++w) at += B.tmp[w];
+    for (int i = b0; i < b1; ++i) {
+        const uint32_t v = B.bin[i];
+        B.bin[i] = at;
+        at += v;
+    }
+    __syncthreads();
+    // the candidates by bin; a bin's entry then holds its end, which is the next one's start
+    for (int i = tid; i < M; i += nth) {
+        const uint32_t k = B.key[i];
+        if (k != kNoKey32) B.slot[atomicAdd(&B.bin[(k - lo) >> shift], 1u)] = (uint16_t)i;
+    }
+    __syncthreads();
+    for (int p = tid; p < valid; p += nth) {
+        const int i = B.slot[p];
+        const uint32_t k = B.key[i], b = (k - lo) >> shift;
+        const int s0 = b ? (int)B.bin[b - 1] : 0, s1 = (int)B.bin[b];
+        if (s0 >= want) continue;
+        int r = s0;
+        for (int q = s0; q < s1; ++q) {
+            const int j = B.slot[q];
+            const uint32_t kj = B.key[j];
+            r += kj < k || (kj == k && j < i);
+        }
+        if (r < want) B.order[r] = (uint16_t)i;
+    }
+    __syncthreads();
+    return valid;
 }
 
 // ----------------------------------------------------------------------------
@@ -655,12 +745,12 @@ struct RankArgs {
 // class 1 (the top key bit), each class ordered by score and then index.  With
 // the target's nearest flag (with tg null: whenever q_ref is set), class 0 is
 // ordered by squared joint distance to the reference q_ref[t] instead
-// (reading c24).  kNoKey past B.
-__device__ __forceinline__ uint64_t rank_key(const RankArgs& A, int t, int64_t b0, int B, int n, int i, bool use_hit) {
-    if (i >= B || (use_hit && A.hit && A.hit[b0 + i])) return kNoKey;
+// (reading c24).  kNoKey32: not ranked.
+__device__ __forceinline__ uint32_t rank_key(const RankArgs& A, int t, int64_t b0, int n, int i, bool use_hit) {
+    if (use_hit && A.hit && A.hit[b0 + i]) return kNoKey32;
     const int64_t g = b0 + i;
     const float sc = A.score[g];
-    if (!(sc < __int_as_float(0x7f800000))) return kNoKey;  // finite only
+    if (!(sc < __int_as_float(0x7f800000))) return kNoKey32;  // finite only
     const float ep = A.tg ? A.tg[t].eps_pos : A.eps_pos, eo = A.tg ? A.tg[t].eps_ori : A.eps_ori;
     const bool conv = A.perr[g] <= ep && A.oerr[g] <= eo;
     const bool nearest = A.q_ref && (!A.tg || (A.tg[t].top_k & kNearestFlag));
@@ -670,10 +760,10 @@ __device__ __forceinline__ uint64_t rank_key(const RankArgs& A, int t, int64_t b
             const float dj = A.th[j * A.ld + g] - A.q_ref[(int64_t)t * A.ld_ref + j];
             d2 = fmaf(dj, dj, d2);
         }
-        return score_key(d2, (uint32_t)i);
+        return d2 == d2 ? score_bits(d2) : kNoKey32;
     }
-    const uint64_t k = score_key(sc, (uint32_t)i);
-    return conv ? k : (k | (1ull << 63));
+    const uint32_t k = score_bits(sc);
+    return conv ? k : (k | 0x80000000u);
 }
 
 // Collision filter of C candidates.  With tg null or uniform set every

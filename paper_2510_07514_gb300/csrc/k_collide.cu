@@ -481,7 +481,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_collide(const CollideAr
 
 // Ranking with the collision filter applied lazily (the top_k collision-free
 // candidates by score are the first top_k collision-free ones in score
-// order): one CTA per target sorts its candidates' keys, then its warps check
+// order): one CTA per target orders its candidates' keys, then its warps check
 // candidates in rank order, one candidate per warp and kWarpsPerBlock at a
 // time, until top_k collision-free ones are found or the ranked candidates
 // run out.  Same output as the collision filter over all candidates followed
@@ -506,20 +506,17 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_rank_lazy(const Collide
     if (!collide_prologue<UNIFORM>(A, smem, L, sc0, n_obj4, &rob)) return;
     const WarpBufs Bf = warp_bufs(smem, L, A);
     const float4* s_scene = reinterpret_cast<const float4*>(smem);
-    uint64_t* keys = reinterpret_cast<uint64_t*>(smem + keys_off);
 
     const TargetDesc& T = R.tg[t];
     const int rid = T.robot, sid = UNIFORM ? 0 : T.scene;
     const int n = rob[rid].n;
     const int64_t b0 = R.b_off[t];
     const int B = (int)(R.b_off[t + 1] - b0);
-    const int N = pow2_at_least(B > 0 ? B : 1);
-    for (int i = threadIdx.x; i < N; i += blockDim.x) keys[i] = rank_key(R, t, b0, B, n, i, false);
+    const Bucket S = bucket_of(smem + keys_off, B > 0 ? B : 1);
+    for (int i = threadIdx.x; i < B; i += blockDim.x) S.key[i] = rank_key(R, t, b0, n, i, false);
     __syncthreads();
-    bitonic_sort(keys, N);
-    int ranked = 0;  // candidates with a key (finite score)
-    for (int base = 0; base < N; base += blockDim.x)
-        ranked += __syncthreads_count(base + (int)threadIdx.x < N && keys[base + threadIdx.x] != kNoKey);
+    // candidates with a key (finite score); the ranks that may be visited below
+    const int ranked = bucket_order(S, B, R.list ? depth + kWarpsPerBlock : B);
     const int top_k = T.top_k & ~kNearestFlag;
 
     WarpRobot<SPL> W;
@@ -534,7 +531,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_rank_lazy(const Collide
         const int p = p0 + warp;
         bool hit = true;
         if (p < ranked) {
-            const int64_t c = b0 + (int64_t)(keys[p] & 0xffffffffu);
+            const int64_t c = b0 + S.order[p];
             unsigned long long t_s = 0, t_b = 0;
             hit = warp_collides<SPL, UNIFORM, GRID>(A, rob, sc0, s_scene, W, Bf, c, rid, sid, t_s, t_b);
             if (lane == 0) {
@@ -563,13 +560,13 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_rank_lazy(const Collide
         // deeper than the bound: the verdicts taken so far are kept (0 free, 1 colliding), the
         // unchecked ranked candidates marked 2 for the collision filter over the listed targets,
         // which spreads them over every SM; the ranking of the listed targets follows it
-        for (int q = threadIdx.x; q < ranked; q += blockDim.x) {
-            uint8_t v = 2;
-            if (q < p0) {
-                v = 1;
-                for (int r = 0; r < count; ++r) v = picks[r] == q ? 0 : v;
-            }
-            A.hit[b0 + (int64_t)(keys[q] & 0xffffffffu)] = v;
+        for (int i = threadIdx.x; i < B; i += blockDim.x)
+            if (S.key[i] != kNoKey32) A.hit[b0 + i] = 2;
+        __syncthreads();
+        for (int q = threadIdx.x; q < p0; q += blockDim.x) {
+            uint8_t v = 1;
+            for (int r = 0; r < count; ++r) v = picks[r] == q ? 0 : v;
+            A.hit[b0 + S.order[q]] = v;
         }
         if (threadIdx.x == 0) R.list[atomicAdd(R.n_list, 1)] = t;
         return;
@@ -578,7 +575,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_rank_lazy(const Collide
     float* oe = R.out_err + R.qe_off[2 * t + 1];
     for (int q = threadIdx.x; q < count * (n + 2); q += blockDim.x) {
         const int r = q / (n + 2), j = q % (n + 2);
-        const int64_t g = b0 + (int64_t)(keys[picks[r]] & 0xffffffffu);
+        const int64_t g = b0 + S.order[picks[r]];
         if (j < n) oq[r * n + j] = R.th[j * R.ld + g];
         else if (j == n) oe[r * 2] = R.perr[g];
         else oe[r * 2 + 1] = R.oerr[g];
@@ -591,9 +588,7 @@ bool launch_rank_lazy_t(const CollideArgs& A, const RankArgs& R, int n_obj4, int
     const CollideLayout L =
         collide_smem_layout(UNIFORM ? n_obj4 : 0, A.rs.n, A.rs.n_max + 2, A.rs.ns_max, A.rs.pairs_max);
     const uint32_t keys_off = (L.total + 15u) / 16u * 16u;
-    int N = 1;
-    while (N < max_b) N <<= 1;
-    const size_t smem = keys_off + 8 * (size_t)N;
+    const size_t smem = keys_off + bucket_smem_bytes(max_b);
     if (smem > 220 * 1024) return false;
     static SmemLimit lim;
     allow_dyn_smem(k_rank_lazy<SPL, UNIFORM, GRID>, lim, 220 * 1024);

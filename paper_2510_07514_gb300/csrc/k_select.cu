@@ -2,11 +2,11 @@
 // (Alg. 2), ranking of the collision-free candidates (Alg. 2, final
 // step), and packing of target poses.
 //
-// One CTA per target sorts 64-bit keys (score bits << 32 | index) in shared
-// memory with a bitonic network; scores are non-negative, so their IEEE bit
-// patterns order like the values, and the index in the low word breaks ties
-// toward the lower candidate.  Invalid entries (padding, collisions, NaN)
-// get the all-ones key and sort last.
+// A target's candidates are ordered by one bucket pass over 32-bit keys in
+// shared memory (bucket_order); ties go to the lower candidate and invalid
+// entries (collisions, NaN) are not ranked.
+#include <algorithm>
+
 #include "hjcd_internal.cuh"
 
 namespace hjcd {
@@ -15,43 +15,47 @@ namespace {
 
 constexpr int kSelThreads = 512;
 
+// Blocks (target, slice): each slice's CTA orders the target's seeds for itself and writes its share
+// of the duplicates, one (duplicate, pair of joints) per thread at a time, so that a lone target's
+// Philox draws spread over many SMs.  Bound by latency for few targets, by the draws for many.
+// Time with one CTA sorting all keys and writing all duplicates -> this: one target of 1000 seeds
+// 20 -> 8.8 us, of 2000 seeds and 24 joints 60 -> 11 us, 1000 targets of 1000 seeds 75 -> 51 us.
 __global__ void __launch_bounds__(kSelThreads) k_topk_dup(const DupArgs A) {
-    extern __shared__ uint64_t keys[];
+    extern __shared__ __align__(16) unsigned char sel_smem[];
     const int t = blockIdx.x;
     const int64_t m0 = A.m_off[t];
     const int M = (int)(A.m_off[t + 1] - m0);
     if (M <= 0) return;
-    const int N = pow2_at_least(M);
-    for (int i = threadIdx.x; i < N; i += blockDim.x)
-        keys[i] = i < M ? score_key(A.score_M[m0 + i], (uint32_t)i) : kNoKey;
+    const Bucket S = bucket_of(sel_smem, M);
+    for (int i = threadIdx.x; i < M; i += blockDim.x) {
+        const float sc = A.score_M[m0 + i];
+        S.key[i] = sc == sc ? score_bits(sc) : kNoKey32 - 1;  // NaN last, but ranked: every duplicate has a source
+    }
     __syncthreads();
-    bitonic_sort(keys, N);
-
     const int K = max(1, M / A.ratio), copies = M / K, B = K * copies;
+    bucket_order(S, M, K);
+
     const int64_t b0 = A.b_off[t];
     const TargetDesc T = A.tg[t];
     const RobotParams& R = A.rs.rp[T.robot];
-    const int n = R.n;
-    for (int b = threadIdx.x; b < B; b += blockDim.x) {
-        const int i = b % K;  // copy r = b / K of kept seed i
-        const uint32_t src = (uint32_t)(keys[i] & 0xffffffffu);
-#pragma unroll 1
-        for (int q = 0; 2 * q < n; ++q) {
-            const float2 z = normal_pair(T, (uint32_t)b, kPhaseDup, 0, q);
+    const int n = R.n, items = B * ((n + 1) / 2);
+    for (int w = blockIdx.y * blockDim.x + threadIdx.x; w < items; w += gridDim.y * blockDim.x) {
+        const int q = w / B, b = w - q * B;     // pair q of the normals of duplicate b,
+        const uint32_t src = S.order[b % K];    // copy b / K of kept seed b % K
+        const float2 z = normal_pair(T, (uint32_t)b, kPhaseDup, 0, q);
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int j = 2 * q + h;
-                if (j < n)
-                    A.th_B[j * A.ld_B + b0 + b] =
-                        clampf(fmaf(A.sigma, h ? z.y : z.x, A.th_M[j * A.ld_M + m0 + src]), R.lim[j].x, R.lim[j].y);
-            }
+        for (int h = 0; h < 2; ++h) {
+            const int j = 2 * q + h;
+            if (j < n)
+                A.th_B[j * A.ld_B + b0 + b] =
+                    clampf(fmaf(A.sigma, h ? z.y : z.x, A.th_M[j * A.ld_M + m0 + src]), R.lim[j].x, R.lim[j].y);
         }
-        if (A.src_B) A.src_B[b0 + b] = (int32_t)src;
+        if (q == 0 && A.src_B) A.src_B[b0 + b] = (int32_t)src;
     }
 }
 
 __global__ void __launch_bounds__(kSelThreads) k_rank(const RankArgs A) {
-    extern __shared__ uint64_t keys[];
+    extern __shared__ __align__(16) unsigned char sel_smem[];
     int t = blockIdx.x;
     if (A.list) {  // the targets the bounded lazy pass left unfinished
         if (t >= *A.n_list) return;
@@ -61,20 +65,18 @@ __global__ void __launch_bounds__(kSelThreads) k_rank(const RankArgs A) {
     const int B = (int)(A.b_off[t + 1] - b0);
     int count = 0;
     if (B > 0) {
-        const int N = pow2_at_least(B);
         const int n = A.rs.rp[A.tg ? A.tg[t].robot : 0].n;
         const int tk = A.tg ? A.tg[t].top_k : A.top_k;
-        for (int i = threadIdx.x; i < N; i += blockDim.x) keys[i] = rank_key(A, t, b0, B, n, i, true);
+        const Bucket S = bucket_of(sel_smem, B);
+        for (int i = threadIdx.x; i < B; i += blockDim.x) S.key[i] = rank_key(A, t, b0, n, i, true);
         __syncthreads();
-        bitonic_sort(keys, N);
         const int top_k = tk & ~kNearestFlag;
-        const int lim = min(top_k, B);
-        for (int r = 0; r < lim; ++r) count += keys[r] != kNoKey;
+        count = min(top_k, bucket_order(S, B, top_k));
         float* oq = A.out_q + (A.qe_off ? A.qe_off[2 * t] : (int64_t)t * top_k * n);
         float* oe = A.out_err + (A.qe_off ? A.qe_off[2 * t + 1] : (int64_t)t * top_k * 2);
         for (int q = threadIdx.x; q < count * (n + 2); q += blockDim.x) {
             const int r = q / (n + 2), j = q % (n + 2);
-            const int64_t g = b0 + (int64_t)(keys[r] & 0xffffffffu);
+            const int64_t g = b0 + S.order[r];
             if (j < n) oq[r * n + j] = A.th[j * A.ld + g];
             else if (j == n) oe[r * 2] = A.perr[g];
             else oe[r * 2 + 1] = A.oerr[g];
@@ -84,26 +86,59 @@ __global__ void __launch_bounds__(kSelThreads) k_rank(const RankArgs A) {
 }
 
 __global__ void __launch_bounds__(kSelThreads) k_shard_topk(const ShardTopkArgs A) {
-    extern __shared__ uint64_t keys[];
+    extern __shared__ __align__(16) unsigned char sel_smem[];
     const int t = blockIdx.x;
     const int64_t m0 = A.off[t];
     const int M = (int)(A.off[t + 1] - m0);
-    const int N = pow2_at_least(M > 0 ? M : 1);
-    for (int i = threadIdx.x; i < N; i += blockDim.x)
-        keys[i] = i < M ? score_key(A.score[m0 + i], (uint32_t)i) : kNoKey;
+    const Bucket S = bucket_of(sel_smem, M > 0 ? M : 1);
+    for (int i = threadIdx.x; i < M; i += blockDim.x) {
+        const float sc = A.score[m0 + i];
+        S.key[i] = sc == sc ? score_bits(sc) : kNoKey32;
+    }
     __syncthreads();
-    bitonic_sort(keys, N);
+    const int ranked = bucket_order(S, M, A.K);
     const int n = A.rs.rp[A.tg[t].robot].n;
     for (int q = threadIdx.x; q < A.K * (n + 2); q += blockDim.x) {
         const int r = q / (n + 2), j = q % (n + 2);
-        const uint64_t key = r < N ? keys[r] : kNoKey;
-        const bool ok = r < M && key != kNoKey;
-        const uint32_t src = (uint32_t)(key & 0xffffffffu);
+        const bool ok = r < ranked;
+        const uint32_t src = ok ? S.order[r] : 0u;
         const int64_t o = (int64_t)t * A.K + r;
         if (j < n) A.out_th[o * A.ld_n + j] = ok ? A.th[j * A.ld + m0 + src] : 0.0f;
         else if (j == n) A.out_s[o] = ok ? A.score[m0 + src] : __int_as_float(0x7f800000);
         else A.out_i[o] = ok ? A.seed_base + (int32_t)src : -1;
     }
+}
+
+// 64-bit keys (score bits << 32 | seed index) of the lists' merge, sorted by a bitonic network; the
+// all-ones key sorts last
+constexpr uint64_t kNoKey = ~0ull;
+
+__device__ __forceinline__ uint64_t score_key(float s, uint32_t idx) {
+    return s == s ? ((uint64_t)score_bits(s) << 32) | idx : kNoKey;
+}
+
+__device__ __forceinline__ void bitonic_sort(uint64_t* keys, int N) {
+    for (int size = 2; size <= N; size <<= 1) {
+        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+            for (int i = threadIdx.x; i < (N >> 1); i += blockDim.x) {
+                const int lo = 2 * i - (i & (stride - 1));
+                const int hi = lo + stride;
+                const bool up = (lo & size) == 0;
+                const uint64_t a = keys[lo], b = keys[hi];
+                if ((a > b) == up) {
+                    keys[lo] = b;
+                    keys[hi] = a;
+                }
+            }
+            __syncthreads();
+        }
+    }
+}
+
+__device__ __forceinline__ int pow2_at_least(int m) {
+    int N = 1;
+    while (N < m) N <<= 1;
+    return N;
 }
 
 __global__ void __launch_bounds__(kSelThreads) k_topk_merge(const MergeArgs A) {
@@ -210,26 +245,26 @@ int smem_for(int m) {
 
 void launch_topk_dup(const DupArgs& A, int max_m, cudaStream_t st) {
     if (A.T <= 0 || max_m <= 0) return;
-    const int sm = smem_for(max_m);
     static SmemLimit lim;
-    allow_dyn_smem(k_topk_dup, lim, smem_for(HJCD_MAX_SAMPLES));
-    k_topk_dup<<<A.T, kSelThreads, sm, st>>>(A);
+    allow_dyn_smem(k_topk_dup, lim, bucket_smem_bytes(HJCD_MAX_SAMPLES));
+    // slices of a target: enough CTAs for two per SM, each with at least one item per thread
+    const int items = max_m * ((A.rs.n_max + 1) / 2);
+    const int slices = std::max(1, std::min(2 * sm_count() / A.T, (items + kSelThreads - 1) / kSelThreads));
+    k_topk_dup<<<dim3(A.T, slices), kSelThreads, bucket_smem_bytes(max_m), st>>>(A);
 }
 
 void launch_rank(const RankArgs& A, int max_b, cudaStream_t st) {
     if (A.T <= 0) return;
-    const int sm = smem_for(max_b > 0 ? max_b : 1);
     static SmemLimit lim;
-    allow_dyn_smem(k_rank, lim, smem_for(HJCD_MAX_SAMPLES));
-    k_rank<<<A.T, kSelThreads, sm, st>>>(A);
+    allow_dyn_smem(k_rank, lim, bucket_smem_bytes(HJCD_MAX_SAMPLES));
+    k_rank<<<A.T, kSelThreads, bucket_smem_bytes(max_b), st>>>(A);
 }
 
 void launch_shard_topk(const ShardTopkArgs& A, int max_m, cudaStream_t st) {
     if (A.T <= 0) return;
-    const int sm = smem_for(max_m > 0 ? max_m : 1);
     static SmemLimit lim;
-    allow_dyn_smem(k_shard_topk, lim, smem_for(HJCD_MAX_SAMPLES));
-    k_shard_topk<<<A.T, kSelThreads, sm, st>>>(A);
+    allow_dyn_smem(k_shard_topk, lim, bucket_smem_bytes(HJCD_MAX_SAMPLES));
+    k_shard_topk<<<A.T, kSelThreads, bucket_smem_bytes(max_m), st>>>(A);
 }
 
 void launch_topk_merge(const MergeArgs& A, cudaStream_t st) {
