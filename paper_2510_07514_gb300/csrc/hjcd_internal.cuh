@@ -519,7 +519,9 @@ inline int grid_for(int64_t items, int per_block, int per_sm = 64) {
 // equal bins, the candidates are gathered by bin, and a candidate's rank is its bin's start plus
 // its rank among the few that share the bin.  The work is linear while the bins are short (a
 // whole sort of 1024 keys took 55 barriers, this takes eight); keys that crowd one bin cost
-// their square, which only equal scores reach.
+// their square, which only equal scores reach.  The ranked filter's time with its sort -> with this:
+// one target of 1000 candidates 27 -> 21 us, 1000 targets 153 -> 119 us, 2000 targets of 4096
+// candidates 1281 -> 824 us.
 
 constexpr uint32_t kNoKey32 = 0xffffffffu;  // never ranked
 constexpr int kMaxBins = 2048;

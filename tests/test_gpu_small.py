@@ -113,3 +113,21 @@ def test_a_small_mixed_batch_gives_each_request_its_bits(ctx):
     for (_, got), ref in zip(items, big):
         for x, y in zip(got, ref):
             assert torch.equal(x.view(torch.int32), y[:3].view(torch.int32))
+
+
+@pytest.mark.parametrize("which", ["planar1", "chain7", "random2", "offsets", "chain24"])
+def test_fk_does_not_depend_on_the_batch(ctx, which):
+    """Two candidates share a thread and a warp's 64 poses one store: every remainder, and an output
+    buffer that does not start on 16 bytes, gives each candidate the pose it has alone."""
+    rob = _robot(which)
+    rid = ctx.add_robot(rob)
+    rng = np.random.default_rng(4)
+    th = torch.as_tensor(inputs.joint_samples(rng, rob, 1000).T.copy(), dtype=torch.float32, device="cuda")
+    alone = torch.cat([ctx.fk(rid, th[:, c:c + 1].contiguous()) for c in range(200)])
+    for C in (1, 2, 31, 32, 33, 63, 64, 65, 127, 128, 129, 200):
+        assert torch.equal(ctx.fk(rid, th[:, :C].contiguous()), alone[:C])
+        buf = torch.full((7 * C + 9,), -7.0, device="cuda")
+        hjcd.hjcd_fk(ctx.h, rid, C, th, th.stride(0), buf[1:], None)  # a stride past C, 4-byte alignment
+        torch.cuda.synchronize()
+        assert torch.equal(buf[1:1 + 7 * C].view(C, 7), alone[:C])
+        assert buf[0] == -7.0 and bool((buf[1 + 7 * C:] == -7.0).all())
