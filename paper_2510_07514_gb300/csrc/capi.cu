@@ -46,6 +46,18 @@ int pointer_kind(const void* p) {
     return 0;
 }
 
+int pointer_reach(const void* p, int device) {
+    if (!p) return -1;
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    if (a.type == cudaMemoryTypeManaged) return 2;
+    if (a.type == cudaMemoryTypeDevice) return a.device == device ? 2 : 1;
+    return 0;
+}
+
 bool pinned_host(const void* p) {
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
@@ -75,6 +87,7 @@ hjcd_status ensure_ws(hjcd_ctx* ctx, size_t bytes) {
 hjcd_status ensure_pin(hjcd_ctx* ctx, size_t bytes) {
     HJCD_CUDA(ctx, cudaEventSynchronize(ctx->pin_free));
     if (bytes <= ctx->pin_cap) return HJCD_OK;
+    HJCD_CUDA(ctx, cudaEventSynchronize(ctx->ws_free));  // a wave in flight may still write its flag there
     if (ctx->pin) HJCD_CUDA(ctx, cudaFreeHost(ctx->pin));
     ctx->pin = nullptr;
     ctx->pin_cap = 0;
@@ -491,10 +504,13 @@ hjcd_status hjcd_set_scene(hjcd_ctx* ctx, int32_t scene_id_or_new, int n_sph, co
     d.cell = cell.empty() ? nullptr : reinterpret_cast<const int32_t*>(base + o_cell);
     S.dev = d;
     S.perm = reinterpret_cast<const int32_t*>(base + o_perm);
-    HJCD_CUDA(ctx, cudaMemcpy(base, &S.dev, sizeof(SceneDev), cudaMemcpyHostToDevice));
-    HJCD_CUDA(ctx, cudaMemcpy(base + o_obj, buf.data(), 16 * (size_t)std::max(nf4, 1), cudaMemcpyHostToDevice));
-    if (!cell.empty()) HJCD_CUDA(ctx, cudaMemcpy(base + o_cell, cell.data(), 4 * cell.size(), cudaMemcpyHostToDevice));
-    HJCD_CUDA(ctx, cudaMemcpy(base + o_perm, perm.data(), 4 * perm.size(), cudaMemcpyHostToDevice));
+    // one copy (a scene rewritten every frame waits for each)
+    std::vector<char> image(bytes);
+    std::memcpy(image.data(), &S.dev, sizeof(SceneDev));
+    std::memcpy(image.data() + o_obj, buf.data(), 16 * (size_t)std::max(nf4, 1));
+    if (!cell.empty()) std::memcpy(image.data() + o_cell, cell.data(), 4 * cell.size());
+    std::memcpy(image.data() + o_perm, perm.data(), 4 * perm.size());
+    HJCD_CUDA(ctx, cudaMemcpy(base, image.data(), bytes, cudaMemcpyHostToDevice));
     S.live = true;
     *scene_id = id;
     return HJCD_OK;
@@ -513,18 +529,17 @@ static hjcd_status solve_items(hjcd_ctx* ctx, const WaveItem* items, int n_items
     if (W.T == 0) return HJCD_OK;
     if (ctx->ws_budget && W.bytes > ctx->ws_budget) return run_waves(ctx, items, n_items, P, s, W);
     if ((st = ensure_ws(ctx, W.bytes))) return st;
-    if ((st = ensure_pin(ctx, W.head))) return st;
+    if ((st = ensure_pin(ctx, W.pin_bytes))) return st;
     HJCD_CUDA(ctx, cudaStreamWaitEvent(s, ctx->ws_free, 0));
     const bool prof = ctx->profile;
-    if ((st = run_wave(ctx, W, items, P, ctx->ws, ctx->pin, s, prof ? ctx->ev : nullptr))) return st;
-    HJCD_CUDA(ctx, cudaEventRecord(ctx->pin_free, s));
+    if ((st = run_wave(ctx, W, items, P, ctx->ws, ctx->pin, s, prof ? ctx->ev : nullptr, ctx->pin_free))) return st;
     HJCD_CUDA(ctx, cudaEventRecord(ctx->ws_free, s));
     if (prof) ctx->ev_valid = true;
     if (W.host_out) {
         HJCD_CUDA(ctx, cudaStreamSynchronize(s));
-        int32_t flag = 0;
-        HJCD_CUDA(ctx, cudaMemcpy(&flag, wave_flag(W, ctx->ws), sizeof flag, cudaMemcpyDeviceToHost));
-        if (flag) return fail(ctx, HJCD_ETIMEOUT, "collision kernel: staging wait ran out");
+        if (W.staged)
+            for (int i = 0; i < n_items; ++i) take_results(W, i, items[i], ctx->pin);
+        if (*wave_flag(ctx->pin)) return fail(ctx, HJCD_ETIMEOUT, "collision kernel: staging wait ran out");
     }
     return HJCD_OK;
 }
@@ -540,7 +555,6 @@ static hjcd_status run_waves(hjcd_ctx* ctx, const WaveItem* items, int n_items, 
     const double per_seed = (double)whole.bytes / (double)std::max<int64_t>(whole.CM, 1);
     const int64_t cap_seeds = std::max<int64_t>(1, (int64_t)(0.9 * (double)ctx->ws_budget / per_seed));
     bool host_out = false;
-    WavePlan last;
     for (int i = 0; i < n_items; ++i) {
         const WaveItem& it = items[i];
         const int n = it.rob->P.n;
@@ -565,21 +579,18 @@ static hjcd_status run_waves(hjcd_ctx* ctx, const WaveItem* items, int n_items, 
             WavePlan W;
             if ((st = plan_wave(ctx, &sub, 1, P, &W))) return st;
             if ((st = ensure_ws(ctx, W.bytes))) return st;
-            if ((st = ensure_pin(ctx, W.head))) return st;  // waits until the previous chunk's image was copied
+            W.staged = false;  // the image is reused by the next chunk
+            if ((st = ensure_pin(ctx, W.pin_bytes))) return st;  // waits until the previous chunk's image was read
             HJCD_CUDA(ctx, cudaStreamWaitEvent(s, ctx->ws_free, 0));
-            if ((st = run_wave(ctx, W, &sub, P, ctx->ws, ctx->pin, s, nullptr))) return st;
-            HJCD_CUDA(ctx, cudaEventRecord(ctx->pin_free, s));
+            if ((st = run_wave(ctx, W, &sub, P, ctx->ws, ctx->pin, s, nullptr, ctx->pin_free))) return st;
             HJCD_CUDA(ctx, cudaEventRecord(ctx->ws_free, s));
             host_out = host_out || W.host_out;
-            last = std::move(W);
             t0 = t1;
         }
     }
     if (host_out) {
         HJCD_CUDA(ctx, cudaStreamSynchronize(s));
-        int32_t flag = 0;
-        HJCD_CUDA(ctx, cudaMemcpy(&flag, wave_flag(last, ctx->ws), sizeof flag, cudaMemcpyDeviceToHost));
-        if (flag) return fail(ctx, HJCD_ETIMEOUT, "collision kernel: staging wait ran out");
+        if (*wave_flag(ctx->pin)) return fail(ctx, HJCD_ETIMEOUT, "collision kernel: staging wait ran out");
     }
     return HJCD_OK;
 }
@@ -707,7 +718,7 @@ static hjcd_status stage_prologue(hjcd_ctx* ctx, int32_t robot_id, int n_targets
     if ((st = ensure_ws(ctx, align_up(sizeof(TargetDesc) * (size_t)n_targets)))) return st;
     HJCD_CUDA(ctx, cudaStreamWaitEvent(s, ctx->ws_free, 0));
     *d_tg = reinterpret_cast<TargetDesc*>(ctx->ws);
-    launch_pack_targets(targets_pq, n_targets, nullptr, stage_template(eps_pos, eps_ori, seed, 0, 0, 1, -1), *d_tg, s);
+    launch_pack_targets(targets_pq, n_targets, stage_template(eps_pos, eps_ori, seed, 0, 0, 1, -1), *d_tg, s);
     return after_launch(ctx, 1);
 }
 
@@ -955,9 +966,6 @@ hjcd_status hjcd_rank(hjcd_ctx* ctx, int32_t robot_id, int n_targets, const int6
                nullptr, out_q, out_err, out_count, q_ref, rob->P.n};
     a.eps_pos = eps_pos;
     a.eps_ori = eps_ori;
-    // rows past a target's count read NaN, as hjcd_solve leaves them
-    HJCD_CUDA(ctx, cudaMemsetAsync(out_q, 0xff, sizeof(float) * (size_t)n_targets * top_k * rob->P.n, s));
-    HJCD_CUDA(ctx, cudaMemsetAsync(out_err, 0xff, sizeof(float) * (size_t)n_targets * top_k * 2, s));
     launch_rank(a, max_b, s);
     return after_launch(ctx, 1);
 }
@@ -1165,7 +1173,7 @@ extern "C" hjcd_status hjcd_solve_noalloc(hjcd_ctx* ctx, int32_t robot_id, int32
     HJCD_CUDA(ctx, cudaMemsetAsync(queue, 0, sizeof(unsigned long long), s));
     HJCD_CUDA(ctx, cudaMemsetAsync(flag, 0, sizeof(int32_t), s));
     k_uniform_offsets<<<(T + 256) / 256, 256, 0, s>>>(d_moff, d_boff, T, M, B);
-    launch_pack_targets(targets_pq, T, nullptr,
+    launch_pack_targets(targets_pq, T,
                         stage_template(opts->eps_pos, opts->eps_ori, opts->seed, P.cd_max_iters, P.lm_max_iters, top_k,
                                        sc ? 0 : -1),
                         d_tg, s);
@@ -1221,9 +1229,6 @@ extern "C" hjcd_status hjcd_solve_noalloc(hjcd_ctx* ctx, int32_t robot_id, int32
     }
     RankArgs ra{rs, d_tg, T, d_boff, thB, CB, sB, pB, oB, collide ? hB : nullptr, top_k, nullptr,
                 out_q, out_err, out_count};
-    // rows past a target's count are NaN, as hjcd_solve leaves them (stream-ordered, no allocation)
-    HJCD_CUDA(ctx, cudaMemsetAsync(out_q, 0xff, sizeof(float) * (size_t)T * top_k * n, s));
-    HJCD_CUDA(ctx, cudaMemsetAsync(out_err, 0xff, sizeof(float) * (size_t)T * top_k * 2, s));
     launch_rank(ra, (int)B, s);
     return after_launch(ctx, collide ? 5 : 4);
 }
@@ -1279,7 +1284,7 @@ hjcd_status hjcd_shard_topk(hjcd_ctx* ctx, int32_t robot_id, int n_targets, cons
     TargetDesc* d_tg = reinterpret_cast<TargetDesc*>(W + o_tg);
     int64_t* d_off = reinterpret_cast<int64_t*>(W + o_off);
     k_uniform_offsets<<<(T + 256) / 256, 256, 0, s>>>(d_off, d_off + T + 1, T, Ms, Ms);
-    launch_pack_targets(targets_pq, T, nullptr,
+    launch_pack_targets(targets_pq, T,
                         stage_template(opts->eps_pos, opts->eps_ori, opts->seed, P.cd_max_iters, P.lm_max_iters, 1, -1),
                         d_tg, s);
     CcdArgs ca{};
@@ -1356,14 +1361,12 @@ hjcd_status hjcd_solve_from_topk(hjcd_ctx* ctx, int32_t robot_id, int32_t scene_
     uint8_t* hB = reinterpret_cast<uint8_t*>(W + o_hB);
     unsigned long long* queue = reinterpret_cast<unsigned long long*>(W + o_q);
     HJCD_CUDA(ctx, cudaMemsetAsync(queue, 0, 16, s));
-    HJCD_CUDA(ctx, cudaMemsetAsync(out_q, 0xff, sizeof(float) * (size_t)T * top_k * rob->P.n, s));
-    HJCD_CUDA(ctx, cudaMemsetAsync(out_err, 0xff, sizeof(float) * (size_t)T * top_k * 2, s));
     k_uniform_offsets<<<(T + 256) / 256, 256, 0, s>>>(d_boff + T + 1, d_boff, T, B, B);
     // each target keeps its index inside the whole request, which keys its random streams
     TargetDesc tmpl = stage_template(opts->eps_pos, opts->eps_ori, opts->seed, P.cd_max_iters, P.lm_max_iters, top_k,
                                      sc ? 0 : -1);
     tmpl.t_local = first_target;
-    launch_pack_targets(targets_pq, T, nullptr, tmpl, d_tg, s);
+    launch_pack_targets(targets_pq, T, tmpl, d_tg, s);
     const RobotSet rs = single_robot_set(*rob);
     KeptDupArgs da{rs, d_tg, T, (int32_t)K, kept_theta, d_boff, thB, CB, P.dup_sigma};
     launch_dup_kept(da, s);

@@ -108,7 +108,7 @@ hjcd_status hjcd_graph_create(hjcd_ctx* ctx, int n_items, const hjcd_batch_item*
     // image itself stays in the graph's pinned buffer for every replay
     const WavePlan& W = G->plan;
     cudaError_t e = cudaMalloc(&G->ws, W.bytes);
-    if (e == cudaSuccess) e = cudaMallocHost(&G->pin, W.head);
+    if (e == cudaSuccess) e = cudaMallocHost(&G->pin, W.pin_bytes);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&G->s, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&G->done, cudaEventDisableTiming);
     if (e != cudaSuccess) {
@@ -166,9 +166,7 @@ hjcd_status hjcd_graph_check(hjcd_graph* G) {
     if (!G) return HJCD_EINVAL;
     hjcd_ctx* ctx = G->ctx;
     HJCD_CUDA(ctx, cudaEventSynchronize(G->done));
-    int32_t flag = 0;
-    HJCD_CUDA(ctx, cudaMemcpy(&flag, wave_flag(G->plan, G->ws), sizeof flag, cudaMemcpyDeviceToHost));
-    if (flag) return fail(ctx, HJCD_ETIMEOUT, "collision kernel: staging wait ran out");
+    if (*wave_flag(G->pin)) return fail(ctx, HJCD_ETIMEOUT, "collision kernel: staging wait ran out");
     return HJCD_OK;
 }
 

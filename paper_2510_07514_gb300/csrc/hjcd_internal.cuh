@@ -709,10 +709,19 @@ struct DupArgs {
     float sigma;
 };
 
-// Output of target t: solutions at out_q + qe_off[2t] (top_k rows of its
-// robot's n), errors at out_err + qe_off[2t+1] (top_k pairs).  With tg null
-// every target takes top_k and robot 0; with qe_off null the blocks are
-// contiguous in target order.
+// Where a wave's target comes from and where its results go: its pose and reference configuration
+// (device or pinned host memory; null: no reference) and its blocks of the outputs (device memory).
+struct TargetIo {
+    const float* pose;  // [7]
+    const float* ref;   // [n]
+    float* q;           // [top_k][n]
+    float* err;         // [top_k][2]
+    int32_t* count;
+};
+
+// Output of target t: to io[t], or with io null in contiguous blocks in target order (top_k rows of
+// its robot's n, top_k pairs of errors); the rows past its count are filled with NaN.  With tg null
+// every target takes top_k and robot 0.
 struct RankArgs {
     RobotSet rs;
     const TargetDesc* tg;
@@ -723,7 +732,7 @@ struct RankArgs {
     const float *score, *perr, *oerr;
     const uint8_t* hit;
     int top_k;
-    const int64_t* qe_off;
+    const TargetIo* io;
     float* out_q;
     float* out_err;
     int32_t* out_count;
@@ -739,6 +748,20 @@ struct RankArgs {
     // tolerances of every target when tg is null (with tg: each target row's own)
     float eps_pos, eps_ori;
 };
+
+// Target t's output blocks
+struct RankOut {
+    float* q;
+    float* err;
+    int32_t* count;
+};
+__device__ __forceinline__ RankOut rank_out(const RankArgs& A, int t, int top_k, int n) {
+    if (A.io) {
+        const TargetIo io = A.io[t];
+        return RankOut{io.q, io.err, io.count};
+    }
+    return RankOut{A.out_q + (int64_t)t * top_k * n, A.out_err + (int64_t)t * top_k * 2, A.out_count + t};
+}
 
 // Ranking key of candidate i of target t (candidates [b0, b0 + B), robot DoF
 // n), never for a colliding candidate (with use_hit) or a non-finite score.
@@ -801,9 +824,6 @@ struct CollideArgs {
     int32_t list_bmax;
 };
 
-// Fill p and q of the target rows from [T][7] poses (quaternion normalised; a
-// zero or non-finite one marks the row invalid with eps_pos = -1).  With meta
-// non-null the other fields come from meta[t], else from tmpl with t_local = t.
 // Per target t: the K = max(1, floor(M_full / ratio)) lowest scores of its
 // candidates [off[t], off[t+1]) (ties to the lower index), written as score,
 // seed index (seed_base + index in the target) and joint vector; +inf / -1
@@ -850,8 +870,22 @@ struct KeptDupArgs {
 };
 void launch_dup_kept(const KeptDupArgs& A, cudaStream_t st);
 
-void launch_pack_targets(const float* pq7, int T, const TargetDesc* meta, const TargetDesc& tmpl, TargetDesc* out,
-                         cudaStream_t st);
+// First launch of a wave: copies the head's image (`bytes`, a multiple of 16, both sides 16-byte
+// aligned) from pinned host memory to the workspace, fills in the target rows' poses and the
+// reference configurations, zeroes the wave's queue heads and error flag.
+struct WaveInitArgs {
+    const char* pin;  // the image
+    char* ws;
+    size_t bytes, o_tg, o_io, o_rp;  // the head's size; target rows, TargetIo rows and robot tables inside it
+    int32_t T;
+    float* ref;       // [T][ld_ref], or null
+    int32_t ld_ref;
+    unsigned long long* zero;  // 6 words
+    int32_t* flag;
+};
+void launch_wave_init(const WaveInitArgs& A, cudaStream_t st);
+// Target rows of [T][7] poses: tmpl with t_local counting up from its own.
+void launch_pack_targets(const float* pq7, int T, const TargetDesc& tmpl, TargetDesc* out, cudaStream_t st);
 void launch_fk(const RobotParams& R, int64_t C, const float* th, int64_t ld, float* out, cudaStream_t st);
 void launch_sample(const RobotParams& R, uint64_t seed, CandMap map, int64_t C, float* th, int64_t ld,
                    cudaStream_t st);

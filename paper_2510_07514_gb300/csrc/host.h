@@ -103,6 +103,7 @@ struct Carve {
 
 hjcd_status after_launch(hjcd_ctx* ctx, int kernels, const char* what = "kernel");
 int pointer_kind(const void* p);  // 1 device/managed, 0 host, -1 null
+int pointer_reach(const void* p, int device);  // as pointer_kind, but 2 where kernels on `device` can use p themselves
 bool pinned_host(const void* p);
 hjcd_status make_current(hjcd_ctx* ctx);
 hjcd_status ensure_ws(hjcd_ctx* ctx, size_t bytes);
@@ -155,31 +156,43 @@ struct WavePlan {
     std::vector<SceneEnt> scenes;
     std::vector<int> item_t0;
     std::vector<int64_t> item_q0, item_e0;
-    std::vector<char> dev_tgt, dev_q, dev_e, dev_c, dev_ref;
+    // per item, pointer_reach of its targets, outputs and reference configurations
+    std::vector<char> at_tgt, at_q, at_e, at_c, at_ref;
     bool has_ref = false;
     int64_t q_total = 0, e_total = 0;
-    // head: copied from the pinned image to the start of the workspace in one copy
-    size_t o_rp = 0, o_rd = 0, o_sd = 0, o_tg = 0, o_moff = 0, o_boff = 0, o_qe = 0, o_pq7 = 0, o_ref = 0, o_inl = 0,
-           head = 0;
+    // head: the start of the pinned image, copied to the start of the workspace by the first launch
+    size_t o_rp = 0, o_rd = 0, o_sd = 0, o_tg = 0, o_moff = 0, o_boff = 0, o_io = 0, o_inl = 0, head = 0;
+    // the rest of the pinned image: poses and references from host memory, the host items' results
+    // (q, err, count) when they are small; pin_bytes: the image and kFlagBytes before it
+    size_t p_pose = 0, p_ref = 0, p_q = 0, p_e = 0, p_c = 0, pin_bytes = 0;
+    bool staged = false;  // host results go through the pinned image
     // the rest of the workspace
-    size_t o_thM = 0, o_thM2 = 0, o_sM = 0, o_thB = 0, o_sB = 0, o_pB = 0, o_oB = 0, o_hB = 0, o_q = 0, o_e = 0, o_c = 0,
-           o_ul = 0, o_sg = 0, o_qf = 0, bytes = 0;
+    size_t o_pose = 0, o_pref = 0, o_ref = 0, o_thM = 0, o_thM2 = 0, o_sM = 0, o_thB = 0, o_sB = 0, o_pB = 0, o_oB = 0,
+           o_hB = 0, o_q = 0, o_e = 0, o_c = 0, o_ul = 0, o_sg = 0, o_qf = 0, bytes = 0;
     bool host_out = false;  // some output goes to host memory
 };
+constexpr size_t kStagedResults = 1 << 20;  // most bytes of results that go through the pinned image
+// A pinned buffer starts with the error flag, at one place whatever the wave: a wave in flight may
+// still write it while the next wave's image, behind it, is filled.
+constexpr size_t kFlagBytes = 256;
 
 // Validate the items and lay out the wave.  Caps from P unless an item sets
 // its own (cd_iters / lm_iters >= 0).
 hjcd_status plan_wave(hjcd_ctx* ctx, const WaveItem* items, int n_items, const hjcd_params& P, WavePlan* out);
 
-// Fill the pinned image (plan.head bytes at `pin`), copy it to `ws`, run the
-// launch sequence of Alg. 2 over the whole wave and copy each item's results
-// out, all on stream s.  Nothing is synchronised.  ev (6 events or null) is
-// recorded around the phases.
+// Fill the pinned buffer (plan.pin_bytes at `pin`) and run the launch sequence of Alg. 2 over the whole
+// wave on stream s.  Results in device memory are written by the kernels; those in host memory are
+// in the image when the stream gets there and are copied from it by take_results (plan.staged), or
+// are copied by the stream.  Nothing is synchronised.  read (or null) is recorded once the image has
+// been read (its flag and results are still written); ev (6 events or null) around the phases.
 hjcd_status run_wave(hjcd_ctx* ctx, const WavePlan& W, const WaveItem* items, const hjcd_params& P, char* ws,
-                     char* pin, cudaStream_t s, cudaEvent_t* ev);
+                     char* pin, cudaStream_t s, cudaEvent_t* ev, cudaEvent_t read = nullptr);
 
-// The wave's error flag (int32, nonzero: a bounded device wait ran out).
-inline int32_t* wave_flag(const WavePlan& W, char* ws) { return reinterpret_cast<int32_t*>(ws + W.o_qf + 8); }
+// Staged results of item i to its buffers (after the stream has finished the wave).
+void take_results(const WavePlan& W, int i, const WaveItem& it, const char* pin);
+
+// The error flag of the last wave run through a pinned buffer (nonzero: a bounded device wait ran out).
+inline int32_t* wave_flag(char* pin) { return reinterpret_cast<int32_t*>(pin); }
 
 // ---- serving loop --------------------------------------------------------------
 

@@ -389,7 +389,7 @@ __device__ __forceinline__ bool collide_prologue(const CollideArgs& A, unsigned 
             // give up: flag the error, give the copy one more bounded wait (the full limit: the
             // copy must land before the CTA's shared memory is released)
             if (threadIdx.x == 0) {
-                atomicExch(A.err_flag, 1);
+                *(volatile int32_t*)A.err_flag = 1;  // any CTA's will do (may be host memory)
                 mbar_wait_bounded(bar, 0);
             }
             return false;
@@ -417,7 +417,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_collide(const CollideAr
     const SceneDev sc0 = A.n_scenes > 0 ? A.scenes[0] : SceneDev{nullptr, 0, 0};
     const int n_obj4 = UNIFORM ? sc0.n_sph + 2 * sc0.n_box : 0;
     if (n_obj4 > (UNIFORM ? A.max_obj4 : 0)) {  // the scene outgrew the shared memory the host sized
-        if (threadIdx.x == 0) atomicExch(A.err_flag, 2);
+        if (threadIdx.x == 0) *(volatile int32_t*)A.err_flag = 2;  // any CTA's will do (may be host memory)
         return;
     }
     // list mode: the candidates of the listed targets only (none listed: nothing to stage)
@@ -495,19 +495,26 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_rank_lazy(const Collide
     __shared__ int n_found;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int t = blockIdx.x;
+    const TargetDesc& T = R.tg[t];
     const SceneDev sc0 = A.n_scenes > 0 ? A.scenes[0] : SceneDev{nullptr, 0, 0};
     const int n_obj4 = UNIFORM ? sc0.n_sph + 2 * sc0.n_box : 0;
-    if (n_obj4 > (UNIFORM ? A.max_obj4 : 0)) {
-        if (threadIdx.x == 0) atomicExch(A.err_flag, 2);
+    const bool outgrown = n_obj4 > (UNIFORM ? A.max_obj4 : 0);
+    if (outgrown && threadIdx.x == 0) *(volatile int32_t*)A.err_flag = 2;  // any CTA's will do (may be host memory)
+    const CollideLayout L =
+        collide_smem_layout(outgrown ? 0 : n_obj4, A.rs.n, A.rs.n_max + 2, A.rs.ns_max, A.rs.pairs_max);
+    const RobotParams* rob;
+    if (outgrown || !collide_prologue<UNIFORM>(A, smem, L, sc0, n_obj4, &rob)) {
+        // no verdicts: no solutions (the error flag is set)
+        const int tk = T.top_k & ~kNearestFlag, nj = A.rs.rp[T.robot].n;
+        const RankOut O = rank_out(R, t, tk, nj);
+        for (int q = threadIdx.x; q < tk * nj; q += blockDim.x) O.q[q] = __int_as_float(0xffffffff);
+        for (int q = threadIdx.x; q < tk * 2; q += blockDim.x) O.err[q] = __int_as_float(0xffffffff);
+        if (threadIdx.x == 0) *O.count = 0;
         return;
     }
-    const CollideLayout L = collide_smem_layout(n_obj4, A.rs.n, A.rs.n_max + 2, A.rs.ns_max, A.rs.pairs_max);
-    const RobotParams* rob;
-    if (!collide_prologue<UNIFORM>(A, smem, L, sc0, n_obj4, &rob)) return;
     const WarpBufs Bf = warp_bufs(smem, L, A);
     const float4* s_scene = reinterpret_cast<const float4*>(smem);
 
-    const TargetDesc& T = R.tg[t];
     const int rid = T.robot, sid = UNIFORM ? 0 : T.scene;
     const int n = rob[rid].n;
     const int64_t b0 = R.b_off[t];
@@ -571,16 +578,17 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_rank_lazy(const Collide
         if (threadIdx.x == 0) R.list[atomicAdd(R.n_list, 1)] = t;
         return;
     }
-    float* oq = R.out_q + R.qe_off[2 * t];
-    float* oe = R.out_err + R.qe_off[2 * t + 1];
-    for (int q = threadIdx.x; q < count * (n + 2); q += blockDim.x) {
+    const RankOut O = rank_out(R, t, top_k, n);
+    for (int q = threadIdx.x; q < top_k * (n + 2); q += blockDim.x) {
         const int r = q / (n + 2), j = q % (n + 2);
-        const int64_t g = b0 + S.order[picks[r]];
-        if (j < n) oq[r * n + j] = R.th[j * R.ld + g];
-        else if (j == n) oe[r * 2] = R.perr[g];
-        else oe[r * 2 + 1] = R.oerr[g];
+        const bool ok = r < count;
+        const int64_t g = b0 + (ok ? S.order[picks[r]] : 0);
+        const float none = __int_as_float(0xffffffff);
+        if (j < n) O.q[r * n + j] = ok ? R.th[j * R.ld + g] : none;
+        else if (j == n) O.err[r * 2] = ok ? R.perr[g] : none;
+        else O.err[r * 2 + 1] = ok ? R.oerr[g] : none;
     }
-    if (threadIdx.x == 0) R.out_count[t] = count;
+    if (threadIdx.x == 0) *O.count = count;
 }
 
 template <int SPL, bool UNIFORM, bool GRID>
@@ -678,7 +686,7 @@ void launch_contacts(const RobotParams& R, const RobotDev& rd, const SceneDev& s
 }
 
 bool launch_rank_lazy(const CollideArgs& A, const RankArgs& R, int max_b, int depth, cudaStream_t st) {
-    if (R.T <= 0 || A.rs.ns_max <= 0 || !R.tg || !R.qe_off) return false;
+    if (R.T <= 0 || A.rs.ns_max <= 0 || !R.tg || !R.io) return false;
     const bool uni = A.uniform && A.rs.n == 1 && A.n_scenes <= 1 && A.max_obj4 <= kMaxStagedObj4;
     const int n4 = A.n_scenes == 1 ? A.max_obj4 : 0;
     if (uni && A.has_grid) return launch_rank_lazy_s<true, true>(A, R, n4, max_b, depth, st);

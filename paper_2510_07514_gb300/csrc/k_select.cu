@@ -63,26 +63,23 @@ __global__ void __launch_bounds__(kSelThreads) k_rank(const RankArgs A) {
     }
     const int64_t b0 = A.b_off[t];
     const int B = (int)(A.b_off[t + 1] - b0);
-    int count = 0;
-    if (B > 0) {
-        const int n = A.rs.rp[A.tg ? A.tg[t].robot : 0].n;
-        const int tk = A.tg ? A.tg[t].top_k : A.top_k;
-        const Bucket S = bucket_of(sel_smem, B);
-        for (int i = threadIdx.x; i < B; i += blockDim.x) S.key[i] = rank_key(A, t, b0, n, i, true);
-        __syncthreads();
-        const int top_k = tk & ~kNearestFlag;
-        count = min(top_k, bucket_order(S, B, top_k));
-        float* oq = A.out_q + (A.qe_off ? A.qe_off[2 * t] : (int64_t)t * top_k * n);
-        float* oe = A.out_err + (A.qe_off ? A.qe_off[2 * t + 1] : (int64_t)t * top_k * 2);
-        for (int q = threadIdx.x; q < count * (n + 2); q += blockDim.x) {
-            const int r = q / (n + 2), j = q % (n + 2);
-            const int64_t g = b0 + S.order[r];
-            if (j < n) oq[r * n + j] = A.th[j * A.ld + g];
-            else if (j == n) oe[r * 2] = A.perr[g];
-            else oe[r * 2 + 1] = A.oerr[g];
-        }
+    const int n = A.rs.rp[A.tg ? A.tg[t].robot : 0].n;
+    const int top_k = (A.tg ? A.tg[t].top_k : A.top_k) & ~kNearestFlag;
+    const RankOut O = rank_out(A, t, top_k, n);
+    const Bucket S = bucket_of(sel_smem, B > 0 ? B : 1);
+    for (int i = threadIdx.x; i < B; i += blockDim.x) S.key[i] = rank_key(A, t, b0, n, i, true);
+    __syncthreads();
+    const int count = min(top_k, bucket_order(S, B, top_k));
+    for (int q = threadIdx.x; q < top_k * (n + 2); q += blockDim.x) {
+        const int r = q / (n + 2), j = q % (n + 2);
+        const bool ok = r < count;
+        const int64_t g = b0 + (ok ? S.order[r] : 0);
+        const float none = __int_as_float(0xffffffff);
+        if (j < n) O.q[r * n + j] = ok ? A.th[j * A.ld + g] : none;
+        else if (j == n) O.err[r * 2] = ok ? A.perr[g] : none;
+        else O.err[r * 2 + 1] = ok ? A.oerr[g] : none;
     }
-    if (threadIdx.x == 0) A.out_count[t] = count;
+    if (threadIdx.x == 0) *O.count = count;
 }
 
 __global__ void __launch_bounds__(kSelThreads) k_shard_topk(const ShardTopkArgs A) {
@@ -207,22 +204,13 @@ __global__ void __launch_bounds__(kSelThreads) k_dup_kept(const KeptDupArgs A) {
     }
 }
 
-__global__ void k_pack_targets(const float* pq7, int T, const TargetDesc* meta, const TargetDesc tmpl,
-                               TargetDesc* out) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= T) return;
-    const float* s = pq7 + 7 * (int64_t)t;
+// pose s (px py pz qw qx qy qz) into row d, its quaternion normalised; a zero or non-finite one marks
+// the target invalid
+__device__ __forceinline__ void set_pose(TargetDesc& d, const float* s) {
     const float qw = s[3], qx = s[4], qy = s[5], qz = s[6];
     const float nn = qw * qw + qx * qx + qy * qy + qz * qz;
     const bool ok = nn > 0.0f && isfinite(nn);
     const float r = ok ? rsqrtf(nn) : 0.0f;
-    TargetDesc d;
-    if (meta) {
-        d = meta[t];
-    } else {
-        d = tmpl;
-        d.t_local = tmpl.t_local + t;  // the template holds the index of the first target
-    }
     d.p[0] = s[0];
     d.p[1] = s[1];
     d.p[2] = s[2];
@@ -230,8 +218,48 @@ __global__ void k_pack_targets(const float* pq7, int T, const TargetDesc* meta, 
     d.q[1] = qx * r;
     d.q[2] = qy * r;
     d.q[3] = qz * r;
-    if (!ok) d.eps_pos = -1.0f;  // a zero quaternion marks the target invalid
+    if (!ok) d.eps_pos = -1.0f;
+}
+
+__global__ void k_pack_targets(const float* pq7, int T, const TargetDesc tmpl, TargetDesc* out) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= T) return;
+    TargetDesc d = tmpl;
+    d.t_local = tmpl.t_local + t;  // the template holds the index of the first target
+    set_pose(d, pq7 + 7 * (int64_t)t);
     out[t] = d;
+}
+
+// One launch in place of a copy of the head, copies of the poses and references, the packing of the
+// poses and three fills: a small wave's time is its chain of stream operations.  The image is read
+// from pinned host memory directly.  With the results written in place (or into the pinned buffer)
+// instead of copied: one Panda pose of 64 seeds 148 -> 123 us, of 1000 seeds between host buffers
+// 228 -> 189 us.
+__global__ void __launch_bounds__(256) k_wave_init(const WaveInitArgs A) {
+    const size_t tid = blockIdx.x * (size_t)blockDim.x + threadIdx.x, nth = (size_t)gridDim.x * blockDim.x;
+    if (tid < 6) A.zero[tid] = 0;
+    if (tid == 6) *A.flag = 0;
+    const uint4* src = reinterpret_cast<const uint4*>(A.pin);
+    uint4* dst = reinterpret_cast<uint4*>(A.ws);
+    const size_t g0 = A.o_tg / 16, g1 = g0 + (size_t)A.T * (sizeof(TargetDesc) / 16);  // the target rows: below
+    for (size_t i = tid; i < A.bytes / 16; i += nth)
+        if (i < g0 || i >= g1) dst[i] = __ldcv(src + i);
+    const RobotParams* rp = reinterpret_cast<const RobotParams*>(A.pin + A.o_rp);
+    for (size_t t = tid; t < (size_t)A.T; t += nth) {
+        union {
+            uint4 w[sizeof(TargetDesc) / 16];
+            TargetDesc d;
+        } row;
+#pragma unroll
+        for (int k = 0; k < (int)(sizeof(TargetDesc) / 16); ++k) row.w[k] = __ldcv(src + g0 + t * (sizeof(TargetDesc) / 16) + k);
+        const TargetIo* io = reinterpret_cast<const TargetIo*>(A.pin + A.o_io) + t;
+        set_pose(row.d, io->pose);
+        reinterpret_cast<TargetDesc*>(A.ws + A.o_tg)[t] = row.d;
+        if (A.ref && io->ref) {
+            const int n = rp[row.d.robot].n;
+            for (int j = 0; j < n; ++j) A.ref[t * A.ld_ref + j] = io->ref[j];
+        }
+    }
 }
 
 int smem_for(int m) {
@@ -280,10 +308,13 @@ void launch_dup_kept(const KeptDupArgs& A, cudaStream_t st) {
     k_dup_kept<<<A.T, kSelThreads, 0, st>>>(A);
 }
 
-void launch_pack_targets(const float* pq7, int T, const TargetDesc* meta, const TargetDesc& tmpl, TargetDesc* out,
-                         cudaStream_t st) {
+void launch_pack_targets(const float* pq7, int T, const TargetDesc& tmpl, TargetDesc* out, cudaStream_t st) {
     if (T <= 0) return;
-    k_pack_targets<<<(T + 127) / 128, 128, 0, st>>>(pq7, T, meta, tmpl, out);
+    k_pack_targets<<<(T + 127) / 128, 128, 0, st>>>(pq7, T, tmpl, out);
+}
+
+void launch_wave_init(const WaveInitArgs& A, cudaStream_t st) {
+    k_wave_init<<<grid_for(std::max<int64_t>(A.T, (int64_t)(A.bytes / 16)), 256, 8), 256, 0, st>>>(A);
 }
 
 }  // namespace hjcd

@@ -51,9 +51,9 @@ struct Slot {
     cudaStream_t s = nullptr;
     char* ws = nullptr;
     size_t ws_cap = 0;
-    char* pin = nullptr;  // head image
+    char* pin = nullptr;  // head image, error flag and (when small) results
     size_t pin_cap = 0;
-    char* pout = nullptr;  // results
+    char* pout = nullptr;  // larger results
     size_t pout_cap = 0;
     std::vector<Req*> reqs;
     std::vector<WaveItem> items;
@@ -128,18 +128,23 @@ constexpr size_t kSlotPin0 = size_t(4) << 20;
 
 // Copy a finished batch's results to the callers' buffers.
 void Server::finish(Slot& sl) {
-    int32_t flag = 0;
     const WavePlan& W = sl.plan;
-    // the flag travels with the results (last 4 bytes of the result image)
-    std::memcpy(&flag, sl.pout + W.q_total * 4 + W.e_total * 4 + (size_t)W.T * 4, sizeof flag);
+    const int32_t flag = *wave_flag(sl.pin);
     const auto now = Clock::now();
     for (size_t i = 0; i < sl.reqs.size(); ++i) {
         Req* r = sl.reqs[i];
         const int T = (int)(r->targets.size() / 7);
         const size_t nq = (size_t)T * r->opts.top_k * r->n, ne = (size_t)T * r->opts.top_k * 2;
-        std::memcpy(r->out_q, sl.pout + 4 * (W.item_q0[i]), 4 * nq);
-        std::memcpy(r->out_err, sl.pout + 4 * (W.q_total + W.item_e0[i]), 4 * ne);
-        std::memcpy(r->out_count, sl.pout + 4 * (W.q_total + W.e_total + W.item_t0[i]), 4 * (size_t)T);
+        if (W.staged) {
+            sl.items[i].out_q = r->out_q;
+            sl.items[i].out_err = r->out_err;
+            sl.items[i].out_count = r->out_count;
+            take_results(W, (int)i, sl.items[i], sl.pin);
+        } else {
+            std::memcpy(r->out_q, sl.pout + 4 * (W.item_q0[i]), 4 * nq);
+            std::memcpy(r->out_err, sl.pout + 4 * (W.q_total + W.item_e0[i]), 4 * ne);
+            std::memcpy(r->out_count, sl.pout + 4 * (W.q_total + W.e_total + W.item_t0[i]), 4 * (size_t)T);
+        }
         r->status = flag ? HJCD_ETIMEOUT : HJCD_OK;
         r->t_done = now;
         r->batch_requests = (int32_t)sl.reqs.size();
@@ -200,7 +205,7 @@ bool Server::launch(Slot& sl, std::vector<Req*>& take) {
             st = plan_wave(c, items.data(), (int)items.size(), P, &W);
         }
         if (st == HJCD_OK && W.bytes > slot_budget) st = HJCD_ENOMEM;
-        const size_t res_bytes = 4 * (size_t)(W.q_total + W.e_total + W.T) + 16;
+        const size_t res_bytes = W.staged ? 0 : 4 * (size_t)(W.q_total + W.e_total + W.T);
         if (st == HJCD_OK && W.bytes > sl.ws_cap) {
             // stream-ordered: freeing the old workspace does not wait for the other streams
             if (sl.ws) cudaFreeAsync(sl.ws, sl.s);
@@ -214,15 +219,15 @@ bool Server::launch(Slot& sl, std::vector<Req*>& take) {
                 sl.ws_cap = cap;
             }
         }
-        if (st == HJCD_OK && W.head > sl.pin_cap) {
+        if (st == HJCD_OK && W.pin_bytes > sl.pin_cap) {
             if (sl.pin) cudaFreeHost(sl.pin);
             sl.pin = nullptr;
             sl.pin_cap = 0;
-            if (cudaMallocHost(&sl.pin, grow(W.head)) != cudaSuccess) {
+            if (cudaMallocHost(&sl.pin, grow(W.pin_bytes)) != cudaSuccess) {
                 cudaGetLastError();
                 st = HJCD_ENOMEM;
             } else {
-                sl.pin_cap = grow(W.head);
+                sl.pin_cap = grow(W.pin_bytes);
             }
         }
         if (st == HJCD_OK && res_bytes > sl.pout_cap) {
@@ -236,8 +241,8 @@ bool Server::launch(Slot& sl, std::vector<Req*>& take) {
                 sl.pout_cap = grow(res_bytes);
             }
         }
-        if (st == HJCD_OK) {
-            // results land in the slot's pinned buffer: q | err | count | flag
+        if (st == HJCD_OK && !W.staged) {
+            // results land in the slot's pinned buffer: q | err | count
             for (size_t i = 0; i < items.size(); ++i) {
                 items[i].out_q = reinterpret_cast<float*>(sl.pout) + W.item_q0[i];
                 items[i].out_err = reinterpret_cast<float*>(sl.pout) + W.q_total + W.item_e0[i];
@@ -248,9 +253,7 @@ bool Server::launch(Slot& sl, std::vector<Req*>& take) {
         const auto now = Clock::now();
         if (st == HJCD_OK) st = run_wave(c, W, items.data(), P, sl.ws, sl.pin, sl.s, nullptr);
         if (st == HJCD_OK) {
-            cudaError_t e = cudaMemcpyAsync(sl.pout + 4 * (size_t)(W.q_total + W.e_total + W.T), wave_flag(W, sl.ws), 4,
-                                            cudaMemcpyDeviceToHost, sl.s);
-            if (e == cudaSuccess) e = cudaLaunchHostFunc(sl.s, on_batch_done, new CbArg{this, &sl});
+            const cudaError_t e = cudaLaunchHostFunc(sl.s, on_batch_done, new CbArg{this, &sl});
             if (e != cudaSuccess) {
                 fatal = cudaGetErrorString(e);
                 st = HJCD_ECUDA;

@@ -116,14 +116,13 @@ hjcd_status hjcd_autotune(hjcd_ctx* ctx, int n_items, const hjcd_batch_item* ite
         hjcd_status r;
         if ((r = plan_wave(ctx, w.data(), n_items, P, &W))) return r;
         if ((r = ensure_ws(ctx, W.bytes))) return r;
-        if ((r = ensure_pin(ctx, W.head))) return r;
+        if ((r = ensure_pin(ctx, W.pin_bytes))) return r;
         std::vector<double> ms;
         for (int k = 0; k <= repeats; ++k) {
             HJCD_CUDA(ctx, cudaStreamWaitEvent(s, ctx->ws_free, 0));
             HJCD_CUDA(ctx, cudaEventRecord(e0, s));
-            if ((r = run_wave(ctx, W, w.data(), P, ctx->ws, ctx->pin, s, nullptr))) return r;
+            if ((r = run_wave(ctx, W, w.data(), P, ctx->ws, ctx->pin, s, nullptr, ctx->pin_free))) return r;
             HJCD_CUDA(ctx, cudaEventRecord(e1, s));
-            HJCD_CUDA(ctx, cudaEventRecord(ctx->pin_free, s));
             HJCD_CUDA(ctx, cudaEventRecord(ctx->ws_free, s));
             HJCD_CUDA(ctx, cudaEventSynchronize(e1));
             float t = 0.0f;

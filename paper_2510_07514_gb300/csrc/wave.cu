@@ -9,14 +9,15 @@
 // Device layout of a wave (one workspace):
 //   head  robot kinematic tables | robot collision descriptors | scene
 //         descriptors | target rows | seed offsets m_off | candidate offsets
-//         b_off | output offsets | target poses [T][7] | inline obstacles
-//         (written in pinned host memory, copied with one transfer)
+//         b_off | each target's sources and outputs | inline obstacles
+//         (written in pinned host memory, copied and completed by the first launch)
 //   PO-CCD joint vectors [n_max][CM] and scores [CM]
 //   PJ-IK joint vectors [n_max][CB], scores, errors, collision verdicts [CB]
-//   outputs (each request's block as it wants it), queue head, error flag
+//   results that the kernels cannot write in place, queue heads
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 
 #include "host.h"
 
@@ -31,11 +32,11 @@ hjcd_status plan_wave(hjcd_ctx* ctx, const WaveItem* items, int n_items, const h
     W.item_t0.resize(n_items);
     W.item_q0.resize(n_items);
     W.item_e0.resize(n_items);
-    W.dev_tgt.resize(n_items);
-    W.dev_q.resize(n_items);
-    W.dev_e.resize(n_items);
-    W.dev_c.resize(n_items);
-    W.dev_ref.resize(n_items);
+    W.at_tgt.resize(n_items);
+    W.at_q.resize(n_items);
+    W.at_e.resize(n_items);
+    W.at_c.resize(n_items);
+    W.at_ref.resize(n_items);
     size_t inl_bytes = 0;
     for (int i = 0; i < n_items; ++i) {
         const WaveItem& it = items[i];
@@ -80,14 +81,15 @@ hjcd_status plan_wave(hjcd_ctx* ctx, const WaveItem* items, int n_items, const h
             inl_bytes += align_up(16 * (size_t)(it.inl_nsph + 2 * it.inl_nbox), 16);
         }
         W.item_scene[i] = sidx;
-        W.dev_tgt[i] = it.T > 0 && pointer_kind(it.targets) == 1;
-        W.dev_q[i] = it.T > 0 && pointer_kind(it.out_q) == 1;
-        W.dev_e[i] = it.T > 0 && pointer_kind(it.out_err) == 1;
-        W.dev_c[i] = it.T > 0 && pointer_kind(it.out_count) == 1;
-        W.dev_ref[i] = it.T > 0 && it.q_ref && pointer_kind(it.q_ref) == 1;
-        W.has_ref = W.has_ref || (it.T > 0 && it.q_ref);
-        W.host_out = W.host_out || (it.T > 0 && (!W.dev_q[i] || !W.dev_e[i] || !W.dev_c[i]));
-        if (it.T > 0 && !W.dev_tgt[i]) {
+        const bool some = it.T > 0;
+        W.at_tgt[i] = some ? pointer_reach(it.targets, ctx->device) : 0;
+        W.at_q[i] = some ? pointer_reach(it.out_q, ctx->device) : 0;
+        W.at_e[i] = some ? pointer_reach(it.out_err, ctx->device) : 0;
+        W.at_c[i] = some ? pointer_reach(it.out_count, ctx->device) : 0;
+        W.at_ref[i] = some && it.q_ref ? pointer_reach(it.q_ref, ctx->device) : 0;
+        W.has_ref = W.has_ref || (some && it.q_ref);
+        W.host_out = W.host_out || (some && (W.at_q[i] == 0 || W.at_e[i] == 0 || W.at_c[i] == 0));
+        if (some && W.at_tgt[i] == 0) {
             for (int t = 0; t < it.T; ++t) {
                 const float* q = it.targets + 7 * (size_t)t + 3;
                 const float nn = q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + q[3] * q[3];
@@ -130,11 +132,17 @@ hjcd_status plan_wave(hjcd_ctx* ctx, const WaveItem* items, int n_items, const h
     W.o_tg = cv.take<TargetDesc>(W.T);
     W.o_moff = cv.take<int64_t>((size_t)W.T + 1);
     W.o_boff = cv.take<int64_t>((size_t)W.T + 1);
-    W.o_qe = cv.take<int64_t>(2 * (size_t)W.T);
-    W.o_pq7 = cv.take<float>(7 * (size_t)W.T);
-    W.o_ref = cv.take<float>(W.has_ref ? (size_t)W.T * W.n_max : 0);
+    W.o_io = cv.take<TargetIo>(W.T);
     W.o_inl = cv.take<char>(inl_bytes);
     W.head = cv.off;
+    bool copy_tgt = false, copy_ref = false;  // poses or references of another device
+    for (int i = 0; i < n_items; ++i) {
+        copy_tgt = copy_tgt || W.at_tgt[i] == 1;
+        copy_ref = copy_ref || W.at_ref[i] == 1;
+    }
+    W.o_pose = cv.take<float>(copy_tgt ? 7 * (size_t)W.T : 0);
+    W.o_pref = cv.take<float>(copy_ref ? (size_t)W.T * W.n_max : 0);
+    W.o_ref = cv.take<float>(W.has_ref ? (size_t)W.T * W.n_max : 0);
     W.o_thM = cv.take<float>((size_t)W.n_max * W.CM);
     W.o_thM2 = cv.take<float>(P.cd_variant == 2 ? (size_t)W.n_max * W.CM : 0);  // lock-step PO-CCD's second buffer
     W.o_sM = cv.take<float>(W.CM);
@@ -148,25 +156,47 @@ hjcd_status plan_wave(hjcd_ctx* ctx, const WaveItem* items, int n_items, const h
     W.o_c = cv.take<int32_t>(W.T);
     W.o_ul = cv.take<int32_t>(W.T);           // targets left to the second collision pass
     W.o_sg = cv.take<int32_t>(2 * (size_t)W.CM);  // PO-CCD candidates handed between segments
-    // queue head, error flag, count of o_ul, counts of o_sg; the PO-CCD segments' queue heads
+    // queue head, (unused), count of o_ul, counts of o_sg; the PO-CCD segments' queue heads
     W.o_qf = cv.take<unsigned long long>(6);
     W.bytes = cv.off;
+
+    Carve pv;
+    pv.off = W.head;
+    W.p_pose = pv.take<float>(7 * (size_t)W.T);
+    W.p_ref = pv.take<float>(W.has_ref ? (size_t)W.T * W.n_max : 0);
+    W.staged = W.host_out && 4 * (size_t)(W.q_total + W.e_total + W.T) <= kStagedResults;
+    W.p_q = pv.take<float>(W.staged ? W.q_total : 0);
+    W.p_e = pv.take<float>(W.staged ? W.e_total : 0);
+    W.p_c = pv.take<int32_t>(W.staged ? W.T : 0);
+    W.pin_bytes = kFlagBytes + pv.off;
     return HJCD_OK;
 }
 
+void take_results(const WavePlan& W, int i, const WaveItem& it, const char* pin) {
+    if (it.T == 0) return;
+    pin += kFlagBytes;
+    const size_t nq = (size_t)it.T * it.top_k * it.rob->P.n, ne = (size_t)it.T * it.top_k * 2;
+    if (W.at_q[i] == 0) std::memcpy(it.out_q, pin + W.p_q + 4 * W.item_q0[i], sizeof(float) * nq);
+    if (W.at_e[i] == 0) std::memcpy(it.out_err, pin + W.p_e + 4 * W.item_e0[i], sizeof(float) * ne);
+    if (W.at_c[i] == 0) std::memcpy(it.out_count, pin + W.p_c + 4 * (size_t)W.item_t0[i], sizeof(int32_t) * (size_t)it.T);
+}
+
 hjcd_status run_wave(hjcd_ctx* ctx, const WavePlan& W, const WaveItem* items, const hjcd_params& P, char* ws,
-                     char* pin, cudaStream_t s, cudaEvent_t* ev) {
+                     char* pin, cudaStream_t s, cudaEvent_t* ev, cudaEvent_t read) {
     if (W.T == 0) return HJCD_OK;
     hjcd_status st;
     // ---- pinned image of the head ----
+    int32_t* const flag = wave_flag(pin);
+    pin += kFlagBytes;
     RobotParams* h_rp = reinterpret_cast<RobotParams*>(pin + W.o_rp);
     RobotDev* h_rd = reinterpret_cast<RobotDev*>(pin + W.o_rd);
     SceneDev* h_sd = reinterpret_cast<SceneDev*>(pin + W.o_sd);
     TargetDesc* h_tg = reinterpret_cast<TargetDesc*>(pin + W.o_tg);
     int64_t* h_moff = reinterpret_cast<int64_t*>(pin + W.o_moff);
     int64_t* h_boff = reinterpret_cast<int64_t*>(pin + W.o_boff);
-    int64_t* h_qe = reinterpret_cast<int64_t*>(pin + W.o_qe);
-    float* h_pq7 = reinterpret_cast<float*>(pin + W.o_pq7);
+    TargetIo* h_io = reinterpret_cast<TargetIo*>(pin + W.o_io);
+    float* h_pose = reinterpret_cast<float*>(pin + W.p_pose);
+    float* h_ref = reinterpret_cast<float*>(pin + W.p_ref);
     for (int r = 0; r < W.NR; ++r) {
         h_rp[r] = W.robots[r]->P;
         h_rd[r] = W.robots[r]->dev;
@@ -194,6 +224,23 @@ hjcd_status run_wave(hjcd_ctx* ctx, const WavePlan& W, const WaveItem* items, co
         const int n = it.rob->P.n;
         const int cd = it.cd_iters >= 0 ? it.cd_iters : P.cd_max_iters;
         const int lm = it.lm_iters >= 0 ? it.lm_iters : P.lm_max_iters;
+        // the item's poses and references where the first launch finds them, its results where the last
+        // one puts them: in place, or beside the image (host, small), or in the workspace
+        const size_t t0 = W.item_t0[i], nq = (size_t)it.top_k * n;
+        const float* pose = W.at_tgt[i] == 2 ? it.targets
+                            : W.at_tgt[i] == 1 ? reinterpret_cast<const float*>(ws + W.o_pose) + 7 * t0 : h_pose + 7 * t0;
+        const float* ref = !it.q_ref ? nullptr
+                           : W.at_ref[i] == 2 ? it.q_ref
+                           : W.at_ref[i] == 1 ? reinterpret_cast<const float*>(ws + W.o_pref) + t0 * W.n_max
+                                              : h_ref + t0 * W.n_max;
+        auto block = [&](int at, auto* user, size_t p_off, size_t o_off, size_t first) {
+            using E = std::remove_reference_t<decltype(*user)>;
+            if (at == 2) return user;
+            return reinterpret_cast<E*>(at == 0 && W.staged ? pin + p_off : ws + o_off) + first;
+        };
+        float* oq = it.T ? block(W.at_q[i], it.out_q, W.p_q, W.o_q, W.item_q0[i]) : nullptr;
+        float* oe = it.T ? block(W.at_e[i], it.out_err, W.p_e, W.o_e, W.item_e0[i]) : nullptr;
+        int32_t* oc = it.T ? block(W.at_c[i], it.out_count, W.p_c, W.o_c, t0) : nullptr;
         for (int t = 0; t < it.T; ++t) {
             const int g = W.item_t0[i] + t;
             TargetDesc d{};
@@ -211,36 +258,25 @@ hjcd_status run_wave(hjcd_ctx* ctx, const WavePlan& W, const WaveItem* items, co
             const int m = it.spt ? it.spt[t] : it.n_samples;
             h_moff[g + 1] = h_moff[g] + m;
             h_boff[g + 1] = h_boff[g] + dup_count(m, P.dup_ratio);
-            h_qe[2 * g] = W.item_q0[i] + (int64_t)t * it.top_k * n;
-            h_qe[2 * g + 1] = W.item_e0[i] + (int64_t)t * it.top_k * 2;
+            h_io[g] = TargetIo{pose + 7 * (size_t)t, ref ? ref + (size_t)t * n : nullptr, oq + t * nq,
+                               oe + (size_t)t * it.top_k * 2, oc + t};
         }
-        if (!W.dev_tgt[i] && it.T > 0)
-            std::memcpy(h_pq7 + 7 * (size_t)W.item_t0[i], it.targets, sizeof(float) * 7 * (size_t)it.T);
-        if (W.has_ref && it.T > 0) {
-            // reference rows at stride n_max (rows of requests without references are not read)
-            float* h_ref = reinterpret_cast<float*>(pin + W.o_ref) + (size_t)W.item_t0[i] * W.n_max;
-            for (int t = 0; t < it.T; ++t)
-                for (int j = 0; j < W.n_max; ++j)
-                    h_ref[(size_t)t * W.n_max + j] =
-                        (it.q_ref && !W.dev_ref[i] && j < n) ? it.q_ref[(size_t)t * n + j] : 0.0f;
-        }
+        if (W.at_tgt[i] == 0 && it.T > 0)
+            std::memcpy(h_pose + 7 * t0, it.targets, sizeof(float) * 7 * (size_t)it.T);
+        if (W.at_ref[i] == 0 && it.q_ref && it.T > 0)
+            std::memcpy(h_ref + t0 * W.n_max, it.q_ref, sizeof(float) * (size_t)it.T * n);
     }
 
-    // ---- host -> device ----
-    HJCD_CUDA(ctx, cudaMemcpyAsync(ws, pin, W.head, cudaMemcpyHostToDevice, s));
-    for (int i = 0; i < W.n_items; ++i)
-        if (W.dev_tgt[i] && items[i].T > 0)
-            HJCD_CUDA(ctx, cudaMemcpyAsync(ws + W.o_pq7 + sizeof(float) * 7 * (size_t)W.item_t0[i], items[i].targets,
-                                           sizeof(float) * 7 * (size_t)items[i].T, cudaMemcpyDeviceToDevice, s));
-    for (int i = 0; i < W.n_items; ++i)
-        if (W.dev_ref[i])
-            HJCD_CUDA(ctx, cudaMemcpy2DAsync(ws + W.o_ref + sizeof(float) * (size_t)W.item_t0[i] * W.n_max,
-                                             sizeof(float) * W.n_max, items[i].q_ref,
-                                             sizeof(float) * items[i].rob->P.n, sizeof(float) * items[i].rob->P.n,
-                                             (size_t)items[i].T, cudaMemcpyDeviceToDevice, s));
-    HJCD_CUDA(ctx, cudaMemsetAsync(ws + W.o_qf, 0, 48, s));
-    HJCD_CUDA(ctx, cudaMemsetAsync(ws + W.o_q, 0xff, sizeof(float) * (size_t)W.q_total, s));  // unfilled rows: NaN
-    HJCD_CUDA(ctx, cudaMemsetAsync(ws + W.o_e, 0xff, sizeof(float) * (size_t)W.e_total, s));
+    // ---- what lies in another device's memory ----
+    for (int i = 0; i < W.n_items; ++i) {
+        const WaveItem& it = items[i];
+        if (W.at_tgt[i] == 1)
+            HJCD_CUDA(ctx, cudaMemcpyAsync(ws + W.o_pose + sizeof(float) * 7 * (size_t)W.item_t0[i], it.targets,
+                                           sizeof(float) * 7 * (size_t)it.T, cudaMemcpyDeviceToDevice, s));
+        if (W.at_ref[i] == 1)
+            HJCD_CUDA(ctx, cudaMemcpyAsync(ws + W.o_pref + sizeof(float) * (size_t)W.item_t0[i] * W.n_max, it.q_ref,
+                                           sizeof(float) * (size_t)it.T * it.rob->P.n, cudaMemcpyDeviceToDevice, s));
+    }
 
     TargetDesc* d_tg = reinterpret_cast<TargetDesc*>(ws + W.o_tg);
     const int64_t* d_moff = reinterpret_cast<const int64_t*>(ws + W.o_moff);
@@ -259,8 +295,12 @@ hjcd_status run_wave(hjcd_ctx* ctx, const WavePlan& W, const WaveItem* items, co
     for (int r = 0; r < W.NR; ++r) rs.plain &= W.robots[r]->P.plain;
 
     if (ev) HJCD_CUDA(ctx, cudaEventRecord(ev[0], s));
-    launch_pack_targets(reinterpret_cast<const float*>(ws + W.o_pq7), W.T, d_tg, TargetDesc{}, d_tg, s);
-    if ((st = after_launch(ctx, 1, "k_pack_targets"))) return st;
+    launch_wave_init(WaveInitArgs{pin, ws, W.head, W.o_tg, W.o_io, W.o_rp, W.T,
+                                  W.has_ref ? reinterpret_cast<float*>(ws + W.o_ref) : nullptr, W.n_max, queue,
+                                  flag},
+                     s);
+    if ((st = after_launch(ctx, 1, "k_wave_init"))) return st;
+    if (read) HJCD_CUDA(ctx, cudaEventRecord(read, s));
 
     // Alg. 2: PO-CCD from uniform seeds
     CcdArgs ca{};
@@ -340,11 +380,8 @@ hjcd_status run_wave(hjcd_ctx* ctx, const WavePlan& W, const WaveItem* items, co
 
     // collision filter and ranking
     const bool collide = W.ns_max > 0;
-    float* q_out = reinterpret_cast<float*>(ws + W.o_q);
-    float* e_out = reinterpret_cast<float*>(ws + W.o_e);
-    int32_t* c_out = reinterpret_cast<int32_t*>(ws + W.o_c);
     RankArgs ra{rs, d_tg, W.T, d_boff, thB, W.CB, sB, pB, oB, collide ? hB : nullptr, 0,
-                reinterpret_cast<const int64_t*>(ws + W.o_qe), q_out, e_out, c_out,
+                reinterpret_cast<const TargetIo*>(ws + W.o_io), nullptr, nullptr, nullptr,
                 W.has_ref ? reinterpret_cast<const float*>(ws + W.o_ref) : nullptr, W.n_max};
     CollideArgs cl{};
     if (collide) {
@@ -369,7 +406,7 @@ hjcd_status run_wave(hjcd_ctx* ctx, const WavePlan& W, const WaveItem* items, co
         cl.th = thB;
         cl.hit = hB;
         cl.cnt = ctx->cnt;
-        cl.err_flag = wave_flag(W, ws);
+        cl.err_flag = flag;
         cl.first_wait_polls = ctx->first_wait_polls.load();
     }
     // the top_k collision-free candidates by score are the first top_k collision-free ones in score
@@ -409,17 +446,19 @@ hjcd_status run_wave(hjcd_ctx* ctx, const WavePlan& W, const WaveItem* items, co
     }
     if (ev) HJCD_CUDA(ctx, cudaEventRecord(ev[5], s));
 
-    // each request's results to its own buffers
+    // results that the kernels left in the workspace
     for (int i = 0; i < W.n_items; ++i) {
         const WaveItem& it = items[i];
         if (it.T == 0) continue;
+        auto out = [&](int at, void* user, const char* from, size_t bytes) -> hjcd_status {
+            if (at == 2 || (at == 0 && W.staged)) return HJCD_OK;
+            HJCD_CUDA(ctx, cudaMemcpyAsync(user, from, bytes, at ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
+            return HJCD_OK;
+        };
         const size_t nq = (size_t)it.T * it.top_k * it.rob->P.n, ne = (size_t)it.T * it.top_k * 2;
-        HJCD_CUDA(ctx, cudaMemcpyAsync(it.out_q, q_out + W.item_q0[i], sizeof(float) * nq,
-                                       W.dev_q[i] ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
-        HJCD_CUDA(ctx, cudaMemcpyAsync(it.out_err, e_out + W.item_e0[i], sizeof(float) * ne,
-                                       W.dev_e[i] ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
-        HJCD_CUDA(ctx, cudaMemcpyAsync(it.out_count, c_out + W.item_t0[i], sizeof(int32_t) * (size_t)it.T,
-                                       W.dev_c[i] ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
+        if ((st = out(W.at_q[i], it.out_q, ws + W.o_q + 4 * W.item_q0[i], sizeof(float) * nq))) return st;
+        if ((st = out(W.at_e[i], it.out_err, ws + W.o_e + 4 * W.item_e0[i], sizeof(float) * ne))) return st;
+        if ((st = out(W.at_c[i], it.out_count, ws + W.o_c + 4 * (size_t)W.item_t0[i], sizeof(int32_t) * (size_t)it.T))) return st;
     }
     return HJCD_OK;
 }

@@ -131,3 +131,31 @@ def test_fk_does_not_depend_on_the_batch(ctx, which):
         torch.cuda.synchronize()
         assert torch.equal(buf[1:1 + 7 * C].view(C, 7), alone[:C])
         assert buf[0] == -7.0 and bool((buf[1 + 7 * C:] == -7.0).all())
+
+
+@pytest.mark.parametrize("T,top_k", [(1, 1), (7, 3), (2000, 64)])
+def test_results_do_not_depend_on_where_the_buffers_live(ctx, T, top_k):
+    """Poses, references and outputs in device or host memory in any mix: small host results come
+    through the library's pinned buffer, larger ones (2000 x 64 rows) by copies."""
+    rob = _robot("chain7")
+    rid = ctx.add_robot(rob)
+    rng = np.random.default_rng(6)
+    th = torch.as_tensor(inputs.joint_samples(rng, rob, T).T.copy(), dtype=torch.float32, device="cuda")
+    tg = ctx.fk(rid, th)
+    qc = torch.as_tensor(inputs.joint_samples(rng, rob, T), dtype=torch.float32, device="cuda")
+    tg_h, qc_h = tg.cpu(), qc.cpu()
+    shapes = ((T, top_k, 7), (T, top_k, 2), (T,))
+    ref = None
+    for mask in (0, 7, 1, 2, 4, 5):
+        out = [torch.full(sh, -1, dtype=torch.int32 if k == 2 else torch.float32, device="cpu" if mask >> k & 1 else "cuda")
+               for k, sh in enumerate(shapes)]
+        src, cur = (tg_h, qc) if mask & 1 else (tg, qc_h)
+        ctx.solve(rid, -1, src, 40, top_k, 9, 7, out=out, q_current=cur)
+        torch.cuda.synchronize()
+        got = [o.cpu().numpy().view(np.uint32) for o in out]
+        if ref is None:
+            ref = got
+            assert (out[2] == min(top_k, 40)).all()
+            assert torch.isnan(out[0][:, 40:]).all() and torch.isnan(out[1][:, 40:]).all()
+        for a, b in zip(got, ref):
+            np.testing.assert_array_equal(a, b)
