@@ -128,40 +128,27 @@ __device__ __forceinline__ float2 quat_angle2(float2 w, float2 vv) {
 // (cos, sin of x/2).  The only differences are those that form the residual's own components, as
 // in the direct evaluation, and the squares are summed, so the closed form is as accurate (a float32
 // emulation against the float64 method agrees to 2e-7 on Panda).
-// The position step needs the end effector only: it and the joint's geometry come first
-// (CcdGeom), so that a caller can let them overlap the error quaternion's chain.
-struct CcdGeom {
-    float nup2, nvp2, nu2, ez, cs, sn, d;
-};
-__device__ __forceinline__ CcdGeom ccd_joint_geom(const V3 pj, const V3 z, const V3 Ep, const V3 pt, float pe2) {
-    CcdGeom g;
+__device__ __forceinline__ CcdTrials ccd_joint_trials(const V3 pj, const V3 z, float thj, float lo, float hi,
+                                                      const V3 Ep, const V3 pt, const Q4 qerr, float nqw,
+                                                      float dphi, float pe2, float inv_p2, float inv_o2) {
+    CcdTrials o;
     const V3 u = Ep - pj;
     const V3 v = pt - pj;
     const float uz = dot(u, z), vz = dot(v, z);
     const V3 up = fma3(-uz, z, u);
     const V3 vp = fma3(-vz, z, v);
-    g.nup2 = dot(up, up);
-    g.nvp2 = dot(vp, vp);
-    g.nu2 = fmaf(uz, uz, g.nup2);
-    const float nv2 = fmaf(vz, vz, g.nvp2);
+    const float nup2 = dot(up, up), nvp2 = dot(vp, vp);
+    const float nu2 = fmaf(uz, uz, nup2), nv2 = fmaf(vz, vz, nvp2);
     const V3 zxu = cross(z, up);
-    g.ez = vz - uz;
-
-    // Eq. theta_proj, signed about the axis: atan2(z.(up x vp), up.vp) = atan2(zxu.vp, up.vp)
-    g.cs = dot(up, vp);
-    g.sn = dot(zxu, vp);
-    const bool deg = g.nu2 < 1e-24f || nv2 < 1e-24f || g.nup2 <= pe2 * g.nu2 || g.nvp2 <= pe2 * nv2;
-    g.d = deg ? 0.0f : atan2_all(g.sn, g.cs);
-    return g;
-}
-
-__device__ __forceinline__ CcdTrials ccd_joint_trials(const CcdGeom& g, const V3 z, float thj, float lo, float hi,
-                                                      const Q4 qerr, float nqw, float dphi, float inv_p2, float inv_o2) {
-    CcdTrials o;
-    const float nup2 = g.nup2, nvp2 = g.nvp2, nu2 = g.nu2, ez = g.ez, cs = g.cs, sn = g.sn, d = g.d;
+    const float ez = vz - uz;
     const float az = dot(qerr.v, z);
     const V3 qp = fma3(-az, z, qerr.v);
     const float qp2 = dot(qp, qp);
+
+    // Eq. theta_proj, signed about the axis: atan2(z.(up x vp), up.vp) = atan2(zxu.vp, up.vp)
+    const float cs = dot(up, vp), sn = dot(zxu, vp);
+    const bool deg = nu2 < 1e-24f || nv2 < 1e-24f || nup2 <= pe2 * nu2 || nvp2 <= pe2 * nv2;
+    const float d = deg ? 0.0f : atan2_all(sn, cs);
     // Eq. ori_update: delta(k) sgn(a.z) phi
     const float dq = (az > 0.0f) ? dphi : ((az < 0.0f) ? -dphi : 0.0f);
 
@@ -204,32 +191,6 @@ __device__ __forceinline__ CcdTrials ccd_joint_trials(const CcdGeom& g, const V3
     o.rq = ang.y;
     o.so = sc.y;
     return o;
-}
-
-// Acceptance of theta_hat (reading: an improvement above gamma in position or in orientation):
-// its residual is the end effector at Ep and the error quaternion turned by da about the distal
-// chosen joint (origin Pa, axis Za) first, then by db about the proximal one; ep0 and eo are the
-// current errors.
-__device__ __forceinline__ bool ccd_accept_pos(float gamma, const V3 Ep, const V3 pt, float ep0, const V3 Pa, const V3 Za,
-                                               float da, const V3 Pb, const V3 Zb, float db) {
-    float sa_, ca_, sb_, cb_;
-    __sincosf(0.5f * da, &sa_, &ca_);
-    __sincosf(0.5f * db, &sb_, &cb_);
-    V3 x = Pa + rotate_half(Za, sa_, ca_, Ep - Pa);
-    x = Pb + rotate_half(Zb, sb_, cb_, x - Pb);
-    const V3 e1 = pt - x;
-    const float ep1 = sqrt_approx(dot(e1, e1));
-    return ep0 - ep1 > gamma;
-}
-__device__ __forceinline__ bool ccd_accept_ori(float gamma, const Q4 qerr, float eo, const V3 Za, float da, const V3 Zb,
-                                               float db) {
-    float sa_, ca_, sb_, cb_;
-    __sincosf(0.5f * da, &sa_, &ca_);
-    __sincosf(0.5f * db, &sb_, &cb_);
-    Q4 q1 = qmul(qerr, Q4{ca_, (-sa_) * Za});
-    q1 = qmul(q1, Q4{cb_, (-sb_) * Zb});
-    const float eo1 = quat_angle(q1.w, dot(q1.v, q1.v));
-    return eo - eo1 > gamma;
 }
 
 // One iteration of a candidate: kinematics with frames into the column, the
@@ -308,8 +269,8 @@ __device__ __forceinline__ int ccd_step(const RobotParams* rob, const RobotParam
         const float2 pa = col.a(j), pb = col.b(j), za = col.c(j);
         const V3 pj = v3(pa.x, pa.y, pb.x);
         const V3 z = v3(za.x, za.y, col.zz(j));
-        const CcdTrials tr = ccd_joint_trials(ccd_joint_geom(pj, z, E.p, pt, pe2), z, pb.y, R.lim[j].x, R.lim[j].y, qerr,
-                                              nqw, dphi, inv_p2, inv_o2);
+        const CcdTrials tr =
+            ccd_joint_trials(pj, z, pb.y, R.lim[j].x, R.lim[j].y, E.p, pt, qerr, nqw, dphi, pe2, inv_p2, inv_o2);
         if (tr.sp < best_p * one_m_tie) {  // joint 0 against +inf
             best_p = tr.sp;
             jp = j;
@@ -343,9 +304,18 @@ __device__ __forceinline__ int ccd_step(const RobotParams* rob, const RobotParam
     col.frame(p_hi ? jp : jo, Pa, Za);  // the distal joint
     col.frame(p_hi ? jo : jp, Pb, Zb);
     const float da = p_hi ? aP : aO, db = p_hi ? aO : aP;
-    const bool acc_p = ccd_accept_pos(P.cd_gamma_pos, E.p, pt, ep0, Pa, Za, da, Pb, Zb, db);
-    const bool acc_o = ccd_accept_ori(P.cd_gamma_ori, qerr, eo, Za, da, Zb, db);
-    const bool acc = acc_p || acc_o;
+    float sa_, ca_, sb_, cb_;
+    __sincosf(0.5f * da, &sa_, &ca_);
+    __sincosf(0.5f * db, &sb_, &cb_);
+    V3 x = Pa + rotate_half(Za, sa_, ca_, E.p - Pa);
+    x = Pb + rotate_half(Zb, sb_, cb_, x - Pb);
+    Q4 q1 = qmul(qerr, Q4{ca_, (-sa_) * Za});
+    q1 = qmul(q1, Q4{cb_, (-sb_) * Zb});
+    const V3 e1 = pt - x;
+    const float ep1 = sqrt_approx(dot(e1, e1));
+    const float eo1 = quat_angle(q1.w, dot(q1.v, q1.v));
+    // acceptance (reading: an improvement above gamma in position or in orientation)
+    const bool acc = (ep0 - ep1 > P.cd_gamma_pos) || (eo - eo1 > P.cd_gamma_ori);
 
     if (TRACE && kk == 0) {
         if (A.tr.jp) A.tr.jp[c] = jp;
@@ -598,9 +568,7 @@ __device__ __forceinline__ void coop_fk_row(const CoopCol& C, const RobotParams&
     float c0 = row == 0 ? 1.0f : 0.0f, c1 = row == 1 ? 1.0f : 0.0f, c2 = row == 2 ? 1.0f : 0.0f, p = 0.0f;
     float2* const fr = C.fr + row * C.nl * kCoopCands + l;
     const float2* const csl = C.cs + l;
-    auto step = [&](int j) {
-        const float4 g = R.dh[j];
-        const float2 cs = csl[j * kCoopCands];
+    auto step = [&](int j, const float4 g, const float2 cs) {
         const float b1 = fmaf(g.x, c1, g.y * c2);
         const float b2 = fmaf(g.x, c2, (-g.y) * c1);
         p = fmaf(g.w, b2, fmaf(g.z, c0, p));
@@ -610,14 +578,46 @@ __device__ __forceinline__ void coop_fk_row(const CoopCol& C, const RobotParams&
         c2 = b2;
         fr[j * kCoopCands] = make_float2(p, c2);
     };
-    if (N) {
+    if (N) {  // all loads come before the stores, which the compiler may not move them across
+        float4 g[N ? N : 1];
+        float2 cs[N ? N : 1];
 #pragma unroll
-        for (int j = 0; j < N; ++j) step(j);
+        for (int j = 0; j < N; ++j) {
+            g[j] = R.dh[j];
+            cs[j] = csl[j * kCoopCands];
+        }
+#pragma unroll
+        for (int j = 0; j < N; ++j) step(j, g[j], cs[j]);
     } else {
 #pragma unroll 4
-        for (int j = 0; j < n; ++j) step(j);
+        for (int j = 0; j < n; ++j) step(j, R.dh[j], csl[j * kCoopCands]);
     }
     C.e[row * kCoopCands + l] = make_float2(c0, c1);
+}
+
+// The part of ccd_joint_trials that needs the end effector only: a joint's geometry and its position
+// step, which here come before the error quaternion is known
+struct CcdGeom {
+    float nup2, nvp2, nu2, ez, cs, sn, d;
+};
+__device__ __forceinline__ CcdGeom ccd_joint_geom(const V3 pj, const V3 z, const V3 Ep, const V3 pt, float pe2) {
+    CcdGeom g;
+    const V3 u = Ep - pj;
+    const V3 v = pt - pj;
+    const float uz = dot(u, z), vz = dot(v, z);
+    const V3 up = fma3(-uz, z, u);
+    const V3 vp = fma3(-vz, z, v);
+    g.nup2 = dot(up, up);
+    g.nvp2 = dot(vp, vp);
+    g.nu2 = fmaf(uz, uz, g.nup2);
+    const float nv2 = fmaf(vz, vz, g.nvp2);
+    const V3 zxu = cross(z, up);
+    g.ez = vz - uz;
+    g.cs = dot(up, vp);
+    g.sn = dot(zxu, vp);
+    const bool deg = g.nu2 < 1e-24f || nv2 < 1e-24f || g.nup2 <= pe2 * g.nu2 || g.nvp2 <= pe2 * nv2;
+    g.d = deg ? 0.0f : atan2_all(g.sn, g.cs);
+    return g;
 }
 
 // One trial of a joint: ccd_joint_trials' operations on one half of its pairs, for the step x
@@ -650,6 +650,32 @@ __device__ __forceinline__ float2 ccd_joint_trial(const CcdGeom& g, float az, fl
     p = fmaf(p, s, 9.999994549e-01f);
     const float ang = ay > ax ? fmaf(__fmul_rn(-2.0f, t), p, 2.0f * 1.57079632679489662f) : __fmul_rn(__fmul_rn(2.0f, t), p);
     return make_float2(fmaf(r2, inv_p2, __fmul_rn(__fmul_rn(ang, ang), inv_o2)), st);
+}
+
+// ccd_step's acceptance of theta_hat by the position and by the orientation:
+// its residual is the end effector at Ep and the error quaternion turned by da about the distal
+// chosen joint (origin Pa, axis Za) first, then by db about the proximal one; ep0 and eo are the
+// current errors.
+__device__ __forceinline__ bool ccd_accept_pos(float gamma, const V3 Ep, const V3 pt, float ep0, const V3 Pa, const V3 Za,
+                                               float da, const V3 Pb, const V3 Zb, float db) {
+    float sa_, ca_, sb_, cb_;
+    __sincosf(0.5f * da, &sa_, &ca_);
+    __sincosf(0.5f * db, &sb_, &cb_);
+    V3 x = Pa + rotate_half(Za, sa_, ca_, Ep - Pa);
+    x = Pb + rotate_half(Zb, sb_, cb_, x - Pb);
+    const V3 e1 = pt - x;
+    const float ep1 = sqrt_approx(dot(e1, e1));
+    return ep0 - ep1 > gamma;
+}
+__device__ __forceinline__ bool ccd_accept_ori(float gamma, const Q4 qerr, float eo, const V3 Za, float da, const V3 Zb,
+                                               float db) {
+    float sa_, ca_, sb_, cb_;
+    __sincosf(0.5f * da, &sa_, &ca_);
+    __sincosf(0.5f * db, &sb_, &cb_);
+    Q4 q1 = qmul(qerr, Q4{ca_, (-sa_) * Za});
+    q1 = qmul(q1, Q4{cb_, (-sb_) * Zb});
+    const float eo1 = quat_angle(q1.w, dot(q1.v, q1.v));
+    return eo - eo1 > gamma;
 }
 
 // RED as for k_ccd; N > 0: the launch's one robot has N joints (unrolled loops); N = 0: any robots
