@@ -691,6 +691,16 @@ struct LmArgs {
     unsigned long long* queue;  // candidate queue head, zero at launch
     int32_t warps;  // warps per CTA: 2, 4 or 8 (anything else: 8, the contexts' default)
     int32_t in_limits;  // 1: every joint vector the launch reads lies within its robot's limits
+    // Where a launch leaves the candidates that need more than its first iterations to the next one
+    // (null: nowhere): their indices and iteration counts [C] and how many there are (zero at launch).
+    // hand_at (set by launch_lm; 0: never): the iteration after which it does.
+    int32_t* list;
+    int32_t* list_k;
+    int32_t* n_list;
+    unsigned long long* queue2;  // the queue head of a launch over the list, zero
+    int32_t hand_at;
+    int32_t list_in;  // set by launch_lm; 1: the launch runs the list's candidates, when there are more than list_lim
+    int32_t list_lim;
 };
 
 struct DupArgs {
@@ -880,7 +890,7 @@ struct WaveInitArgs {
     int32_t T;
     float* ref;       // [T][ld_ref], or null
     int32_t ld_ref;
-    unsigned long long* zero;  // 6 words
+    unsigned long long* zero;  // 7 words
     int32_t* flag;
 };
 void launch_wave_init(const WaveInitArgs& A, cudaStream_t st);
@@ -890,7 +900,7 @@ void launch_fk(const RobotParams& R, int64_t C, const float* th, int64_t ld, flo
 void launch_sample(const RobotParams& R, uint64_t seed, CandMap map, int64_t C, float* th, int64_t ld,
                    cudaStream_t st);
 void launch_ccd(const CcdArgs& A, bool trace, cudaStream_t st);
-void launch_lm(const LmArgs& A, bool trace, cudaStream_t st);
+int launch_lm(const LmArgs& A, bool trace, cudaStream_t st);  // the number of launches
 void launch_topk_dup(const DupArgs& A, int max_m, cudaStream_t st);
 void launch_rank(const RankArgs& A, int max_b, cudaStream_t st);
 void launch_collide(const CollideArgs& A, cudaStream_t st);

@@ -227,13 +227,15 @@ struct LmCta {
     int* fl;
     int* pl;
     int* np;
+    int* drained;  // some lane found the queue empty
 };
 template <int WARPS>
-__host__ __device__ constexpr int lm_cta_words() { return WARPS + 2 * WARPS * 32 + 1; }
+__host__ __device__ constexpr int lm_cta_words() { return WARPS + 2 * WARPS * 32 + 2; }
 template <int WARPS>
 __device__ __forceinline__ LmCta<WARPS> lm_cta(float* f) {
     int* b = reinterpret_cast<int*>(f);
-    return LmCta<WARPS>{reinterpret_cast<unsigned*>(b), b + WARPS, b + WARPS + WARPS * 32, b + WARPS + 2 * WARPS * 32};
+    return LmCta<WARPS>{reinterpret_cast<unsigned*>(b), b + WARPS, b + WARPS + WARPS * 32, b + WARPS + 2 * WARPS * 32,
+                        b + WARPS + 2 * WARPS * 32 + 1};
 }
 
 // 1/2 |W r|^2 of a residual r = (e, om)
@@ -436,7 +438,8 @@ __device__ __noinline__ void dogleg_prepare(const LmW S, int l, int n, float Rt,
 
 // RED = false: the launch's joint vectors lie within the limits of plain robots (no offsets and
 // no range reduction in the kinematics steps; the same bits)
-template <bool TRACE, int WARPS, bool RED>
+// HAND: the launch leaves candidates to a later one (hand_at) or runs those that were left (list_in)
+template <bool TRACE, int WARPS, bool RED, bool HAND>
 __global__ void __launch_bounds__(WARPS * 32, 16 / WARPS) k_lm(const LmArgs A) {
     extern __shared__ __align__(16) float smem_f[];
     __shared__ float alphas[kMaxLsDepth + 1];
@@ -449,13 +452,21 @@ __global__ void __launch_bounds__(WARPS * 32, 16 / WARPS) k_lm(const LmArgs A) {
     // the state of slot sl = warp * 32 + lane, whichever thread works on it
     auto slot_state = [&](int sl) { return LmW{warps_f + (sl >> 5) * words, A.rs.n_max}; };
     const LmCta<WARPS> CL = lm_cta<WARPS>(warps_f + WARPS * words);
+    if (HAND) {
+        if (threadIdx.x == 0) CL.drained[0] = 0;
+        __syncthreads();
+    }
 
     const hjcd_params& P = A.P;
     const float Rt = P.lm_trust_R;
     unsigned long long n_it = 0, n_fk = 0, n_sc = 0;
 
+    const bool list = HAND && A.list_in;
+    const int64_t items = list ? (int64_t)*A.n_list : A.C;
+    if (list && items <= A.list_lim) return;  // few: the spread kernel's
     bool has = false;
-    int64_t c = 0;
+    int rounds = 0;
+    int64_t qi = 0, c = 0;  // place in the queue, candidate
     int32_t t = 0, s = 0, kk = 0, cap = 0;
     TargetDesc T{};
 
@@ -465,13 +476,14 @@ __global__ void __launch_bounds__(WARPS * 32, 16 / WARPS) k_lm(const LmArgs A) {
         if (need) {
             const int leader = __ffs(need) - 1;
             long long base = 0;
-            if (lane == leader) base = (long long)atomicAdd(A.queue, (unsigned long long)__popc(need));
+            if (lane == leader) base = (long long)atomicAdd(list ? A.queue2 : A.queue, (unsigned long long)__popc(need));
             base = __shfl_sync(0xffffffffu, base, leader);
             if (!has) {
-                c = base + __popc(need & ((1u << lane) - 1u));
-                if (c < A.C && A.map.lookup(c, t, s)) {
+                qi = base + __popc(need & ((1u << lane) - 1u));
+                c = list && qi < items ? (int64_t)A.list[qi] : qi;
+                if (qi < items && A.map.lookup(c, t, s)) {
                     T = A.tg[t];
-                    kk = 0;
+                    kk = list ? A.list_k[qi] : 0;
                     cap = A.n_iters >= 0 ? A.n_iters : T.lm_iters;
                     if (T.eps_pos > 0.0f) {
                         has = true;
@@ -604,11 +616,13 @@ __global__ void __launch_bounds__(WARPS * 32, 16 / WARPS) k_lm(const LmArgs A) {
         }
 
         // ---- the failure path over the CTA: the failing slots of all warps, compacted ----
-        // (the same barrier ends the loop once no lane holds a candidate and the queue is drained:
-        // a lane whose candidate just finished still holds an index below C and asks again)
+        // (the same barrier ends the loop once no lane holds a candidate and the queue is drained)
         const unsigned fail = __ballot_sync(0xffffffffu, failed);
         if (lane == 0) CL.wm[warp] = fail;
-        if (!__syncthreads_or(has || c < A.C)) break;
+        // (a lane whose candidate just finished still holds a place below the end and asks again)
+        if (HAND && qi >= items) CL.drained[0] = 1;
+        if (!__syncthreads_or(has || qi < items)) break;
+        const bool drained = HAND && CL.drained[0] != 0;  // some lane asked in vain: no candidate is left in the queue
         int nf = 0, before = 0;
 #pragma unroll
         for (int w = 0; w < WARPS; ++w) {
@@ -732,6 +746,21 @@ __global__ void __launch_bounds__(WARPS * 32, 16 / WARPS) k_lm(const LmArgs A) {
             ++n_it;
         }
         __syncwarp();
+        if (HAND && A.hand_at > 0 && ++rounds >= A.hand_at && drained) {
+            // the candidates that are left, packed afresh, take less time in the kernel that spreads a
+            // candidate over a CTA
+            const unsigned m = __ballot_sync(0xffffffffu, has);
+            int at = 0;
+            if (lane == 0 && m) at = atomicAdd(A.n_list, __popc(m));
+            at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
+            if (has) {
+                A.list[at] = (int32_t)c;
+                A.list_k[at] = kk;
+#pragma unroll 1
+                for (int j = 0; j < n; ++j) A.th[j * A.ld + c] = S.th(j, lane);
+            }
+            break;
+        }
     }
     if (A.cnt) {
         n_it = warp_sum(n_it);
@@ -832,8 +861,9 @@ __device__ __forceinline__ Frame lmc_flange(const LmC& C, const RobotParams& R, 
 __device__ __constant__ int8_t kTriRow[21] = {0, 1, 1, 2, 2, 2, 3, 3, 3, 3, 4, 4, 4, 4, 4, 5, 5, 5, 5, 5, 5};
 __device__ __constant__ int8_t kTriCol[21] = {0, 0, 1, 0, 1, 2, 0, 1, 2, 3, 0, 1, 2, 3, 4, 0, 1, 2, 3, 4, 5};
 
-// RED as for k_lm; N > 0: the launch's one robot has N joints (unrolled loops); N = 0: any robots
-template <bool RED, int N>
+// RED as for k_lm; N > 0: the launch's one robot has N joints (unrolled loops); N = 0: any robots;
+// LIST: the candidates that a k_lm launch handed over, from the iterations they had reached
+template <bool RED, int N, bool LIST>
 __global__ void __launch_bounds__(kCoopLmWarps * 32, 1) k_lm_coop(const LmArgs A) {
     extern __shared__ __align__(16) float smem_f[];
     __shared__ float alphas[kCoopMaxA + 1];
@@ -859,11 +889,14 @@ __global__ void __launch_bounds__(kCoopLmWarps * 32, 1) k_lm_coop(const LmArgs A
         return make_float2(cn, sn);
     };
 
-    for (int64_t base = kCoopCands * (int64_t)blockIdx.x; base < A.C; base += kCoopCands * (int64_t)gridDim.x) {
+    const int64_t items = LIST ? (int64_t)*A.n_list : A.C;
+    if (LIST && items > A.list_lim) return;  // too many: the other kernel's
+    for (int64_t base = kCoopCands * (int64_t)blockIdx.x; base < items; base += kCoopCands * (int64_t)gridDim.x) {
         __syncthreads();  // the last group's state is no longer read
-        const int64_t c = base + l;
         int32_t t = 0, s = 0;
-        bool have = c < A.C;
+        bool have = base + l < items;
+        const int64_t c = LIST && have ? (int64_t)A.list[base + l] : base + l;
+        const int kbase = LIST && have ? A.list_k[base + l] : 0;  // iterations taken before the hand-over
         if (have) have = A.map.lookup(c, t, s);
         const TargetDesc T = A.tg[have ? t : 0];
         const RobotParams& R = N ? rob[0] : rob[have ? T.robot : 0];
@@ -885,7 +918,7 @@ __global__ void __launch_bounds__(kCoopLmWarps * 32, 1) k_lm_coop(const LmArgs A
         if (u == 0) C.si(kStat) = 0;
         __syncthreads();
 
-        for (int kk = 0;; ++kk) {
+        for (int kk = kbase;; ++kk) {
             // kinematics with frames
             if (u < 3) lmc_fk_row<N, true>(C, R, n, 0, u);
             __syncthreads();
@@ -1151,6 +1184,14 @@ __global__ void __launch_bounds__(kCoopLmWarps * 32, 1) k_lm_coop(const LmArgs A
                 }
             }
             __syncthreads();
+            if (!LIST && kk + 1 == A.hand_at) {  // the candidates that are left are packed afresh by the next launch
+                if (u == 0 && alive) {
+                    const int at = atomicAdd(A.n_list, 1);
+                    A.list[at] = (int32_t)c;
+                    A.list_k[at] = kk + 1;
+                }
+                break;
+            }
         }
         if (mine)
             for (int j = u; j < n; j += U) A.th[j * A.ld + c] = C.th(j);
@@ -1167,42 +1208,43 @@ __global__ void __launch_bounds__(kCoopLmWarps * 32, 1) k_lm_coop(const LmArgs A
     }
 }
 
-template <bool RED, int N>
+template <bool RED, int N, bool LIST>
 void launch_lm_coop_n(const LmArgs& A, int warps, cudaStream_t st) {
     const size_t smem = robots_smem_bytes(A.rs.n) + coop_lm_bytes(A.rs.n_max, A.P.lm_A);
     static SmemLimit lim;
-    allow_dyn_smem(k_lm_coop<RED, N>, lim, robots_smem_bytes(kMaxLaunchRobots) + coop_lm_bytes(N ? N : kMaxDof, kCoopMaxA));
+    allow_dyn_smem(k_lm_coop<RED, N, LIST>, lim,
+                   robots_smem_bytes(kMaxLaunchRobots) + coop_lm_bytes(N ? N : kMaxDof, kCoopMaxA));
     int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lm_coop<RED, N>, 32 * warps, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lm_coop<RED, N, LIST>, 32 * warps, smem);
     const int g = (int)std::min<int64_t>((A.C + kCoopCands - 1) / kCoopCands, (int64_t)sm_count() * std::max(per_sm, 1));
-    k_lm_coop<RED, N><<<g, 32 * warps, smem, st>>>(A);
+    k_lm_coop<RED, N, LIST><<<g, 32 * warps, smem, st>>>(A);
 }
 
-template <bool RED>
+template <bool RED, bool LIST>
 void launch_lm_coop(const LmArgs& A, int warps, cudaStream_t st) {
     const int n = A.rs.n == 1 ? A.rs.n_max : 0;
-    if (n == 6) launch_lm_coop_n<RED, 6>(A, warps, st);
-    else if (n == 7) launch_lm_coop_n<RED, 7>(A, warps, st);
-    else launch_lm_coop_n<RED, 0>(A, warps, st);
+    if (n == 6) launch_lm_coop_n<RED, 6, LIST>(A, warps, st);
+    else if (n == 7) launch_lm_coop_n<RED, 7, LIST>(A, warps, st);
+    else launch_lm_coop_n<RED, 0, LIST>(A, warps, st);
 }
 
-template <bool TRACE, int WARPS, bool RED>
+template <bool TRACE, int WARPS, bool RED, bool HAND>
 void launch_lm_t(const LmArgs& A, cudaStream_t st) {
     const size_t smem = robots_smem_bytes(A.rs.n) +
                         sizeof(float) * ((size_t)lm_warp_words(A.rs.n_max, A.P.lm_A) * WARPS + lm_cta_words<WARPS>());
     static SmemLimit lim;
-    allow_dyn_smem(k_lm<TRACE, WARPS, RED>, lim,
+    allow_dyn_smem(k_lm<TRACE, WARPS, RED, HAND>, lim,
                    robots_smem_bytes(kMaxLaunchRobots) +
                        sizeof(float) * ((size_t)lm_warp_words(kMaxDof, kMaxLsDepth) * WARPS + lm_cta_words<WARPS>()));
     int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lm<TRACE, WARPS, RED>, WARPS * 32, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lm<TRACE, WARPS, RED, HAND>, WARPS * 32, smem);
     if (per_sm < 1) per_sm = 1;
     const int64_t want = (A.C + 32 * WARPS - 1) / (32 * WARPS);
     const int g = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)sm_count() * per_sm));
-    k_lm<TRACE, WARPS, RED><<<g, WARPS * 32, smem, st>>>(A);
+    k_lm<TRACE, WARPS, RED, HAND><<<g, WARPS * 32, smem, st>>>(A);
 }
 
-template <bool TRACE, bool RED>
+template <bool TRACE, bool RED, bool HAND>
 void launch_lm_w(const LmArgs& A, cudaStream_t st) {
     // fewer warps per CTA when the requested count's state does not fit in shared memory
     int optin = 0;
@@ -1212,33 +1254,69 @@ void launch_lm_w(const LmArgs& A, cudaStream_t st) {
     // a batch too small to give every SM a CTA of two warps (a single target, say): two-warp CTAs,
     // spread over more SMs with shorter lock-step stages (latency, not throughput, is at stake)
     if (A.C <= (int64_t)sm_count() * 64) warps = 2;
-    // (the CTA lists: 65 words per warp and one; 256 bytes kept for the kernel's static arrays)
-    while (warps > 2 && robots_smem_bytes(A.rs.n) + (per_warp + sizeof(float) * 65) * warps + 4 + 256 > (size_t)optin)
+    // (the CTA lists: 65 words per warp and two; 256 bytes kept for the kernel's static arrays)
+    while (warps > 2 && robots_smem_bytes(A.rs.n) + (per_warp + sizeof(float) * 65) * warps + 8 + 256 > (size_t)optin)
         warps /= 2;
-    if (warps == 2) launch_lm_t<TRACE, 2, RED>(A, st);
-    else if (warps == 4) launch_lm_t<TRACE, 4, RED>(A, st);
-    else launch_lm_t<TRACE, 8, RED>(A, st);
+    if (warps == 2) launch_lm_t<TRACE, 2, RED, HAND>(A, st);
+    else if (warps == 4) launch_lm_t<TRACE, 4, RED, HAND>(A, st);
+    else launch_lm_t<TRACE, 8, RED, HAND>(A, st);
 }
 
 }  // namespace
 
-void launch_lm(const LmArgs& A, bool trace, cudaStream_t st) {
-    if (A.C <= 0) return;
+int launch_lm(const LmArgs& B, bool trace, cudaStream_t st) {
+    if (B.C <= 0) return 0;
+    LmArgs A = B;
+    A.hand_at = A.list_in = A.list_lim = 0;
+    const bool coop = !trace && A.P.lm_A <= kCoopMaxA;
+    const bool plain = A.in_limits && A.rs.plain;
+    const int64_t sms = sm_count();
+    auto lanes = [&]() {
+        const bool hand = A.hand_at > 0 || A.list_in;
+        if (trace) launch_lm_w<true, true, false>(A, st);
+        else if (hand && plain) launch_lm_w<false, false, true>(A, st);
+        else if (hand) launch_lm_w<false, true, true>(A, st);
+        else if (plain) launch_lm_w<false, false, false>(A, st);
+        else launch_lm_w<false, true, false>(A, st);
+    };
     // Up to 64 candidates per SM (two resident CTAs of 16 on every SM, twice) the spread kernel's
     // shorter iterations win; past that its extra work does.  Phase time of the polish, spread /
     // one lane per candidate, us (7, 20, 24 joints): 1000 candidates 74 / 172, 123 / 328, 137 / 360;
     // 4000: 86 / 200, 168 / 346, 182 / 356; 8000: 166 / 221, 322 / 346, 338 / 356; 16000: 311 / 240,
     // 594 / 395, 616 / 363.  Twelve warps while a CTA has its SM to itself (8: 76, 139, 150), eight
     // (two CTAs per SM) beyond.
-    if (!trace && A.P.lm_A <= kCoopMaxA && A.C <= (int64_t)sm_count() * 4 * kCoopCands) {
-        const int warps = A.C <= (int64_t)sm_count() * kCoopCands ? 12 : 8;
-        if (A.in_limits && A.rs.plain) launch_lm_coop<false>(A, warps, st);
-        else launch_lm_coop<true>(A, warps, st);
-        return;
+    //
+    // Where the caller gives a list, batches of up to 216 candidates per SM leave the candidates that
+    // need more than a few iterations to a second launch, packed afresh: most candidates converge
+    // in those, and the rest (a fifth of Panda's run to the cap of 20) fit the spread kernel.  Up to 80 per
+    // SM four iterations of the spread kernel, beyond six of one lane per candidate; more than 64 per
+    // SM left (a chain that rarely reaches its targets) go on with one lane each.  One launch / two, us
+    // (7, 12, 20 joints, and 6 joints of which a third run to the cap): 5000: 156 / 102, 219 / 137, 291 /
+    // 178, 145 / 104; 8000: 168 / 111, 240 / 154, 322 / 203, 158 / 166; 16000: 248 / 150, 305 / 195, 403 /
+    // 254, 276 / 287; 32000: 248 / 205, 334 / 285, 406 / 369, 281 / 295; 48000 no gain.
+    if (!coop || A.C > (A.list ? sms * 216 : sms * 4 * kCoopCands)) {
+        lanes();
+        return 1;
     }
-    if (trace) launch_lm_w<true, true>(A, st);
-    else if (A.in_limits && A.rs.plain) launch_lm_w<false, false>(A, st);
-    else launch_lm_w<false, true>(A, st);
+    const bool hand = A.list && A.C > sms * 2 * kCoopCands;
+    const bool spread = A.C <= (hand ? sms * 80 : sms * 4 * kCoopCands);
+    if (hand) A.hand_at = spread ? 4 : 6;
+    if (spread) {
+        const int warps = A.C <= sms * kCoopCands ? 12 : 8;
+        if (plain) launch_lm_coop<false, false>(A, warps, st);
+        else launch_lm_coop<true, false>(A, warps, st);
+    } else {
+        lanes();
+    }
+    if (!hand) return 1;
+    A.hand_at = 0;
+    A.list_lim = spread ? 0x7fffffff : (int)(sms * 4 * kCoopCands);
+    if (plain) launch_lm_coop<false, true>(A, 8, st);
+    else launch_lm_coop<true, true>(A, 8, st);
+    if (spread) return 2;
+    A.list_in = 1;
+    lanes();
+    return 3;
 }
 
 }  // namespace hjcd

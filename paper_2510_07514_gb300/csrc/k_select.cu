@@ -237,8 +237,8 @@ __global__ void k_pack_targets(const float* pq7, int T, const TargetDesc tmpl, T
 // 228 -> 189 us.
 __global__ void __launch_bounds__(256) k_wave_init(const WaveInitArgs A) {
     const size_t tid = blockIdx.x * (size_t)blockDim.x + threadIdx.x, nth = (size_t)gridDim.x * blockDim.x;
-    if (tid < 6) A.zero[tid] = 0;
-    if (tid == 6) *A.flag = 0;
+    if (tid < 7) A.zero[tid] = 0;
+    if (tid == 7) *A.flag = 0;
     const uint4* src = reinterpret_cast<const uint4*>(A.pin);
     uint4* dst = reinterpret_cast<uint4*>(A.ws);
     const size_t g0 = A.o_tg / 16, g1 = g0 + (size_t)A.T * (sizeof(TargetDesc) / 16);  // the target rows: below

@@ -82,16 +82,21 @@ def test_small_batches_give_the_bits_of_large_ones(ctx, stage, which):
                 np.testing.assert_array_equal(x.view(np.uint32), np.ascontiguousarray(y[..., a:b]).view(np.uint32))
 
 
-@pytest.mark.parametrize("which,seeds", [("random0", 997), ("chain7", 1000), ("chain12", 333), ("random5", 500)])
-def test_small_solves_give_the_rows_of_large_ones(ctx, which, seeds):
+@pytest.mark.parametrize("which,seeds,cap", [("random0", 997, 20), ("chain7", 1000, 20), ("chain12", 333, 20), ("random5", 500, 20),
+                                             ("chain7", 256, 0), ("chain7", 256, 4), ("chain7", 256, 6), ("random0", 256, 7)])
+def test_small_solves_give_the_rows_of_large_ones(ctx, which, seeds, cap):
+    """Every size class of the polish (spread; spread, then the rest packed afresh; one lane per
+    candidate, then few or many left) against one launch of one lane per candidate, also with caps
+    around the iterations after which the candidates are packed afresh."""
     rob = _robot(which)
     rid = ctx.add_robot(rob)
-    T = 10500 // seeds + 1
+    T = 36000 // seeds + 1
+    params = api.make_params(lm_max_iters=cap)
     th = torch.as_tensor(inputs.joint_samples(np.random.default_rng(3), rob, T).T.copy(), dtype=torch.float32, device="cuda")
     tg = ctx.fk(rid, th)
-    big = ctx.solve(rid, -1, tg, seeds, 16, 5, rob.n)
-    for t in (1, 3):
-        small = ctx.solve(rid, -1, tg[:t].contiguous(), seeds, 16, 5, rob.n)
+    big = ctx.solve(rid, -1, tg, seeds, 64, 5, rob.n, params=params)
+    for t in (1, 3, 6000 // seeds, 11500 // seeds, 14000 // seeds, 30000 // seeds):
+        small = ctx.solve(rid, -1, tg[:t].contiguous(), seeds, 64, 5, rob.n, params=params)
         for x, y in zip(small, big):
             assert torch.equal(x.view(torch.int32), y[:t].view(torch.int32))
 
