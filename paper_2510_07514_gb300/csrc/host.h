@@ -141,6 +141,7 @@ struct WaveItem {
 };
 
 struct WavePlan {
+    std::vector<int> order;  // the items, longest chains first: their targets' rows follow it
     int n_items = 0, T = 0, NR = 0, NS = 0;
     int64_t CM = 0, CB = 0;
     int max_m = 0, max_b = 0, min_m = 0;  // min_m == max_m: every target has max_m seeds

@@ -96,14 +96,26 @@ hjcd_status plan_wave(hjcd_ctx* ctx, const WaveItem* items, int n_items, const h
                 if (!(nn > 0.0f) || !std::isfinite(nn)) return fail(ctx, HJCD_EINVAL, "item %d target %d: zero quaternion", i, t);
             }
         }
-        // seeds and candidates
+        for (int t = 0; t < it.T; ++t) {
+            const int m = it.spt ? it.spt[t] : it.n_samples;
+            if (m < 1 || m > HJCD_MAX_SAMPLES)
+                return fail(ctx, HJCD_EINVAL, "item %d target %d: seed count %d outside [1, %d]", i, t, m, HJCD_MAX_SAMPLES);
+        }
+    }
+    // rows, seeds and candidates, the items with the longest chains first: their candidates take longest,
+    // so the kernels' queues end on short work, and candidates that share a CTA of the polish, which
+    // wait for one another, are of similar length.  Eight chains of 6 to 20 joints x 40 targets in
+    // ascending order 3.57 -> 3.38 ms (shortest first: 3.60); a burst of 20 served requests 1.75 -> 1.57.
+    W.order.resize(n_items);
+    for (int i = 0; i < n_items; ++i) W.order[i] = i;
+    std::stable_sort(W.order.begin(), W.order.end(), [&](int x, int y) { return items[x].rob->P.n > items[y].rob->P.n; });
+    for (int i : W.order) {
+        const WaveItem& it = items[i];
         W.item_t0[i] = W.T;
         W.item_q0[i] = W.q_total;
         W.item_e0[i] = W.e_total;
         for (int t = 0; t < it.T; ++t) {
             const int m = it.spt ? it.spt[t] : it.n_samples;
-            if (m < 1 || m > HJCD_MAX_SAMPLES)
-                return fail(ctx, HJCD_EINVAL, "item %d target %d: seed count %d outside [1, %d]", i, t, m, HJCD_MAX_SAMPLES);
             const int64_t b = dup_count(m, P.dup_ratio);
             W.CM += m;
             W.CB += b;
@@ -220,7 +232,7 @@ hjcd_status run_wave(hjcd_ctx* ctx, const WavePlan& W, const WaveItem* items, co
         }
     }
     h_moff[0] = h_boff[0] = 0;
-    for (int i = 0; i < W.n_items; ++i) {
+    for (int i : W.order) {
         const WaveItem& it = items[i];
         const int n = it.rob->P.n;
         const int cd = it.cd_iters >= 0 ? it.cd_iters : P.cd_max_iters;
