@@ -33,13 +33,16 @@ constexpr int kCcdThreads = 128;
 // accesses hit 32 different banks): per joint j the pairs (px, py), (pz, theta_j), (zx, zy),
 // (zz, -) of joint j's frame after its kinematics step, 8 n words in all; each pair moves as one
 // 64-bit access
-template <int TH>
+template <int TH, bool PACK = false>
 struct ColT {
+    static constexpr int kWords = 8;  // per joint
     float2* base;  // this thread's first pair
+    __device__ __forceinline__ ColT(float2* b, int) : base(b) {}
+    __device__ __forceinline__ ColT lane(int d) const { return ColT(base + d, 0); }  // the column d threads on
+    __device__ __forceinline__ float& zz(int j) const { return base[(4 * j + 3) * TH].x; }
     __device__ __forceinline__ float2& a(int j) const { return base[4 * j * TH]; }
     __device__ __forceinline__ float2& b(int j) const { return base[(4 * j + 1) * TH]; }
     __device__ __forceinline__ float2& c(int j) const { return base[(4 * j + 2) * TH]; }
-    __device__ __forceinline__ float& zz(int j) const { return base[(4 * j + 3) * TH].x; }
     __device__ __forceinline__ float& th(int j) const { return b(j).y; }
     // joint j's origin and axis
     __device__ __forceinline__ void frame(int j, V3& p, V3& z) const {
@@ -54,7 +57,35 @@ struct ColT {
         zz(j) = F.c2.z;
     }
 };
-constexpr int kColWordsPerJoint = 8;
+// The same with zz in words of its own after all the pairs, 7 n words in all: one address more to
+// keep (2.5% of a Panda launch), but room for more resident CTAs of long chains.
+template <int TH>
+struct ColT<TH, true> {
+    static constexpr int kWords = 7;
+    float2* base;  // this thread's first pair
+    float* zb;     // this thread's first zz
+    __device__ __forceinline__ ColT(float2* b, float* z) : base(b), zb(z) {}
+    // the column of a CTA whose thread 0 has its first pair at b - threadIdx.x, for chains of n joints
+    __device__ __forceinline__ ColT(float2* b, int n)
+        : base(b), zb(reinterpret_cast<float*>(b - threadIdx.x + 3 * n * TH) + threadIdx.x) {}
+    __device__ __forceinline__ ColT lane(int d) const { return ColT(base + d, zb + d); }
+    __device__ __forceinline__ float2& a(int j) const { return base[3 * j * TH]; }
+    __device__ __forceinline__ float2& b(int j) const { return base[(3 * j + 1) * TH]; }
+    __device__ __forceinline__ float2& c(int j) const { return base[(3 * j + 2) * TH]; }
+    __device__ __forceinline__ float& zz(int j) const { return zb[j * TH]; }
+    __device__ __forceinline__ float& th(int j) const { return b(j).y; }
+    __device__ __forceinline__ void frame(int j, V3& p, V3& z) const {
+        const float2 pa = a(j), pb = b(j), za = c(j);
+        p = v3(pa.x, pa.y, pb.x);
+        z = v3(za.x, za.y, zz(j));
+    }
+    __device__ __forceinline__ void set_frame(int j, const Frame& F, float theta) const {
+        a(j) = make_float2(F.p.x, F.p.y);
+        b(j) = make_float2(F.p.z, theta);
+        c(j) = make_float2(F.c2.x, F.c2.y);
+        zz(j) = F.c2.z;
+    }
+};
 
 // the joint vector alone, theta[n] (the seed-sampling kernel)
 template <int TH>
@@ -205,9 +236,9 @@ constexpr int kSlotWords = 8;  // per-thread shared-memory slot of the cooperati
 __constant__ uint32_t kDivMagic[13] = {0, 65536, 32768, 21846, 16384, 13108, 10923, 9363, 8192, 7282, 6554, 5958, 5462};
 static_assert((kMaxDof + 1) / 2 <= 12, "the normal pairs of a joint vector index kDivMagic");
 
-template <bool TRACE, int TH, bool RED = true>
+template <bool TRACE, int TH, bool RED = true, bool PACK = false>
 __device__ __forceinline__ int ccd_step(const RobotParams* rob, const RobotParams& R, const TargetDesc& T,
-                                        const hjcd_params& P, const ColT<TH>& col, uint32_t* slots, const CcdArgs& A,
+                                        const hjcd_params& P, const ColT<TH, PACK>& col, uint32_t* slots, const CcdArgs& A,
                                         int64_t c, uint32_t s, int kk, int cap, float delta_k, const V3 pt, float pe2,
                                         float one_m_tie, float inv_p2, float inv_o2, float& ep2, float& eo) {
     const int n = R.n;
@@ -364,7 +395,7 @@ __device__ __forceinline__ int ccd_step(const RobotParams* rob, const RobotParam
             Tq.key[1] = q[1];
             Tq.t_local = (int32_t)q[2];
             const float2 z = normal_pair(Tq, q[3], kPhaseCd, q[4], b);
-            const ColT<TH> cs{col.base - lane + sl};
+            const ColT<TH, PACK> cs = col.lane(sl - lane);
             const int j0 = 2 * b, j1 = 2 * b + 1;
             cs.th(j0) = clampf(fmaf(P.cd_sigma, z.x, cs.th(j0)), Rs.lim[j0].x, Rs.lim[j0].y);
             if (j1 < Rs.n) cs.th(j1) = clampf(fmaf(P.cd_sigma, z.y, cs.th(j1)), Rs.lim[j1].x, Rs.lim[j1].y);
@@ -381,9 +412,9 @@ __device__ __forceinline__ int ccd_step(const RobotParams* rob, const RobotParam
 #endif
 // RED = false: the launch's joint vectors lie within the limits of plain robots (no offsets and
 // no range reduction in the kinematics steps; the same bits)
-template <bool TRACE, int TH, bool RED>
+template <bool TRACE, int TH, bool RED, bool PACK>
 __global__ void __launch_bounds__(TH, HJCD_CCD_THREADS_PER_SM / TH) k_ccd(const CcdArgs A) {
-    using Col = ColT<TH>;
+    using Col = ColT<TH, PACK>;
     extern __shared__ __align__(16) float sm[];
     const RobotParams* rob = stage_robots(sm, A.rs);
     uint32_t* const slots = reinterpret_cast<uint32_t*>(sm + robots_smem_bytes(A.rs.n) / sizeof(float));
@@ -419,7 +450,7 @@ __global__ void __launch_bounds__(TH, HJCD_CCD_THREADS_PER_SM / TH) k_ccd(const 
         const TargetDesc T = A.tg[t];
         const RobotParams& R = rob[T.robot];
         const int n = R.n;
-        const Col col{colbase};
+        const Col col(colbase, A.rs.n_max);
         const V3 pt = v3(T.p[0], T.p[1], T.p[2]);
         if (!A.list_in) ++n_cand;
 
@@ -455,7 +486,7 @@ __global__ void __launch_bounds__(TH, HJCD_CCD_THREADS_PER_SM / TH) k_ccd(const 
                 handed = true;
                 break;
             }
-            const int r = ccd_step<TRACE, TH, RED>(rob, R, T, P, col, slots, A, c, (uint32_t)s, kk, cap, delta_k, pt, pe2,
+            const int r = ccd_step<TRACE, TH, RED, PACK>(rob, R, T, P, col, slots, A, c, (uint32_t)s, kk, cap, delta_k, pt, pe2,
                                               one_m_tie, inv_p2, inv_o2, ep2, eo);
             if (r == 1) iters = kk;
             if (r) break;
@@ -915,7 +946,7 @@ __global__ void __launch_bounds__(TH, 4) k_ccd_lock(const CcdArgs A) {
     const TargetDesc T = A.tg[t];
     const RobotParams& R = rob[T.robot];
     const int n = R.n;
-    const ColT<TH> col{colbase};
+    const ColT<TH> col(colbase, A.rs.n_max);
     const int64_t m0 = A.map.off[t];
     const int M = (int)(A.map.off[t + 1] - m0);
     const bool valid = T.eps_pos > 0.0f;
@@ -999,20 +1030,38 @@ __global__ void __launch_bounds__(kCcdThreads) k_sample(const RobotParams R, uin
 }
 
 
+template <bool PACK>
+size_t ccd_smem(int robots, int n, int th) {
+    return robots_smem_bytes(robots) + sizeof(float) * (ColT<64, PACK>::kWords * n + kSlotWords) * th;
+}
+
+template <bool TRACE, int TH, bool RED, bool PACK>
+int prepare_ccd(const CcdArgs& A) {  // resident CTAs per SM
+    static SmemLimit lim;
+    allow_dyn_smem(k_ccd<TRACE, TH, RED, PACK>, lim, ccd_smem<PACK>(kMaxLaunchRobots, kMaxDof, TH));
+    int per_sm = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ccd<TRACE, TH, RED, PACK>, TH,
+                                                  ccd_smem<PACK>(A.rs.n, A.rs.n_max, TH));
+    return std::max(per_sm, 1);
+}
+
+template <bool TRACE, int TH, bool RED, bool PACK>
+void launch_ccd_p(const CcdArgs& A, int per_sm, cudaStream_t st) {
+    int g = grid_for(A.C, TH, 16 * 128 / TH);
+    if (A.queue) g = std::min(g, sm_count() * per_sm);  // the resident CTAs only: the queue spreads the items
+    k_ccd<TRACE, TH, RED, PACK><<<g, TH, ccd_smem<PACK>(A.rs.n, A.rs.n_max, TH), st>>>(A);
+}
+
 template <bool TRACE, int TH, bool RED>
 void launch_ccd_t(const CcdArgs& A, cudaStream_t st) {
-    const size_t smem =
-        robots_smem_bytes(A.rs.n) + sizeof(float) * (kColWordsPerJoint * A.rs.n_max + kSlotWords) * TH;
-    static SmemLimit lim;
-    allow_dyn_smem(k_ccd<TRACE, TH, RED>, lim,
-                   robots_smem_bytes(kMaxLaunchRobots) + sizeof(float) * (kColWordsPerJoint * kMaxDof + kSlotWords) * TH);
-    int g = grid_for(A.C, TH, 16 * 128 / TH);
-    if (A.queue) {  // the resident CTAs only: the queue spreads the items
-        int per_sm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ccd<TRACE, TH, RED>, TH, smem);
-        g = std::min(g, sm_count() * std::max(per_sm, 1));
+    const int per_sm = prepare_ccd<TRACE, TH, RED, false>(A);
+    if (!TRACE) {
+        // the packed column where it lets a fifth more CTAs reside (8 robots of up to 20 joints: 4 -> 5,
+        // 1.42 -> 1.27 ms; at 12 joints, 7 -> 8, it costs 1%)
+        const int packed = prepare_ccd<TRACE, TH, RED, !TRACE>(A);
+        if (5 * packed >= 6 * per_sm) return launch_ccd_p<TRACE, TH, RED, !TRACE>(A, packed, st);
     }
-    k_ccd<TRACE, TH, RED><<<g, TH, smem, st>>>(A);
+    launch_ccd_p<TRACE, TH, RED, false>(A, per_sm, st);
 }
 
 template <bool RED, int N>
@@ -1047,11 +1096,9 @@ void launch_ccd(const CcdArgs& A, bool trace, cudaStream_t st) {
     if (A.C <= 0) return;
     if (A.P.cd_variant == 2) {  // one CTA per target (offset maps only)
         const size_t smem =
-            robots_smem_bytes(A.rs.n) + sizeof(float) * (kColWordsPerJoint * A.rs.n_max + kSlotWords) * 128;
+            ccd_smem<false>(A.rs.n, A.rs.n_max, 128);
         static SmemLimit lim;
-        allow_dyn_smem(k_ccd_lock<128>, lim,
-                       robots_smem_bytes(kMaxLaunchRobots) +
-                           sizeof(float) * (kColWordsPerJoint * kMaxDof + kSlotWords) * 128);
+        allow_dyn_smem(k_ccd_lock<128>, lim, ccd_smem<false>(kMaxLaunchRobots, kMaxDof, 128));
         k_ccd_lock<128><<<A.map.T, 128, smem, st>>>(A);
         return;
     }

@@ -120,6 +120,26 @@ def test_a_small_mixed_batch_gives_each_request_its_bits(ctx):
             assert torch.equal(x.view(torch.int32), y[:3].view(torch.int32))
 
 
+def test_a_large_mixed_batch_gives_each_request_its_bits(ctx):
+    """Eight robots of 6 to 20 joints with uneven seed counts in one batch (the packed PO-CCD column,
+    rows in descending chain length) against each request alone."""
+    rng = np.random.default_rng(12)
+    items, alone = [], []
+    for k in range(8):
+        rob = _robot("random%d" % k)
+        rid = ctx.add_robot(rob)
+        th = torch.as_tensor(inputs.joint_samples(rng, rob, 20).T.copy(), dtype=torch.float32, device="cuda")
+        tg = ctx.fk(rid, th)
+        spt = rng.integers(30, 700, 20).astype(np.int32)
+        items.append(ctx.batch_item(rid, -1, tg, int(spt.max()), 8, 21 + k, rob.n, samples_per_target=spt))
+        alone.append(ctx.solve(rid, -1, tg, int(spt.max()), 8, 21 + k, rob.n, samples_per_target=spt))
+    ctx.solve_batch([it for it, _ in items])
+    torch.cuda.synchronize()
+    for (_, got), ref in zip(items, alone):
+        for x, y in zip(got, ref):
+            assert torch.equal(x.view(torch.int32), y.view(torch.int32))
+
+
 @pytest.mark.parametrize("which", ["planar1", "chain7", "random2", "offsets", "chain24"])
 def test_fk_does_not_depend_on_the_batch(ctx, which):
     """Two candidates share a thread and a warp's 64 poses one store: every remainder, and an output
