@@ -1255,8 +1255,19 @@ void launch_lm_w(const LmArgs& A, cudaStream_t st) {
     // spread over more SMs with shorter lock-step stages (latency, not throughput, is at stake)
     if (A.C <= (int64_t)sm_count() * 64) warps = 2;
     // (the CTA lists: 65 words per warp and two; 256 bytes kept for the kernel's static arrays)
-    while (warps > 2 && robots_smem_bytes(A.rs.n) + (per_warp + sizeof(float) * 65) * warps + 8 + 256 > (size_t)optin)
-        warps /= 2;
+    auto bytes = [&](int w) { return robots_smem_bytes(A.rs.n) + (per_warp + sizeof(float) * 65) * w + 8 + 256; };
+    while (warps > 2 && bytes(warps) > (size_t)optin) warps /= 2;
+    // or where that lets a fifth more warps reside, or as many of no more than eight (which then wait at
+    // barriers of their own).  us with eight warps -> so, 250 targets x 1000 seeds: 12 joints (one CTA of 8
+    // warps, three of 4) 864 -> 707, 16 joints (8, 5 of 2) 853 -> 787, 18 joints (8, 4 of 2) 836 -> 774, 24
+    // joints (4, 3 of 2) 1202 -> 905; 7 and 9 joints keep two CTAs of 8 (512 against 565 with 2).
+    int sm_bytes = 0;
+    cudaDeviceGetAttribute(&sm_bytes, cudaDevAttrMaxSharedMemoryPerMultiprocessor, current_device());
+    auto resident = [&](int w) { return std::min(16, (int)((size_t)sm_bytes / (bytes(w) + 1024)) * w); };
+    for (int w = warps / 2; w >= 2; w /= 2) {
+        const int r = resident(w), r0 = resident(warps);
+        if (5 * r >= 6 * r0 || (r >= r0 && r0 <= 8)) warps = w;
+    }
     if (warps == 2) launch_lm_t<TRACE, 2, RED, HAND>(A, st);
     else if (warps == 4) launch_lm_t<TRACE, 4, RED, HAND>(A, st);
     else launch_lm_t<TRACE, 8, RED, HAND>(A, st);
