@@ -785,8 +785,12 @@ __global__ void __launch_bounds__(WARPS * 32, 16 / WARPS) k_lm(const LmArgs A) {
 // perturbation's draws are made beside the factorisations.  Each quantity is formed by k_lm's
 // operations in their order (the sums over the joints and over the rows as well), so the results
 // are its bits.  Bound by latency: thirteen exchanges per iteration, the residuals (a lone warp's
-// chain of about 150 dependent instructions) and the 6 x 6 solve the longest stages.  One Panda
-// target of 1000 seeds: 74 us for at most 20 iterations, where k_lm takes 172 us.
+// chain of about 150 dependent instructions) and the 6 x 6 solve the longest stages; about an eighth of
+// the warps' time outside barriers is instruction fetch (a stage's code runs once per iteration and all of
+// it does not stay in the first cache), so work moved beside other work pays only where it adds little
+// code.  Loads stand ahead of stores, which the compiler does not move them across.  One Panda target of
+// 1000 seeds: 70 us for at most 20 iterations, where k_lm takes 172 us (74 before the loads were moved
+// ahead in the kinematics rows, columns and matrix entries).
 constexpr int kCoopCands = 16;    // candidates per CTA
 constexpr int kCoopLmWarps = 16;  // most warps per CTA
 constexpr int kCoopMaxA = 6;      // deepest line search taken here
@@ -827,9 +831,7 @@ template <int N, bool FRAMES>
 __device__ __forceinline__ void lmc_fk_row(const LmC& C, const RobotParams& R, int n_, int set, int row) {
     const int n = N ? N : n_;
     float c0 = row == 0 ? 1.0f : 0.0f, c1 = row == 1 ? 1.0f : 0.0f, c2 = row == 2 ? 1.0f : 0.0f, p = 0.0f;
-    auto step = [&](int j) {
-        const float4 g = R.dh[j];
-        const float2 cs = C.cs(set, j);
+    auto step = [&](int j, const float4 g, const float2 cs) {
         const float b1 = fmaf(g.x, c1, g.y * c2);
         const float b2 = fmaf(g.x, c2, (-g.y) * c1);
         p = fmaf(g.w, b2, fmaf(g.z, c0, p));
@@ -842,12 +844,19 @@ __device__ __forceinline__ void lmc_fk_row(const LmC& C, const RobotParams& R, i
             C.fr(3 + row, j) = c2;
         }
     };
-    if (N) {
+    if (N) {  // all loads come before the stores, which the compiler may not move them across
+        float4 g[N ? N : 1];
+        float2 cs[N ? N : 1];
 #pragma unroll
-        for (int j = 0; j < N; ++j) step(j);
+        for (int j = 0; j < N; ++j) {
+            g[j] = R.dh[j];
+            cs[j] = C.cs(set, j);
+        }
+#pragma unroll
+        for (int j = 0; j < N; ++j) step(j, g[j], cs[j]);
     } else {
 #pragma unroll 4
-        for (int j = 0; j < n; ++j) step(j);
+        for (int j = 0; j < n; ++j) step(j, R.dh[j], C.cs(set, j));
     }
     C.e(set, row) = make_float4(c0, c1, c2, p);
 }
@@ -889,6 +898,15 @@ __global__ void __launch_bounds__(kCoopLmWarps * 32, 1) k_lm_coop(const LmArgs A
         return make_float2(cn, sn);
     };
 
+    // the normal matrices' entries of this unit: q and q + U of 42, their operands found once
+    auto entry = [&](int q, const float*& a, const float*& b) {
+        const int k = q < 21 ? q : q - 21;
+        a = q < 21 ? &C.sc(kTriRow[k], 0) : &C.jc(kTriRow[k], 0);
+        b = q < 21 ? &C.sc(kTriCol[k], 0) : &C.jc(kTriCol[k], 0);
+    };
+    const float *a0, *b0, *a1, *b1;
+    entry(u, a0, b0);  // (u < 32)
+    entry(min(u + U, 41), a1, b1);
     const int64_t items = LIST ? (int64_t)*A.n_list : A.C;
     if (LIST && items > A.list_lim) return;  // too many: the other kernel's
     for (int64_t base = kCoopCands * (int64_t)blockIdx.x; base < items; base += kCoopCands * (int64_t)gridDim.x) {
@@ -918,6 +936,11 @@ __global__ void __launch_bounds__(kCoopLmWarps * 32, 1) k_lm_coop(const LmArgs A
         if (u == 0) C.si(kStat) = 0;
         __syncthreads();
 
+        auto trial_sincos = [&](int i, int j) {  // of trial i's angle of joint j
+            const float dir = i <= lsA ? C.st(j) : fmaf(C.s(kWgn), C.dgn(j), C.s(kWgd) * C.g(j));
+            const float al = i <= lsA ? alphas[i] : 1.0f;
+            C.cs(1 + i, j) = sincos_of(R, j, clampf(fmaf(al, dir, C.th(j)), R.lim[j].x, R.lim[j].y));
+        };
         for (int kk = kbase;; ++kk) {
             // kinematics with frames
             if (u < 3) lmc_fk_row<N, true>(C, R, n, 0, u);
@@ -996,13 +1019,19 @@ __global__ void __launch_bounds__(kCoopLmWarps * 32, 1) k_lm_coop(const LmArgs A
                 }
             } else {
                 for (int j = u; j < n; j += U - 2) {
-                    float col[6], dd = 1e-9f;
+                    float col[6], w[6], dd = 1e-9f;
 #pragma unroll
                     for (int r = 0; r < 6; ++r) {
-                        col[r] = C.jc(r, j) * C.s(kW + r);
-                        dd = fmaf(col[r], col[r], dd);
-                        C.jc(r, j) = col[r];
+                        col[r] = C.jc(r, j);
+                        w[r] = C.s(kW + r);
                     }
+#pragma unroll
+                    for (int r = 0; r < 6; ++r) {
+                        col[r] *= w[r];
+                        dd = fmaf(col[r], col[r], dd);
+                    }
+#pragma unroll
+                    for (int r = 0; r < 6; ++r) C.jc(r, j) = col[r];
                     const float rs = rsqrtf(dd);
                     C.dd(j) = dd;
 #pragma unroll
@@ -1012,14 +1041,23 @@ __global__ void __launch_bounds__(kCoopLmWarps * 32, 1) k_lm_coop(const LmArgs A
             __syncthreads();
 
             // the normal matrices: entry q of the scaled columns' (LM), of the columns' (Gauss-Newton)
-            for (int q = u; q < 42; q += U) {
-                const int k = q < 21 ? q : q - 21;
-                const float* a = q < 21 ? &C.sc(kTriRow[k], 0) : &C.jc(kTriRow[k], 0);
-                const float* b = q < 21 ? &C.sc(kTriCol[k], 0) : &C.jc(kTriCol[k], 0);
-                float m = 0.0f;
+            {
+                float m0 = 0.0f, m1 = 0.0f;
+#pragma unroll(N ? N : 4)
+                for (int j = 0; j < n; ++j) {
+                    m0 = fmaf(a0[j * kCoopCands], b0[j * kCoopCands], m0);
+                    m1 = fmaf(a1[j * kCoopCands], b1[j * kCoopCands], m1);
+                }
+                C.s(kM + u) = m0;
+                if (u + U < 42) C.s(kM + u + U) = m1;
+                for (int q = u + 2 * U; q < 42; q += U) {
+                    const float *a, *b;
+                    entry(q, a, b);
+                    float m = 0.0f;
 #pragma unroll 4
-                for (int j = 0; j < n; ++j) m = fmaf(a[j * kCoopCands], b[j * kCoopCands], m);
-                C.s(kM + q) = m;
+                    for (int j = 0; j < n; ++j) m = fmaf(a[j * kCoopCands], b[j * kCoopCands], m);
+                    C.s(kM + q) = m;
+                }
             }
             __syncthreads();
 
@@ -1083,7 +1121,8 @@ __global__ void __launch_bounds__(kCoopLmWarps * 32, 1) k_lm_coop(const LmArgs A
             }
             __syncthreads();
 
-            // the dogleg's weights; the single coordinate
+            // the dogleg's weights; the single coordinate; of long chains, the sines and cosines of the line
+            // search beside them (24 joints: 133 -> 129 us; of short ones all trials' take two passes of the next stage)
             if (warp == 0) {
                 const float ac = C.s(kAc);
                 float ngn2 = 0.0f, qa = 0.0f, qb = 0.0f;
@@ -1117,16 +1156,13 @@ __global__ void __launch_bounds__(kCoopLmWarps * 32, 1) k_lm_coop(const LmArgs A
                     C.s(kSv + r) = __fdividef(col[r], C.s(kW + r));
                     C.s(kSz + r) = __fdividef(col[3 + r], C.s(kW + 3 + r));
                 }
+            } else if (!N) {
+                for (int w = u - 4; w < (nt - 1) * n; w += U - 4) trial_sincos(w / n, w % n);
             }
             __syncthreads();
 
             // sines and cosines of the trials' angles
-            for (int w = u; w < nt * n; w += U) {
-                const int i = N ? w / (N ? N : 1) : w / n, j = w - i * n;
-                const float dir = i <= lsA ? C.st(j) : fmaf(C.s(kWgn), C.dgn(j), C.s(kWgd) * C.g(j));
-                const float al = i <= lsA ? alphas[i] : 1.0f;
-                C.cs(1 + i, j) = sincos_of(R, j, clampf(fmaf(al, dir, C.th(j)), R.lim[j].x, R.lim[j].y));
-            }
+            for (int w = (N ? 0 : (nt - 1) * n) + u; w < nt * n; w += U) trial_sincos(w / n, w % n);
             __syncthreads();
 
             // the trials' kinematics rows
@@ -1177,7 +1213,7 @@ __global__ void __launch_bounds__(kCoopLmWarps * 32, 1) k_lm_coop(const LmArgs A
                     C.th(j) = th;
                     C.cs(0, j) = sincos_of(R, j, th);
                 }
-                if (u == 0) {  // the passes and trials the sequential method evaluates
+                if (u == U - 2) {  // the passes and trials the sequential method evaluates
                     ++n_it;
                     n_fk += pick >= 0 && pick < nt ? pick + 1 : nt;
                     if (pick < 0 || pick >= nt) n_sc += pick < 0 ? lsA + 1 : pick - nt + 1;
@@ -1292,9 +1328,9 @@ int launch_lm(const LmArgs& B, bool trace, cudaStream_t st) {
     };
     // Up to 64 candidates per SM (two resident CTAs of 16 on every SM, twice) the spread kernel's
     // shorter iterations win; past that its extra work does.  Phase time of the polish, spread /
-    // one lane per candidate, us (7, 20, 24 joints): 1000 candidates 74 / 172, 123 / 328, 137 / 360;
-    // 4000: 86 / 200, 168 / 346, 182 / 356; 8000: 166 / 221, 322 / 346, 338 / 356; 16000: 311 / 240,
-    // 594 / 395, 616 / 363.  Twelve warps while a CTA has its SM to itself (8: 76, 139, 150), eight
+    // one lane per candidate, us (7, 20, 24 joints): 1000 candidates 70 / 172, 115 / 328, 129 / 360;
+    // 4000: 84 / 200, 164 / 346, 178 / 356; 8000: 166 / 221, 322 / 346, 338 / 356; 16000: 311 / 240,
+    // 594 / 395, 616 / 363 (the last two with loads not yet ahead of the stores, 3 to 6% of its time).  Twelve warps while a CTA has its SM to itself (8: 76, 139, 150), eight
     // (two CTAs per SM) beyond.
     //
     // Where the caller gives a list, batches of up to 216 candidates per SM leave the candidates that
