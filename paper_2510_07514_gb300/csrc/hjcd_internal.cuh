@@ -314,6 +314,24 @@ __device__ __forceinline__ void fk_step(const RobotParams& R, int j, float theta
     F.c2 = v3(b2.x, b2.y, b2z);
 }
 
+// fk_step's operations with the cosine c and sine s of the joint's angle given
+__device__ __forceinline__ void fk_step_cs(const RobotParams& R, int j, float c, float s, Frame& F) {
+    const float4 g = R.dh[j];
+    const float ca = g.x, sa = g.y;
+    const float2 b1 = fma2(bc2(ca), xy(F.c1), mul2(bc2(sa), xy(F.c2)));
+    const float b1z = fmaf(ca, F.c1.z, sa * F.c2.z);
+    const float2 b2 = fma2(bc2(ca), xy(F.c2), mul2(bc2(-sa), xy(F.c1)));
+    const float b2z = fmaf(ca, F.c2.z, (-sa) * F.c1.z);
+    const float2 p = fma2(bc2(g.w), b2, fma2(bc2(g.z), xy(F.c0), xy(F.p)));
+    F.p = v3(p.x, p.y, fmaf(g.w, b2z, fmaf(g.z, F.c0.z, F.p.z)));
+    const float2 n0 = fma2(bc2(c), xy(F.c0), mul2(bc2(s), b1));
+    const float2 n1 = fma2(bc2(c), b1, mul2(bc2(-s), xy(F.c0)));
+    const float n0z = fmaf(c, F.c0.z, s * b1z), n1z = fmaf(c, b1z, (-s) * F.c0.z);
+    F.c0 = v3(n0.x, n0.y, n0z);
+    F.c1 = v3(n1.x, n1.y, n1z);
+    F.c2 = v3(b2.x, b2.y, b2z);
+}
+
 // flange frame from the last joint frame
 __device__ __forceinline__ Frame fk_flange(const RobotParams& R, const Frame& F) {
     Frame E;

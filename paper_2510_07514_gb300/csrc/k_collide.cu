@@ -145,6 +145,30 @@ struct WarpBufs {
     int* list;
 };
 
+// Makes robot rid the warp's current one.
+template <int SPL>
+__device__ __forceinline__ void warp_robot(const CollideArgs& A, const RobotParams* rob, WarpRobot<SPL>& W,
+                                           const WarpBufs& Bf, int rid) {
+    const int lane = threadIdx.x & 31;
+    W.cur = rid;
+    const RobotDev rd = A.rs.rd[rid];
+    W.n_m = rob[rid].n;
+    W.pairs_m = rd.n_pairs;
+    const int ns = rd.n_sph, nbr = W.n_m + 2;
+#pragma unroll
+    for (int q = 0; q < SPL; ++q) {
+        const int i = lane + 32 * q;
+        W.lb[q] = i < ns ? __ldg(rd.body + i) : -1;
+        W.ls[q] = i < ns ? __ldg(rd.sph + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    W.lco = lane < nbr ? __ldg(rd.coarse + lane) : make_float4(0.f, 0.f, 0.f, 0.f);
+    __syncwarp();
+    for (int i = lane; i < nbr; i += 32) Bf.wrange[i] = __ldg(rd.range + i);
+    for (int i = lane; i < W.pairs_m; i += 32) Bf.wpairs[i] = __ldg(rd.pairs + i);
+    __syncwarp();
+    W.bmask = __ballot_sync(0xffffffffu, lane < nbr && Bf.wrange[lane].y > 0);  // bodies with spheres
+}
+
 // Collision verdict of candidate c (robot row rid, scene row sid, -1: none),
 // warp-uniform; t_s / t_b accumulate the sphere and box tests.  SELF: the self-collision part only.
 template <int SPL, bool UNIFORM, bool GRID, bool SELF = false>
@@ -159,25 +183,7 @@ __device__ __forceinline__ bool warp_collides(const CollideArgs& A, const RobotP
     int2* const wrange = Bf.wrange;
     int2* const wpairs = Bf.wpairs;
     int* const list = Bf.list;
-    if (rid != W.cur) {
-        W.cur = rid;
-        const RobotDev rd = A.rs.rd[rid];
-        W.n_m = rob[rid].n;
-        W.pairs_m = rd.n_pairs;
-        const int ns = rd.n_sph, nbr = W.n_m + 2;
-#pragma unroll
-        for (int q = 0; q < SPL; ++q) {
-            const int i = lane + 32 * q;
-            W.lb[q] = i < ns ? __ldg(rd.body + i) : -1;
-            W.ls[q] = i < ns ? __ldg(rd.sph + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        W.lco = lane < nbr ? __ldg(rd.coarse + lane) : make_float4(0.f, 0.f, 0.f, 0.f);
-        __syncwarp();
-        for (int i = lane; i < nbr; i += 32) wrange[i] = __ldg(rd.range + i);
-        for (int i = lane; i < W.pairs_m; i += 32) wpairs[i] = __ldg(rd.pairs + i);
-        __syncwarp();
-        W.bmask = __ballot_sync(0xffffffffu, lane < nbr && wrange[lane].y > 0);  // bodies with spheres
-    }
+    if (rid != W.cur) warp_robot<SPL>(A, rob, W, Bf, rid);
     const RobotParams& R = rob[rid];
     const int n = UNIFORM ? A.u_n : W.n_m, nb = n + 2, n_pairs = UNIFORM ? A.u_pairs : W.pairs_m;
     // obstacles: the staged copy (shared memory) or the scene's table (global, read-only path)
@@ -200,9 +206,13 @@ __device__ __forceinline__ bool warp_collides(const CollideArgs& A, const RobotP
     for (int q = 0; q < SPL; ++q) ws[q] = W.ls[q];
     float4 wc = W.lco;
     Frame F = frame_identity();
+    // a lane loads and reduces one joint's angle; the chain then takes them in turn (a load per joint
+    // inside the chain made it wait for each: ranking of 1000 targets x 1000 189 us, so 155)
+    float sj = 0.0f, cj = 1.0f;
+    if (lane < n) sincos_red(A.th[lane * A.ld + c] + R.off[lane], &sj, &cj);
 #pragma unroll 1
     for (int j = 0; j < n; ++j) {
-        fk_step(R, j, A.th[j * A.ld + c], F);
+        fk_step_cs(R, j, __shfl_sync(0xffffffffu, cj, j), __shfl_sync(0xffffffffu, sj, j), F);
 #pragma unroll
         for (int q = 0; q < SPL; ++q)
             if (W.lb[q] == j + 1) ws[q] = to_world(F, W.ls[q]);
@@ -365,10 +375,11 @@ __device__ __forceinline__ bool warp_collides(const CollideArgs& A, const RobotP
 // CTA prologue of the collision kernels: the obstacles of a single scene
 // staged by one bulk copy (UNIFORM), the robots' kinematic tables with plain
 // loads.  False (error flag set) when the staging wait ran out or the scene
-// outgrew the shared memory the host sized; the CTA must return.
-template <bool UNIFORM>
+// outgrew the shared memory the host sized; the CTA must return.  `meanwhile`
+// runs (all threads, the robots staged) while the copy is under way.
+template <bool UNIFORM, class F>
 __device__ __forceinline__ bool collide_prologue(const CollideArgs& A, unsigned char* smem, const CollideLayout& L,
-                                                 const SceneDev& sc0, int n_obj4, const RobotParams** rob) {
+                                                 const SceneDev& sc0, int n_obj4, const RobotParams** rob, F&& meanwhile) {
     float4* s_scene = reinterpret_cast<float4*>(smem);
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem + L.bar);
     const uint32_t bytes = 16u * (uint32_t)n_obj4;
@@ -385,6 +396,7 @@ __device__ __forceinline__ bool collide_prologue(const CollideArgs& A, unsigned 
         }
     }
     *rob = stage_robots(smem + L.robots, A.rs);
+    meanwhile();
     if (UNIFORM) {
         const uint32_t polls = A.first_wait_polls < 0 ? kWaitLimit
                                : (uint32_t)(A.first_wait_polls < (int64_t)kWaitLimit ? A.first_wait_polls : kWaitLimit);
@@ -429,7 +441,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_collide(const CollideAr
     if (items == 0) return;
     const CollideLayout L = collide_smem_layout(n_obj4, A.rs.n, A.rs.n_max + 2, A.rs.ns_max, A.rs.pairs_max);
     const RobotParams* rob;
-    if (!collide_prologue<UNIFORM>(A, smem, L, sc0, n_obj4, &rob)) return;
+    if (!collide_prologue<UNIFORM>(A, smem, L, sc0, n_obj4, &rob, [] {})) return;
     const WarpBufs Bf = warp_bufs(smem, L, A);
     const float4* s_scene = reinterpret_cast<const float4*>(smem);
 
@@ -507,7 +519,20 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_rank_lazy(const Collide
     const CollideLayout L =
         collide_smem_layout(outgrown ? 0 : n_obj4, A.rs.n, A.rs.n_max + 2, A.rs.ns_max, A.rs.pairs_max);
     const RobotParams* rob;
-    if (outgrown || !collide_prologue<UNIFORM>(A, smem, L, sc0, n_obj4, &rob)) {
+    const int rid = T.robot, sid = UNIFORM ? 0 : T.scene;
+    const int64_t b0 = R.b_off[t];
+    const int B = (int)(R.b_off[t + 1] - b0);
+    const Bucket S = bucket_of(smem + keys_off, B > 0 ? B : 1);
+    WarpBufs Bf;
+    WarpRobot<SPL> W;
+    // the keys and the warps' robot load while the scene's copy is under way
+    auto meanwhile = [&] {
+        const int n = rob[rid].n;
+        for (int i = threadIdx.x; i < B; i += blockDim.x) S.key[i] = rank_key(R, t, b0, n, i, false);
+        Bf = warp_bufs(smem, L, A);
+        warp_robot<SPL>(A, rob, W, Bf, rid);
+    };
+    if (outgrown || !collide_prologue<UNIFORM>(A, smem, L, sc0, n_obj4, &rob, meanwhile)) {
         // no verdicts: no solutions (the error flag is set)
         const int tk = T.top_k & ~kNearestFlag, nj = A.rs.rp[T.robot].n;
         const RankOut O = rank_out(R, t, tk, nj);
@@ -516,24 +541,13 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_rank_lazy(const Collide
         if (threadIdx.x == 0) *O.count = 0;
         return;
     }
-    const WarpBufs Bf = warp_bufs(smem, L, A);
     const float4* s_scene = reinterpret_cast<const float4*>(smem);
-
-    const int rid = T.robot, sid = UNIFORM ? 0 : T.scene;
     const int n = rob[rid].n;
-    const int64_t b0 = R.b_off[t];
-    const int B = (int)(R.b_off[t + 1] - b0);
-    const Bucket S = bucket_of(smem + keys_off, B > 0 ? B : 1);
-    for (int i = threadIdx.x; i < B; i += blockDim.x) S.key[i] = rank_key(R, t, b0, n, i, false);
     __syncthreads();
     // candidates with a key (finite score); the ranks that may be visited below
     const int ranked = bucket_order(S, B, R.list ? depth + kWarpsPerBlock : B);
     const int top_k = T.top_k & ~kNearestFlag;
 
-    WarpRobot<SPL> W;
-    W.cur = -1;
-    W.n_m = W.pairs_m = 0;
-    W.bmask = 0;
     unsigned long long tests = 0, btests = 0, ncand = 0;
     if (threadIdx.x == 0) n_found = 0;
     __syncthreads();
@@ -689,7 +703,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, SPL <= 2 ? 3 : 2) k_colli
     }
     const CollideLayout L = collide_smem_layout(n_obj4, A.rs.n, A.rs.n_max + 2, A.rs.ns_max, A.rs.pairs_max);
     const RobotParams* rob;
-    if (!collide_prologue<true>(A, smem, L, sc0, n_obj4, &rob)) return;
+    if (!collide_prologue<true>(A, smem, L, sc0, n_obj4, &rob, [] {})) return;
     const WarpBufs Bf = warp_bufs(smem, L, A);
     const float4* const obj = reinterpret_cast<const float4*>(smem);
     const RobotParams& R = rob[0];
