@@ -713,6 +713,7 @@ __device__ __forceinline__ bool ccd_accept_ori(float gamma, const Q4 qerr, float
 template <bool RED, int N>
 __global__ void __launch_bounds__(kCoopMaxWarps * 32, 1) k_ccd_coop(const CcdArgs A) {
     extern __shared__ __align__(16) float sm[];
+    grid_follow();
     __shared__ long long s_base;
     const RobotParams* rob = stage_robots(sm, A.rs);
     const int WJ = ((int)blockDim.x >> 5) - 1;  // the warps that share the joints
@@ -1072,7 +1073,7 @@ void launch_ccd_coop_n(const CcdArgs& A, int warps, cudaStream_t st) {
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ccd_coop<RED, N>, 32 * warps, smem);
     const int g = (int)std::min<int64_t>((A.C + kCoopCands - 1) / kCoopCands, (int64_t)sm_count() * std::max(per_sm, 1));
-    k_ccd_coop<RED, N><<<g, 32 * warps, smem, st>>>(A);
+    launch_next<CcdArgs>(k_ccd_coop<RED, N>, g, 32 * warps, smem, st, A);
 }
 
 template <bool RED>

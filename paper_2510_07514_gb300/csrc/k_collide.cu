@@ -429,6 +429,7 @@ __device__ __forceinline__ WarpBufs warp_bufs(unsigned char* smem, const Collide
 template <int SPL, bool UNIFORM, bool GRID>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_collide(const CollideArgs A) {
     extern __shared__ __align__(128) unsigned char smem[];
+    grid_follow();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const SceneDev sc0 = A.n_scenes > 0 ? A.scenes[0] : SceneDev{nullptr, 0, 0};
     const int n_obj4 = UNIFORM ? sc0.n_sph + 2 * sc0.n_box : 0;
@@ -506,6 +507,7 @@ template <int SPL, bool UNIFORM, bool GRID>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_rank_lazy(const CollideArgs A, const RankArgs R,
                                                                   uint32_t keys_off, int depth) {
     extern __shared__ __align__(128) unsigned char smem[];
+    grid_follow();
     __shared__ int verdict[kWarpsPerBlock];
     __shared__ int picks[HJCD_MAX_TOPK];
     __shared__ int n_found;
@@ -618,7 +620,8 @@ bool launch_rank_lazy_t(const CollideArgs& A, const RankArgs& R, int n_obj4, int
     if (smem > 220 * 1024) return false;
     static SmemLimit lim;
     allow_dyn_smem(k_rank_lazy<SPL, UNIFORM, GRID>, lim, 220 * 1024);
-    k_rank_lazy<SPL, UNIFORM, GRID><<<R.T, kWarpsPerBlock * 32, smem, st>>>(A, R, keys_off, depth);
+    launch_next<CollideArgs, RankArgs, uint32_t, int>(k_rank_lazy<SPL, UNIFORM, GRID>, R.T, kWarpsPerBlock * 32, smem, st,
+                                                      A, R, keys_off, depth);
     return true;
 }
 
@@ -638,7 +641,7 @@ void launch_collide_t(const CollideArgs& A, int n_obj4, cudaStream_t st) {
     static SmemLimit lim;
     allow_dyn_smem(k_collide<SPL, UNIFORM, GRID>, lim, 227 * 1024);
     const int g = grid_for(A.C, kWarpsPerBlock, 8);
-    k_collide<SPL, UNIFORM, GRID><<<g, kWarpsPerBlock * 32, smem, st>>>(A);
+    launch_next<CollideArgs>(k_collide<SPL, UNIFORM, GRID>, g, kWarpsPerBlock * 32, smem, st, A);
 }
 
 template <bool UNIFORM, bool GRID>

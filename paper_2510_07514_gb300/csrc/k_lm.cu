@@ -875,6 +875,7 @@ __device__ __constant__ int8_t kTriCol[21] = {0, 0, 1, 0, 1, 2, 0, 1, 2, 3, 0, 1
 template <bool RED, int N, bool LIST>
 __global__ void __launch_bounds__(kCoopLmWarps * 32, 1) k_lm_coop(const LmArgs A) {
     extern __shared__ __align__(16) float smem_f[];
+    grid_follow();
     __shared__ float alphas[kCoopMaxA + 1];
     if (threadIdx.x == 0) ls_alphas(alphas, A.P.lm_A, A.P.lm_beta);  // visible after the staging barrier
     const RobotParams* rob = stage_robots(smem_f, A.rs);
@@ -1253,7 +1254,7 @@ void launch_lm_coop_n(const LmArgs& A, int warps, cudaStream_t st) {
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lm_coop<RED, N, LIST>, 32 * warps, smem);
     const int g = (int)std::min<int64_t>((A.C + kCoopCands - 1) / kCoopCands, (int64_t)sm_count() * std::max(per_sm, 1));
-    k_lm_coop<RED, N, LIST><<<g, 32 * warps, smem, st>>>(A);
+    launch_next<LmArgs>(k_lm_coop<RED, N, LIST>, g, 32 * warps, smem, st, A);
 }
 
 template <bool RED, bool LIST>

@@ -22,6 +22,7 @@ constexpr int kSelThreads = 512;
 // 20 -> 8.8 us, of 2000 seeds and 24 joints 60 -> 11 us, 1000 targets of 1000 seeds 75 -> 51 us.
 __global__ void __launch_bounds__(kSelThreads) k_topk_dup(const DupArgs A) {
     extern __shared__ __align__(16) unsigned char sel_smem[];
+    grid_follow();
     const int t = blockIdx.x;
     const int64_t m0 = A.m_off[t];
     const int M = (int)(A.m_off[t + 1] - m0);
@@ -56,6 +57,7 @@ __global__ void __launch_bounds__(kSelThreads) k_topk_dup(const DupArgs A) {
 
 __global__ void __launch_bounds__(kSelThreads) k_rank(const RankArgs A) {
     extern __shared__ __align__(16) unsigned char sel_smem[];
+    grid_follow();
     int t = blockIdx.x;
     if (A.list) {  // the targets the bounded lazy pass left unfinished
         if (t >= *A.n_list) return;
@@ -278,14 +280,14 @@ void launch_topk_dup(const DupArgs& A, int max_m, cudaStream_t st) {
     // slices of a target: enough CTAs for two per SM, each with at least one item per thread
     const int items = max_m * ((A.rs.n_max + 1) / 2);
     const int slices = std::max(1, std::min(2 * sm_count() / A.T, (items + kSelThreads - 1) / kSelThreads));
-    k_topk_dup<<<dim3(A.T, slices), kSelThreads, bucket_smem_bytes(max_m), st>>>(A);
+    launch_next<DupArgs>(k_topk_dup, dim3(A.T, slices), kSelThreads, bucket_smem_bytes(max_m), st, A);
 }
 
 void launch_rank(const RankArgs& A, int max_b, cudaStream_t st) {
     if (A.T <= 0) return;
     static SmemLimit lim;
     allow_dyn_smem(k_rank, lim, bucket_smem_bytes(HJCD_MAX_SAMPLES));
-    k_rank<<<A.T, kSelThreads, bucket_smem_bytes(max_b), st>>>(A);
+    launch_next<RankArgs>(k_rank, A.T, kSelThreads, bucket_smem_bytes(max_b), st, A);
 }
 
 void launch_shard_topk(const ShardTopkArgs& A, int max_m, cudaStream_t st) {
