@@ -502,15 +502,18 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_collide(const CollideAr
 // candidates in rank order, one candidate per warp and kWarpsPerBlock at a
 // time, until top_k collision-free ones are found or the ranked candidates
 // run out.  Same output as the collision filter over all candidates followed
-// by k_rank.
+// by k_rank.  A launch of few targets has CTAs of twice the warps, which check
+// the next kWarpsPerBlock candidates too in case the first do not settle it; what
+// they find counts only then.
+constexpr int kRankWarps = 2 * kWarpsPerBlock;
 template <int SPL, bool UNIFORM, bool GRID>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32) k_rank_lazy(const CollideArgs A, const RankArgs R,
+__global__ void __launch_bounds__(kRankWarps * 32) k_rank_lazy(const CollideArgs A, const RankArgs R,
                                                                   uint32_t keys_off, int depth) {
     extern __shared__ __align__(128) unsigned char smem[];
     grid_follow();
-    __shared__ int verdict[kWarpsPerBlock];
+    __shared__ int verdict[kRankWarps];
     __shared__ int picks[HJCD_MAX_TOPK];
-    __shared__ int n_found;
+    __shared__ int n_found, n_checked;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int t = blockIdx.x;
     const TargetDesc& T = R.tg[t];
@@ -554,28 +557,32 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_rank_lazy(const Collide
     if (threadIdx.x == 0) n_found = 0;
     __syncthreads();
     int p0 = 0;
-    for (; p0 < ranked && n_found < top_k && (!R.list || p0 < depth); p0 += kWarpsPerBlock) {
-        const int p = p0 + warp;
+    const int warps = (int)blockDim.x >> 5, limit = R.list ? min(ranked, depth) : ranked;
+    while (p0 < limit && n_found < top_k) {
+        const int p = p0 + warp, g0 = p0 + warp / kWarpsPerBlock * kWarpsPerBlock;  // its group's first
         bool hit = true;
-        if (p < ranked) {
+        unsigned long long t_s = 0, t_b = 0;
+        if (p < ranked && g0 < limit) {
             const int64_t c = b0 + S.order[p];
-            unsigned long long t_s = 0, t_b = 0;
             hit = warp_collides<SPL, UNIFORM, GRID>(A, rob, sc0, s_scene, W, Bf, c, rid, sid, t_s, t_b);
-            if (lane == 0) {
-                tests += t_s;
-                btests += t_b;
-                ++ncand;
-            }
         }
         if (lane == 0) verdict[warp] = hit ? 1 : 0;
         __syncthreads();
         if (threadIdx.x == 0) {
-            int f = n_found;
-            for (int w = 0; w < kWarpsPerBlock && f < top_k; ++w)
-                if (p0 + w < ranked && !verdict[w]) picks[f++] = p0 + w;
+            int f = n_found, g = p0;
+            for (; g < p0 + warps && g < limit && f < top_k; g += kWarpsPerBlock)
+                for (int q = g; q < g + kWarpsPerBlock && f < top_k; ++q)
+                    if (q < ranked && !verdict[q - p0]) picks[f++] = q;
             n_found = f;
+            n_checked = g;
         }
         __syncthreads();
+        if (lane == 0 && p < ranked && g0 < n_checked) {
+            tests += t_s;
+            btests += t_b;
+            ++ncand;
+        }
+        p0 = n_checked;
     }
     const int count = n_found;
     if (A.cnt && lane == 0) {
@@ -615,12 +622,19 @@ template <int SPL, bool UNIFORM, bool GRID>
 bool launch_rank_lazy_t(const CollideArgs& A, const RankArgs& R, int n_obj4, int max_b, int depth, cudaStream_t st) {
     const CollideLayout L =
         collide_smem_layout(UNIFORM ? n_obj4 : 0, A.rs.n, A.rs.n_max + 2, A.rs.ns_max, A.rs.pairs_max);
-    const uint32_t keys_off = (L.total + 15u) / 16u * 16u;
+    // Twice the warps while the targets leave the SMs room for them (two such CTAs each): a cluttered
+    // target's rounds are a chain that nothing else hides.  Ranking phase, us: 97 targets x 1000 in 220
+    // obstacles 87 -> 75, one target among 24 obstacles 30 -> 24; past that the SMs are full of CTAs.
+    const int cap = 220 * 1024;
+    auto keys_at = [&](int w) { return (L.total + (w - kWarpsPerBlock) * L.warp_bytes + 15u) / 16u * 16u; };
+    int warps = kRankWarps;
+    if (R.T > 2 * sm_count() || 2 * (keys_at(warps) + bucket_smem_bytes(max_b)) > (size_t)cap) warps = kWarpsPerBlock;
+    const uint32_t keys_off = keys_at(warps);
     const size_t smem = keys_off + bucket_smem_bytes(max_b);
-    if (smem > 220 * 1024) return false;
+    if (smem > (size_t)cap) return false;
     static SmemLimit lim;
-    allow_dyn_smem(k_rank_lazy<SPL, UNIFORM, GRID>, lim, 220 * 1024);
-    launch_next<CollideArgs, RankArgs, uint32_t, int>(k_rank_lazy<SPL, UNIFORM, GRID>, R.T, kWarpsPerBlock * 32, smem, st,
+    allow_dyn_smem(k_rank_lazy<SPL, UNIFORM, GRID>, lim, cap);
+    launch_next<CollideArgs, RankArgs, uint32_t, int>(k_rank_lazy<SPL, UNIFORM, GRID>, R.T, warps * 32, smem, st,
                                                       A, R, keys_off, depth);
     return true;
 }

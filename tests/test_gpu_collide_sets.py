@@ -71,3 +71,19 @@ def test_large_sets_give_the_verdicts_of_small_ones(ctx, which, kind):
     for a, b in ((0, 11000), (11000, 22000), (22000, BIG)):
         assert torch.equal(ctx.collide(rid, sid, th[:, a:b].contiguous()), big[a:b])
     assert set(big.unique().tolist()) <= {0, 1}
+
+
+@pytest.mark.parametrize("top_k,boxes", [(1, 20), (3, 0), (16, 20)])
+def test_ranking_of_few_targets_equals_that_of_many(ctx, top_k, boxes):
+    """The collision-aware ranking takes CTAs of twice the warps for few targets; a target's index
+    keys its random streams, so the first ones of a long list are the same solves."""
+    rng = np.random.default_rng(40 + top_k)
+    rob = inputs.panda()
+    scene = inputs.random_scene(rng, 200, boxes)
+    rid, sid = ctx.add_robot(rob), ctx.set_scene(scene)
+    tg = ctx.fk(rid, torch.as_tensor(inputs.joint_samples(rng, rob, 400).T.copy(), dtype=torch.float32, device="cuda"))
+    many = ctx.solve(rid, sid, tg, 128, top_k, 3, rob.n)
+    for T in (1, 2, 97):
+        few = ctx.solve(rid, sid, tg[:T].contiguous(), 128, top_k, 3, rob.n)
+        for x, y in zip(few, many):
+            assert torch.equal(x.view(torch.int32), y[:T].view(torch.int32))
