@@ -211,9 +211,11 @@ void hjcd_graph_destroy(hjcd_graph* graph);
 /* ---- launch configuration and autotuning --------------------------------------- */
 
 /* Candidates per CTA of the PO-CCD kernel (64, 128 or 256; default 64) and
- * warps per CTA of the PJ-IK kernel (2, 4 or 8; default 8) for every later
- * launch of the context; launches of at most 64 candidates per SM take kernels
- * of their own, which have a fixed configuration.  Results do not depend on them. */
+ * most warps per CTA of the PJ-IK kernel (2, 4 or 8; default 8; fewer are taken
+ * where more warps then fit an SM) for every later launch of the context;
+ * launches of at most 64 candidates per SM, and the later PJ-IK iterations of
+ * up to 216, may take kernels of their own with a fixed configuration.  Results
+ * do not depend on them. */
 hjcd_status hjcd_set_launch_config(hjcd_ctx* ctx, int32_t ccd_block, int32_t lm_warps);
 
 typedef struct hjcd_tune_report {

@@ -549,9 +549,9 @@ __global__ void __launch_bounds__(TH, HJCD_CCD_THREADS_PER_SM / TH) k_ccd(const 
 //      the others draw the perturbation that the lanes about to reject will need
 //   5. every half warp: the accepted update or the perturbation of its joints, their sines and cosines
 // The arithmetic is ccd_step's, operation by operation, so the results are its bits.  Bound by
-// latency: about 3000 cycles per iteration on Panda (kinematics rows 500, residual 890, trials 460,
-// choice and acceptance 550, update 450, the barriers the rest).  One target of 1000 seeds: 55 us for
-// at most 32 iterations, where k_ccd takes 125 us.
+// latency: about 2800 cycles per iteration on Panda (kinematics rows 370, residual 760, trials 475,
+// choice and acceptance 525, update 345, the barriers the rest).  One target of 1000 seeds: 45 us for
+// at most 32 iterations, where k_ccd takes 119 us (kernel times).
 constexpr int kCoopCands = 16;     // candidates per CTA
 constexpr int kCoopMaxWarps = 16;  // joint warps and the residual's
 

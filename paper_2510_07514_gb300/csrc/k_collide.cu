@@ -622,16 +622,17 @@ template <int SPL, bool UNIFORM, bool GRID>
 bool launch_rank_lazy_t(const CollideArgs& A, const RankArgs& R, int n_obj4, int max_b, int depth, cudaStream_t st) {
     const CollideLayout L =
         collide_smem_layout(UNIFORM ? n_obj4 : 0, A.rs.n, A.rs.n_max + 2, A.rs.ns_max, A.rs.pairs_max);
-    // Twice the warps while the targets leave the SMs room for them (two such CTAs each): a cluttered
-    // target's rounds are a chain that nothing else hides.  Ranking phase, us: 97 targets x 1000 in 220
-    // obstacles 87 -> 75, one target among 24 obstacles 30 -> 24; past that the SMs are full of CTAs.
-    const int cap = 220 * 1024;
+    // Twice the warps while the targets leave the SMs room for them (at most two such CTAs each): a
+    // cluttered target's rounds are a chain that nothing else hides.  Ranking phase, us: 97 targets x 1000
+    // in 220 obstacles 87 -> 75, one target among 24 obstacles 30 -> 24; past that the SMs are full of CTAs.
+    const size_t cap = 220 * 1024;
     auto keys_at = [&](int w) { return (L.total + (w - kWarpsPerBlock) * L.warp_bytes + 15u) / 16u * 16u; };
-    int warps = kRankWarps;
-    if (R.T > 2 * sm_count() || 2 * (keys_at(warps) + bucket_smem_bytes(max_b)) > (size_t)cap) warps = kWarpsPerBlock;
+    const int64_t per_sm = (R.T + sm_count() - 1) / sm_count();
+    const bool room = per_sm <= 2 && per_sm * (keys_at(kRankWarps) + bucket_smem_bytes(max_b)) <= cap;
+    const int warps = room ? kRankWarps : kWarpsPerBlock;
     const uint32_t keys_off = keys_at(warps);
     const size_t smem = keys_off + bucket_smem_bytes(max_b);
-    if (smem > (size_t)cap) return false;
+    if (smem > cap) return false;
     static SmemLimit lim;
     allow_dyn_smem(k_rank_lazy<SPL, UNIFORM, GRID>, lim, cap);
     launch_next<CollideArgs, RankArgs, uint32_t, int>(k_rank_lazy<SPL, UNIFORM, GRID>, R.T, warps * 32, smem, st,
