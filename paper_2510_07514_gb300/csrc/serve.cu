@@ -94,8 +94,9 @@ namespace {
 // waiting: requests that arrive closely together then share one launch sequence, whose time is
 // mostly the latency of its longest candidate, instead of each taking a slot of its own, while a
 // lone request, or a queue that can fill the GPU, is launched at once.  A burst of 20 requests (1 to 8
-// targets each): 1.95 ms against 2.20 without the pace; a Poisson trace at 2000 requests/s: p50 0.56
-// against 0.44 ms, p99 1.42 against 1.35 ms, at 4000/s p99 1.70 against 1.69 ms.
+// targets each): 1.69 ms against 1.76 without the pace; a Poisson trace at 2000 requests/s: p50 0.46
+// against 0.36 ms, p99 1.16 against 1.12 ms (1.28 and 1.10 requests per wave); at 4000/s p99 1.52
+// against 1.56 ms, at 8000/s 2.30 against 2.29 ms.
 constexpr std::chrono::microseconds kPace(250);
 constexpr int64_t kFillSeeds = 64;
 
