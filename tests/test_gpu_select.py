@@ -9,7 +9,7 @@ from paper_2510_07514_gb300 import api, build, hjcd, inputs
 
 pytestmark = pytest.mark.gpu
 
-SIZES = [1, 2, 31, 32, 33, 64, 1000, 1024, 1025, 2048, 2049, 8191, 8192]
+SIZES = [1, 2, 31, 32, 33, 64, 127, 128, 129, 1000, 1024, 1025, 2048, 2049, 8191, 8192]
 
 
 @pytest.fixture(scope="module")
