@@ -578,7 +578,8 @@ __device__ __forceinline__ uint32_t score_bits(float s) {
 
 // Up to this many keys are ranked by counting, without the bucket pass' seven barriers (64 keys: the
 // selection and the ranking of a solve 1.5 us less each, end to end 125 -> 122 us; the comparisons
-// grow with the square, and at 256 keys they are the longer way).
+// grow with the square, and at 256 keys they are the longer way).  COUNT = false leaves that out, for
+// the collision-aware ranking, whose registers it takes past 80 and so a third CTA off each SM.
 constexpr int kCountKeys = 128;
 
 // bins of a pass over M keys
@@ -614,9 +615,10 @@ __device__ __forceinline__ Bucket bucket_of(void* smem, int M) {
 // B.order[r] for r < min(want, returned) from B.key[0, M) (visible to the whole CTA when it is
 // called); returns the number of keys other than kNoKey32.  All threads of the CTA take part
 // (a multiple of 32, at most 1024); ends with a barrier.
+template <bool COUNT = true>
 __device__ __forceinline__ int bucket_order(const Bucket& B, int M, int want) {
     const int tid = threadIdx.x, nth = blockDim.x, lane = tid & 31, warp = tid >> 5;
-    if (M <= kCountKeys) {  // every key against every other, four threads a key
+    if (COUNT && M <= kCountKeys) {  // every key against every other, four threads a key
         int valid = 0;
         for (int i0 = 0; i0 < max(M, 1); i0 += nth / 4) {
             const int i = i0 + tid / 4;

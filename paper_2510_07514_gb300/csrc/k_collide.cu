@@ -550,7 +550,7 @@ __global__ void __launch_bounds__(kRankWarps * 32) k_rank_lazy(const CollideArgs
     const int n = rob[rid].n;
     __syncthreads();
     // candidates with a key (finite score); the ranks that may be visited below
-    const int ranked = bucket_order(S, B, R.list ? depth + kWarpsPerBlock : B);
+    const int ranked = bucket_order<false>(S, B, R.list ? depth + kWarpsPerBlock : B);
     const int top_k = T.top_k & ~kNearestFlag;
 
     unsigned long long tests = 0, btests = 0, ncand = 0;
