@@ -170,8 +170,8 @@ __device__ __forceinline__ void warp_robot(const CollideArgs& A, const RobotPara
 }
 
 // Collision verdict of candidate c (robot row rid, scene row sid, -1: none),
-// warp-uniform; t_s / t_b accumulate the sphere and box tests.  SELF: the self-collision part only.
-template <int SPL, bool UNIFORM, bool GRID, bool SELF = false>
+// warp-uniform; t_s / t_b accumulate the sphere and box tests.
+template <int SPL, bool UNIFORM, bool GRID>
 __device__ __forceinline__ bool warp_collides(const CollideArgs& A, const RobotParams* rob, const SceneDev& sc0,
                                               const float4* s_scene, WarpRobot<SPL>& W, const WarpBufs& Bf, int64_t c,
                                               int rid, int sid, unsigned long long& t_s, unsigned long long& t_b) {
@@ -189,8 +189,7 @@ __device__ __forceinline__ bool warp_collides(const CollideArgs& A, const RobotP
     // obstacles: the staged copy (shared memory) or the scene's table (global, read-only path)
     const float4* obj = s_scene;
     int n_osph = 0, n_obox = 0;
-    if (SELF) {
-    } else if (UNIFORM) {
+    if (UNIFORM) {
         n_osph = A.u_osph;
         n_obox = A.u_obox;
     } else if (sid >= 0) {
@@ -678,14 +677,20 @@ void launch_collide_s(const CollideArgs& A, int n_obj4, cudaStream_t st) {
 // set where the obstacle can touch a bounding sphere centred in the cell (a margin covers the
 // rounding of the cell index).  The obstacles that overlap the body's bounding sphere go to a
 // lane's list and are then tested against the body's link spheres.  Pairs of bodies are tested by lane
-// as well, bounding sphere against bounding sphere and then against the later body's link spheres;
-// the few candidates that have such a pair get the warp routine's self test.  The tests that decide are the other kernel's, on the same spheres, so the verdicts are
-// equal.  Bound by issue, mostly the walk over near obstacles, whose counts differ between lanes.
-// 400k Panda configurations, 60 link spheres, 220 obstacles (27% free): 332 us, where a warp per
+// as well: bounding sphere against bounding sphere, the later body's link spheres against the earlier
+// one's bounding sphere, and where both overlap link sphere against link sphere, for which the warp
+// walks the chain again up to the earlier body (its frames would not fit shared memory).  The tests
+// that decide are the other kernel's, on the same spheres, so the verdicts are equal.  Bound by issue,
+// mostly the walk over near obstacles, whose counts differ between lanes.  With a whole warp on each
+// candidate that has such a pair, a chain whose bodies crowd one another gained nothing (200k
+// candidates without obstacles, link sphere tests by warp / by lane, us: Panda 111 / 86, 12 joints
+// 583 / 433, 20 joints 2115 / 933; a warp per candidate from the start 228, 612 and 1258).
+// 400k Panda configurations, 60 link spheres, 220 obstacles (27% free): 307 us, where a warp per
 // candidate takes 835 us.
 constexpr int kCells = 6;           // per axis
 constexpr int kLaneList = 12;       // overlapping obstacles a lane holds before it tests them
-constexpr int64_t kLaneMinCands = 32768;
+constexpr int64_t kLaneMinCands = 32768, kLaneMinCandsLong = 49152;
+constexpr int kLaneLong = 8, kLaneFewObjs = 64;  // joints above and obstacles below which the latter counts
 constexpr int kLaneMaxWords = 16;   // obstacles: 32 per word of a cell's mask, spheres and boxes in words of their own
 static_assert(kCells * kCells * kCells <= kWarpsPerBlock * 32, "a cell per thread");
 constexpr float kSmallBody = 0.6f;  // bounding radii up to this part of the largest have masks of their own
@@ -706,8 +711,8 @@ __host__ __device__ __forceinline__ LaneLayout lane_layout(uint32_t from, int ns
     return L;
 }
 
-template <int SPL>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32, SPL <= 2 ? 3 : 2) k_collide_lane(const CollideArgs A) {
+template <int PER_SM>
+__global__ void __launch_bounds__(kWarpsPerBlock * 32, PER_SM) k_collide_lane(const CollideArgs A) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ float s_lo[3], s_inv[3];
     __shared__ uint32_t s_pair[kMaxBodies];  // bit a of entry b: bodies a < b are checked for self-collision
@@ -719,16 +724,15 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, SPL <= 2 ? 3 : 2) k_colli
         if (tid == 0) *(volatile int32_t*)A.err_flag = 2;
         return;
     }
-    const CollideLayout L = collide_smem_layout(n_obj4, A.rs.n, A.rs.n_max + 2, A.rs.ns_max, A.rs.pairs_max);
+    const CollideLayout L = collide_smem_layout(n_obj4, A.rs.n, 0, 0, 0);
     const RobotParams* rob;
     if (!collide_prologue<true>(A, smem, L, sc0, n_obj4, &rob, [] {})) return;
-    const WarpBufs Bf = warp_bufs(smem, L, A);
     const float4* const obj = reinterpret_cast<const float4*>(smem);
     const RobotParams& R = rob[0];
     const int n = A.u_n, nb = n + 2, n_pairs = A.u_pairs, n_osph = A.u_osph, n_obox = A.u_obox;
     const int w_sph = (n_osph + 31) / 32, words = w_sph + (n_obox + 31) / 32;
     const RobotDev rd = A.rs.rd[0];
-    const LaneLayout M = lane_layout(L.total, A.rs.ns_max, nb, words);
+    const LaneLayout M = lane_layout(L.warp, A.rs.ns_max, nb, words);
     float4* const lsph = reinterpret_cast<float4*>(smem + M.sph);
     float4* const lco = reinterpret_cast<float4*>(smem + M.co);
     int2* const lrange = reinterpret_cast<int2*>(smem + M.range);
@@ -822,7 +826,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, SPL <= 2 ? 3 : 2) k_colli
     for (int64_t c0 = 32 * ((int64_t)blockIdx.x * kWarpsPerBlock + warp); c0 < A.C; c0 += 32 * nwarps) {
         const int64_t c = c0 + lane;
         const bool have = c < A.C;
-        bool hit = !have, need = false;  // need: a pair of bodies that the warp has to test
+        bool hit = !have;
         unsigned t_s = 0, t_b = 0;
 
         // one body at frame F: its bounding sphere's centre, then the obstacles near it
@@ -897,45 +901,64 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, SPL <= 2 ? 3 : 2) k_colli
                      });
             }
             // earlier bodies whose bounding sphere overlaps this one's and one of its link spheres
-            for (uint32_t m = s_pair[b]; m && !hit && !need; m &= m - 1u) {
+            auto bound = [&](int a) {
+                return make_float4(cc[(3 * a) * 32], cc[(3 * a + 1) * 32], cc[(3 * a + 2) * 32], lco[a].w);
+            };
+            uint32_t pairs = 0;
+            for (uint32_t m = s_pair[b]; m && !hit; m &= m - 1u) {
                 const int a = __ffs(m) - 1;
-                const float4 ca = make_float4(cc[(3 * a) * 32], cc[(3 * a + 1) * 32], cc[(3 * a + 2) * 32], lco[a].w);
+                const float4 ca = bound(a);
                 ++t_s;
                 if (sph_sph(ca, co)) {
+                    bool o = false;
                     t_s += rg.y;
 #pragma unroll 4
-                    for (int i = rg.x; i < rg.x + rg.y; ++i) need |= sph_sph(to_world(F, lsph[i]), ca);
+                    for (int i = rg.x; i < rg.x + rg.y; ++i) o |= sph_sph(to_world(F, lsph[i]), ca);
+                    pairs |= o ? 1u << a : 0u;
                 }
+            }
+            // their link spheres against this body's: the chain is walked again up to the last of them
+            uint32_t left = __reduce_or_sync(0xffffffffu, pairs);
+            Frame G = frame_identity();
+#pragma unroll 1
+            for (int a = 0; left; ++a) {
+                if (a > 0) fk_step(R, a - 1, have ? A.th[(a - 1) * A.ld + c] : 0.0f, G);
+                if (!(left >> a & 1u)) continue;
+                if (pairs >> a & 1u) {
+                    const int2 ra = lrange[a];
+                    const float4 ca = bound(a);
+#pragma unroll 1
+                    for (int i = rg.x; i < rg.x + rg.y && !hit; ++i) {
+                        const float4 wb = to_world(F, lsph[i]);
+                        if (!sph_sph(wb, ca)) continue;
+                        t_s += ra.y;
+#pragma unroll 4
+                        for (int k = ra.x; k < ra.x + ra.y; ++k) hit |= sph_sph(to_world(G, lsph[k]), wb);
+                    }
+                    t_s += rg.y;
+                }
+                pairs = hit ? 0u : pairs & ~(1u << a);
+                left = __reduce_or_sync(0xffffffffu, pairs);
             }
         };
 
         Frame F = frame_identity();
-        body(0, F);
+        float theta = have ? A.th[c] : 0.0f;  // the next joint's, loaded a body ahead
 #pragma unroll 1
-        for (int j = 0; j < n; ++j) {
-            fk_step(R, j, have ? A.th[j * A.ld + c] : 0.0f, F);
-            body(j + 1, F);
-        }
-        body(n + 1, fk_flange(R, F));
-
-        // self-collision of the candidates that have such a pair
-        need = need && !hit;
-        unsigned long long ws_ = 0, wb_ = 0;
-        for (unsigned m = __ballot_sync(0xffffffffu, need); m; m &= m - 1u) {
-            const int src = __ffs(m) - 1;
-            WarpRobot<SPL> W;  // loaded for each such candidate: kept, it would cost every lane's walk registers
-            W.cur = -1;
-            W.n_m = W.pairs_m = 0;
-            W.bmask = 0;
-            const bool h = warp_collides<SPL, true, false, true>(A, rob, sc0, obj, W, Bf, c0 + src, 0, -1, ws_, wb_);
-            if (lane == src) hit = h;
-            __syncwarp();
+        for (int b = 0; b < nb; ++b) {  // (one copy of the body's code)
+            if (b > n) {
+                F = fk_flange(R, F);
+            } else if (b > 0) {
+                fk_step(R, b - 1, theta, F);
+                if (b < n && have) theta = A.th[b * A.ld + c];
+            }
+            body(b, F);
         }
         if (have) {
             A.hit[c] = hit ? 1 : 0;
             ++ncand;
         }
-        tests += t_s + (lane == 0 ? ws_ : 0ull);
+        tests += t_s;
         btests += t_b;
     }
     if (A.cnt) {
@@ -950,28 +973,33 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, SPL <= 2 ? 3 : 2) k_colli
     }
 }
 
-template <int SPL>
-bool launch_collide_lane_t(const CollideArgs& A, cudaStream_t st) {
-    const int words = (A.u_osph + 31) / 32 + (A.u_obox + 31) / 32;
-    const CollideLayout L =
-        collide_smem_layout(A.u_osph + 2 * A.u_obox, A.rs.n, A.rs.n_max + 2, A.rs.ns_max, A.rs.pairs_max);
-    const size_t smem = lane_layout(L.total, A.rs.ns_max, A.u_n + 2, words).total;
-    if (smem > 220 * 1024) return false;
+template <int PER_SM>
+int lane_ctas(size_t smem) {  // resident CTAs per SM
     static SmemLimit lim;
-    allow_dyn_smem(k_collide_lane<SPL>, lim, 220 * 1024);
+    allow_dyn_smem(k_collide_lane<PER_SM>, lim, 220 * 1024);
     int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_collide_lane<SPL>, kWarpsPerBlock * 32, smem);
-    const int g = grid_for(A.C, kWarpsPerBlock * 32, std::max(per_sm, 1));
-    k_collide_lane<SPL><<<g, kWarpsPerBlock * 32, smem, st>>>(A);
-    return true;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_collide_lane<PER_SM>, kWarpsPerBlock * 32, smem);
+    return std::max(per_sm, 1);
 }
 
 bool launch_collide_lane(const CollideArgs& A, cudaStream_t st) {
-    const int ns = A.rs.ns_max;
-    if (ns <= 32) return launch_collide_lane_t<1>(A, st);
-    if (ns <= 64) return launch_collide_lane_t<2>(A, st);
-    if (ns <= 128) return launch_collide_lane_t<4>(A, st);
-    return launch_collide_lane_t<8>(A, st);
+    const int words = (A.u_osph + 31) / 32 + (A.u_obox + 31) / 32;
+    const CollideLayout L = collide_smem_layout(A.u_osph + 2 * A.u_obox, A.rs.n, 0, 0, 0);
+    const size_t smem = lane_layout(L.warp, A.rs.ns_max, A.u_n + 2, words).total;
+    if (smem > 220 * 1024) return false;
+    constexpr int kThreads = kWarpsPerBlock * 32;
+    // Four CTAs per SM (64 registers, a few spilled) for a short chain and more candidates than three
+    // hold at once, else three (80): 400k Panda configurations among 220 obstacles 351 -> 343 us, 200k of 6
+    // joints among 110 218 -> 210; 100k of them 140 -> 145, 200k of 20 joints without obstacles 940 -> 1031.
+    if (A.u_n <= kLaneLong && A.C > (int64_t)sm_count() * 3 * kThreads) {
+        const int per_sm = lane_ctas<4>(smem);
+        if (per_sm > 3) {
+            k_collide_lane<4><<<grid_for(A.C, kThreads, per_sm), kThreads, smem, st>>>(A);
+            return true;
+        }
+    }
+    k_collide_lane<3><<<grid_for(A.C, kThreads, lane_ctas<3>(smem)), kThreads, smem, st>>>(A);
+    return true;
 }
 
 constexpr int kContactTile = 8;  // configurations per CTA of the contact kernel
@@ -1046,11 +1074,14 @@ void launch_collide(const CollideArgs& A, cudaStream_t st) {
     const bool uni = A.uniform && A.rs.n == 1 && A.n_scenes <= 1 && A.max_obj4 <= kMaxStagedObj4;
     const int n4 = A.n_scenes == 1 ? A.max_obj4 : 0;
     // From 32768 candidates on, a candidate per lane: below, its 32 candidates per warp leave the GPU
-    // underfilled.  Time, us, by lane / by warp: Panda with 60 spheres among 220 obstacles 16000: 100 / 74,
-    // 32000: 106 / 111, 100000: 143 / 260, 400000: 332 / 832; without obstacles 32000: 70 / 67, 400000:
-    // 157 / 414; a 20-joint chain with 189 spheres among 110: 32000: 250 / 322, 400000: 1500 / 2925.
+    // underfilled; from 49152 on for a long chain among few obstacles, whose time is the pairs' tests and
+    // their latency.  us, by lane / by warp: Panda with 60 spheres, 32768 candidates: no obstacles 53 / 66,
+    // 110: 80 / 100; 6 joints, 73 spheres: 54 / 90, 92 / 146; 12 joints, 127 spheres: 154 / 134, 20 obstacles
+    // 166 / 149, 110: 167 / 193; 20 joints, 197 spheres: 307 / 265, 295 / 286, 251 / 323, and at 49152
+    // 12 joints 179 / 180, 20 joints 385 / 367, 110 obstacles 269 / 454.
     const int words = (A.u_osph + 31) / 32 + (A.u_obox + 31) / 32;
-    if (uni && !A.has_grid && !A.list && words <= kLaneMaxWords && A.C >= kLaneMinCands && launch_collide_lane(A, st)) return;
+    const int64_t from = A.u_n > kLaneLong && A.u_osph + A.u_obox < kLaneFewObjs ? kLaneMinCandsLong : kLaneMinCands;
+    if (uni && !A.has_grid && !A.list && words <= kLaneMaxWords && A.C >= from && launch_collide_lane(A, st)) return;
     if (uni && A.has_grid) launch_collide_s<true, true>(A, n4, st);
     else if (uni) launch_collide_s<true, false>(A, n4, st);
     else if (A.has_grid) launch_collide_s<false, true>(A, 0, st);
