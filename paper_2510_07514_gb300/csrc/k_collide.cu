@@ -675,7 +675,7 @@ void launch_collide_s(const CollideArgs& A, int n_obj4, cudaStream_t st) {
 // comes up, against the obstacles near it only: every CTA cuts the box that holds the obstacles,
 // grown by the largest bounding radius, into 6 x 6 x 6 cells and keeps a bit per cell and obstacle,
 // set where the obstacle can touch a bounding sphere centred in the cell (a margin covers the
-// rounding of the cell index).  The obstacles that overlap the body's bounding sphere go to a
+// rounding of the cell index and of the coordinates, which may be large against a cell).  The obstacles that overlap the body's bounding sphere go to a
 // lane's list and are then tested against the body's link spheres.  Pairs of bodies are tested by lane
 // as well: bounding sphere against bounding sphere, the later body's link spheres against the earlier
 // one's bounding sphere, and where both overlap link sphere against link sphere, for which the warp
@@ -694,6 +694,7 @@ constexpr int kLaneLong = 8, kLaneFewObjs = 64;  // joints above and obstacles b
 constexpr int kLaneMaxWords = 16;   // obstacles: 32 per word of a cell's mask, spheres and boxes in words of their own
 static_assert(kCells * kCells * kCells <= kWarpsPerBlock * 32, "a cell per thread");
 constexpr float kSmallBody = 0.6f;  // bounding radii up to this part of the largest have masks of their own
+constexpr float kFewUlps = 4e-7f, kSomeUlps = 1e-6f;  // of a coordinate: the margins for its rounding
 
 struct LaneLayout {
     uint32_t sph, co, range, mask, warp, warp_bytes, total;
@@ -777,7 +778,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, PER_SM) k_collide_lane(co
             a = fminf(a, __shfl_xor_sync(0xffffffffu, a, d));
             e = fmaxf(e, __shfl_xor_sync(0xffffffffu, e, d));
         }
-        const float grow = rmax + 1e-3f * (e - a + rmax);
+        const float grow = rmax + 1e-3f * (e - a + rmax) + kFewUlps * fmaxf(fabsf(a), fabsf(e));
         lo[k] = a - grow;
         hi[k] = e + grow;
     }
@@ -797,8 +798,9 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, PER_SM) k_collide_lane(co
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             const float h = (hi[k] - lo[k]) / (float)kCells;
-            a[k] = lo[k] + h * ((float)ix[k] - 1e-3f);
-            e[k] = lo[k] + h * ((float)ix[k] + 1.001f);
+            const float round = kFewUlps * fmaxf(fabsf(lo[k]), fabsf(hi[k]));
+            a[k] = lo[k] + h * ((float)ix[k] - 1e-3f) - round;
+            e[k] = lo[k] + h * ((float)ix[k] + 1.001f) + round;
         }
         for (int w = 0; w < words; ++w) {
             uint32_t m = 0, ms = 0;
@@ -904,16 +906,21 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, PER_SM) k_collide_lane(co
             auto bound = [&](int a) {
                 return make_float4(cc[(3 * a) * 32], cc[(3 * a + 1) * 32], cc[(3 * a + 2) * 32], lco[a].w);
             };
+            auto widen = [](float4 s) {  // a test against it only saves work, and must not miss by rounding
+                s.w += kSomeUlps * (fabsf(s.x) + fabsf(s.y) + fabsf(s.z));
+                return s;
+            };
             uint32_t pairs = 0;
             for (uint32_t m = s_pair[b]; m && !hit; m &= m - 1u) {
                 const int a = __ffs(m) - 1;
                 const float4 ca = bound(a);
                 ++t_s;
                 if (sph_sph(ca, co)) {
+                    const float4 cw = widen(ca);
                     bool o = false;
                     t_s += rg.y;
 #pragma unroll 4
-                    for (int i = rg.x; i < rg.x + rg.y; ++i) o |= sph_sph(to_world(F, lsph[i]), ca);
+                    for (int i = rg.x; i < rg.x + rg.y; ++i) o |= sph_sph(to_world(F, lsph[i]), cw);
                     pairs |= o ? 1u << a : 0u;
                 }
             }
@@ -926,7 +933,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, PER_SM) k_collide_lane(co
                 if (!(left >> a & 1u)) continue;
                 if (pairs >> a & 1u) {
                     const int2 ra = lrange[a];
-                    const float4 ca = bound(a);
+                    const float4 ca = widen(bound(a));
 #pragma unroll 1
                     for (int i = rg.x; i < rg.x + rg.y && !hit; ++i) {
                         const float4 wb = to_world(F, lsph[i]);
