@@ -564,10 +564,17 @@ inline int grid_for(int64_t items, int per_block, int per_sm = 64) {
 // keys is found by one bucket pass in shared memory: the keys' range is cut into up to kMaxBins
 // equal bins, the candidates are gathered by bin, and a candidate's rank is its bin's start plus
 // its rank among the few that share the bin.  The work is linear while the bins are short (a
-// whole sort of 1024 keys took 55 barriers, this takes eight); keys that crowd one bin cost
-// their square, which only equal scores reach.  The ranked filter's time with its sort -> with this:
-// one target of 1000 candidates 27 -> 21 us, 1000 targets 153 -> 119 us, 2000 targets of 4096
-// candidates 1281 -> 824 us.
+// whole sort of 1024 keys took 55 barriers, this takes eight).  The ranked filter's time with its
+// sort -> with this: one target of 1000 candidates 27 -> 21 us, 1000 targets 153 -> 119 us, 2000
+// targets of 4096 candidates 1281 -> 824 us.
+//
+// Keys that crowd a bin would cost their square: equal scores (every seed of an invalid target scores
+// infinity, so a padding row of a batch does that), a few distinct ones, or scores squeezed together by
+// keys far away.  The bins therefore span the ordinary keys only (finite and non-negative; not the NaN
+// of the top-K, not the ranking's class 1) where those hold every wanted rank, and a pass that finds more
+// than kCrowd keys in a bin with a wanted rank leaves the order to a radix sort.  The top quarter of 8192
+// scores, 600 targets: spread 445 us, all equal 268 (by their square 9460), 20% NaN 451; all of them in
+// order: 397, 308, 511.  16 targets of 8192 seeds, eight of them padding rows: a solve 5340 -> 684 us.
 
 constexpr uint32_t kNoKey32 = 0xffffffffu;  // never ranked
 constexpr int kMaxBins = 2048;
@@ -581,6 +588,8 @@ __device__ __forceinline__ uint32_t score_bits(float s) {
 // grow with the square, and at 256 keys they are the longer way).  COUNT = false leaves that out, for
 // the collision-aware ranking, whose registers it takes past 80 and so a third CTA off each SM.
 constexpr int kCountKeys = 128;
+constexpr int kCrowd = 128;  // more are sorted: 128 in every bin take about as long as the sort
+constexpr uint32_t kOrdinary = 0x7f800000u;  // keys below are finite non-negative scores (of class 0)
 
 // bins of a pass over M keys
 __host__ __device__ __forceinline__ int bucket_bins(int M) {
@@ -612,6 +621,91 @@ __device__ __forceinline__ Bucket bucket_of(void* smem, int M) {
     return B;
 }
 
+// The crowded case of bucket_order: a radix sort of the `valid` candidates with a key, by
+// min(key - lo, top) and then index.  Each pass takes a digit; a warp ranks its contiguous part of the
+// sequence 32 at a time by matching digits, so the order is stable and the time does not depend on
+// the keys.  (Digits of up to 8 bits, as the warps' counts fit the bins' memory; equal keys take one
+// pass.)  Not inlined: it is rarely taken, and the callers' registers and code stay as they are.
+__device__ __forceinline__ void bucket_sort(const Bucket B, int M, int valid, uint32_t lo, uint32_t top) {
+    const int tid = threadIdx.x, nth = blockDim.x, lane = tid & 31, warp = tid >> 5, W = nth >> 5;
+    int D = 8;
+    while ((W << D) > 2 * B.bins || (1 << D) > nth) --D;
+    const int R = 1 << D, span = 32 - __clz(top);
+    uint16_t* const mine = reinterpret_cast<uint16_t*>(B.bin) + warp * R;  // [warp][digit]
+    uint16_t *src = B.slot, *dst = B.order;
+    int shift = 0;
+    do {
+        const bool first = shift == 0;  // the candidates in index order, those without a key left out
+        const int n = first ? M : valid;
+        const int part = ((n + W - 1) / W + 31) & ~31, p0 = min(n, warp * part), p1 = min(n, p0 + part);
+        // this lane's candidate at p and its digit (R: none)
+        auto digit = [&](int p, int& cand) {
+            cand = p < p1 ? (first ? p : (int)src[p]) : 0;
+            const uint32_t k = p < p1 ? B.key[cand] : kNoKey32;
+            return k != kNoKey32 ? (int)(min(k - lo, top) >> shift & (uint32_t)(R - 1)) : R;
+        };
+        __syncthreads();
+#pragma unroll 1
+        for (int i = tid; i < W * R; i += nth) reinterpret_cast<uint16_t*>(B.bin)[i] = 0;
+        __syncthreads();
+#pragma unroll 1
+        for (int p = p0 + lane; p - lane < p1; p += 32) {
+            int cand;
+            const int d = digit(p, cand);
+            const unsigned peers = __match_any_sync(0xffffffffu, d);
+            if (d < R && lane == __ffs(peers) - 1) mine[d] += (uint16_t)__popc(peers);
+            __syncwarp();
+        }
+        __syncthreads();
+        // where each warp's candidates of a digit begin
+        uint16_t* const col = reinterpret_cast<uint16_t*>(B.bin) + tid;
+        uint32_t sum = 0;
+        if (tid < R)
+#pragma unroll 1
+            for (int w = 0; w < W; ++w) {
+                const uint32_t v = col[w * R];
+                col[w * R] = (uint16_t)sum;
+                sum += v;
+            }
+        uint32_t inc = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += v;
+        }
+        if (lane == 31) B.tmp[warp] = inc;
+        __syncthreads();
+        uint32_t at = inc - sum;
+#pragma unroll 1
+        for (int w = 0; w < warp; ++w) at += B.tmp[w];
+        if (tid < R)
+#pragma unroll 1
+            for (int w = 0; w < W; ++w) col[w * R] = (uint16_t)(col[w * R] + at);
+        __syncthreads();
+#pragma unroll 1
+        for (int p = p0 + lane; p - lane < p1; p += 32) {
+            int cand;
+            const int d = digit(p, cand);
+            const unsigned peers = __match_any_sync(0xffffffffu, d);
+            const int to = d < R ? mine[d] + __popc(peers & ((1u << lane) - 1u)) : 0;
+            __syncwarp();
+            if (d < R && lane == __ffs(peers) - 1) mine[d] += (uint16_t)__popc(peers);
+            if (d < R) dst[to] = (uint16_t)cand;
+            __syncwarp();
+        }
+        uint16_t* const t = src;
+        src = dst;
+        dst = t;
+        shift += D;
+    } while (shift < span);
+    __syncthreads();
+    if (src != B.order) {
+#pragma unroll 1
+        for (int i = tid; i < valid; i += nth) B.order[i] = src[i];
+        __syncthreads();
+    }
+}
+
 // B.order[r] for r < min(want, returned) from B.key[0, M) (visible to the whole CTA when it is
 // called); returns the number of keys other than kNoKey32.  All threads of the CTA take part
 // (a multiple of 32, at most 1024); ends with a barrier.
@@ -640,38 +734,41 @@ __device__ __forceinline__ int bucket_order(const Bucket& B, int M, int want) {
         return valid;
     }
     const int bins = B.bins;
-    // range and number of the keys
-    uint32_t lo = kNoKey32, hi = 0;
-    int cnt = 0;
+    // range and number of the keys; of the ordinary ones
+    uint32_t lo = kNoKey32, hi = 0, hi0 = 0, cnt = 0;  // (cnt: two halves)
     for (int i = tid; i < M; i += nth) {
         const uint32_t k = B.key[i];
         if (k != kNoKey32) {
             lo = min(lo, k);
             hi = max(hi, k);
-            ++cnt;
+            hi0 = k < kOrdinary ? max(hi0, k) : hi0;
+            cnt += k < kOrdinary ? 0x10001u : 1u;
         }
     }
     for (int i = tid; i < bins; i += nth) B.bin[i] = 0;
-    if (tid < 3) B.tmp[32 + tid] = tid == 0 ? kNoKey32 : 0u;
+    if (tid < 4) B.tmp[32 + tid] = tid == 0 ? kNoKey32 : 0u;
     __syncthreads();
     lo = __reduce_min_sync(0xffffffffu, lo);
     hi = __reduce_max_sync(0xffffffffu, hi);
+    hi0 = __reduce_max_sync(0xffffffffu, hi0);
     cnt = __reduce_add_sync(0xffffffffu, cnt);
     if (lane == 0 && cnt) {
         atomicMin(&B.tmp[32], lo);
         atomicMax(&B.tmp[33], hi);
-        atomicAdd(&B.tmp[34], (uint32_t)cnt);
+        atomicMax(&B.tmp[34], hi0);
+        atomicAdd(&B.tmp[35], cnt);
     }
     __syncthreads();
     lo = B.tmp[32];
-    hi = B.tmp[33];
-    const int valid = (int)B.tmp[34];
+    const int valid = (int)(B.tmp[35] & 0xffffu);
+    hi = want <= (int)(B.tmp[35] >> 16) ? B.tmp[34] : B.tmp[33];  // (keys above share the last bin)
     const int span = valid ? 32 - __clz(hi - lo) : 0;  // bits of the range
     const int shift = max(0, span - (31 - __clz(bins)));
+    auto bin_of = [&](uint32_t k) { return min((k - lo) >> shift, (uint32_t)bins - 1u); };
     // bin sizes, their starts (an exclusive scan: a run of bins per thread)
     for (int i = tid; i < M; i += nth) {
         const uint32_t k = B.key[i];
-        if (k != kNoKey32) atomicAdd(&B.bin[(k - lo) >> shift], 1u);
+        if (k != kNoKey32) atomicAdd(&B.bin[bin_of(k)], 1u);
     }
     __syncthreads();
     const int per = (bins + nth - 1) / nth, b0 = min(bins, tid * per), b1 = min(bins, b0 + per);
@@ -687,21 +784,26 @@ __device__ __forceinline__ int bucket_order(const Bucket& B, int M, int want) {
     __syncthreads();
     uint32_t at = inc - sum;
     for (int w = 0; w < warp; ++w) at += B.tmp[w];
+    bool crowded = false;
     for (int i = b0; i < b1; ++i) {
         const uint32_t v = B.bin[i];
         B.bin[i] = at;
+        crowded |= v > kCrowd && (int)at < want;
         at += v;
     }
-    __syncthreads();
+    if (__syncthreads_or(crowded)) {
+        bucket_sort(B, M, valid, lo, hi - lo + 1u);
+        return valid;
+    }
     // the candidates by bin; a bin's entry then holds its end, which is the next one's start
     for (int i = tid; i < M; i += nth) {
         const uint32_t k = B.key[i];
-        if (k != kNoKey32) B.slot[atomicAdd(&B.bin[(k - lo) >> shift], 1u)] = (uint16_t)i;
+        if (k != kNoKey32) B.slot[atomicAdd(&B.bin[bin_of(k)], 1u)] = (uint16_t)i;
     }
     __syncthreads();
     for (int p = tid; p < valid; p += nth) {
         const int i = B.slot[p];
-        const uint32_t k = B.key[i], b = (k - lo) >> shift;
+        const uint32_t k = B.key[i], b = bin_of(k);
         const int s0 = b ? (int)B.bin[b - 1] : 0, s1 = (int)B.bin[b];
         if (s0 >= want) continue;
         int r = s0;

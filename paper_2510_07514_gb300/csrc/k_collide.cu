@@ -504,10 +504,11 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_collide(const CollideAr
 // by k_rank.  A launch of few targets has CTAs of twice the warps, which check
 // the next kWarpsPerBlock candidates too in case the first do not settle it; what
 // they find counts only then.
+// (Registers: three CTAs of 8 warps on an SM, or one of 16.)
 constexpr int kRankWarps = 2 * kWarpsPerBlock;
 template <int SPL, bool UNIFORM, bool GRID>
-__global__ void __launch_bounds__(kRankWarps * 32) k_rank_lazy(const CollideArgs A, const RankArgs R,
-                                                                  uint32_t keys_off, int depth) {
+__global__ void __maxnreg__(SPL <= 2 ? 80 : 128)
+    k_rank_lazy(const CollideArgs A, const RankArgs R, uint32_t keys_off, int depth) {
     extern __shared__ __align__(128) unsigned char smem[];
     grid_follow();
     __shared__ int verdict[kRankWarps];

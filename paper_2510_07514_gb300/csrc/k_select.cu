@@ -20,7 +20,7 @@ constexpr int kSelThreads = 512;
 // Philox draws spread over many SMs.  Bound by latency for few targets, by the draws for many.
 // Time with one CTA sorting all keys and writing all duplicates -> this: one target of 1000 seeds
 // 20 -> 8.8 us, of 2000 seeds and 24 joints 60 -> 11 us, 1000 targets of 1000 seeds 75 -> 51 us.
-__global__ void __launch_bounds__(kSelThreads) k_topk_dup(const DupArgs A) {
+__global__ void __launch_bounds__(kSelThreads, 3) k_topk_dup(const DupArgs A) {
     extern __shared__ __align__(16) unsigned char sel_smem[];
     grid_follow();
     const int t = blockIdx.x;
@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(kSelThreads) k_topk_dup(const DupArgs A) {
     }
 }
 
-__global__ void __launch_bounds__(kSelThreads) k_rank(const RankArgs A) {
+__global__ void __launch_bounds__(kSelThreads, 3) k_rank(const RankArgs A) {
     extern __shared__ __align__(16) unsigned char sel_smem[];
     grid_follow();
     int t = blockIdx.x;
@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(kSelThreads) k_rank(const RankArgs A) {
     if (threadIdx.x == 0) *O.count = count;
 }
 
-__global__ void __launch_bounds__(kSelThreads) k_shard_topk(const ShardTopkArgs A) {
+__global__ void __launch_bounds__(kSelThreads, 4) k_shard_topk(const ShardTopkArgs A) {
     extern __shared__ __align__(16) unsigned char sel_smem[];
     const int t = blockIdx.x;
     const int64_t m0 = A.off[t];
