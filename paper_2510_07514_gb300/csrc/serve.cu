@@ -4,10 +4,10 @@
 // the server and returns at once.  One scheduler thread forms batches from
 // the pending requests in arrival order and launches each batch as a packed
 // solve (wave.cu) on one of max_inflight slots -- a stream with its own device
-// workspace and pinned buffers -- as soon as a slot is free (batches of few
-// seeds a short pace apart, see kPace), so requests that arrive while others
-// run are admitted as slots free up and their work overlaps on the device.  A batch is bounded by max_batch_requests, by
-// max_batch_seeds and by the slot's share of the memory budget (admission by
+// workspace and pinned buffers -- as soon as a slot is free (while others run,
+// batches of few seeds a short pace apart: kPace), so requests that arrive
+// while others run are admitted as slots free up and their work overlaps on
+// the device.  A batch is bounded by max_batch_requests, by max_batch_seeds and by the slot's share of the memory budget (admission by
 // device memory); a request that cannot fit a slot alone fails with
 // HJCD_ENOMEM.  When a batch's copies back to pinned memory complete, a host
 // callback wakes the scheduler, which copies each request's results into its
@@ -79,8 +79,8 @@ struct Server {
     int64_t next_id = 1;
     bool stopping = false;
     std::vector<Slot> slots;
-    bool launched = false;
     Clock::time_point t_last;  // the last batch's launch
+    bool split = false;        // the last batch left requests behind for lack of memory
     std::string fatal;  // first CUDA failure of the scheduler
 
     void run();
@@ -90,14 +90,15 @@ struct Server {
 
 namespace {
 
-// A batch follows the last one by at least kPace while fewer than kFillSeeds seeds per SM are
-// waiting: requests that arrive closely together then share one launch sequence, whose time is
-// mostly the latency of its longest candidate, instead of each taking a slot of its own, while a
-// lone request, or a queue that can fill the GPU, is launched at once.  A burst of 20 requests (1 to 8
-// targets each): 1.69 ms against 1.76 without the pace; a Poisson trace at 2000 requests/s: p50 0.46
-// against 0.36 ms, p99 1.16 against 1.12 ms (1.28 and 1.10 requests per wave); at 4000/s p99 1.52
-// against 1.56 ms, at 8000/s 2.30 against 2.29 ms.
-constexpr std::chrono::microseconds kPace(250);
+// While a batch is on the device, the next one follows its launch by at least kPace if all that waits
+// would fit that one batch with room for more and is fewer than kFillSeeds seeds per SM: requests
+// that arrive closely together then share one launch sequence, whose time is mostly the latency of its
+// longest candidate, instead of each taking a slot of its own.  An idle device, requests that cannot
+// share a batch and a queue that can fill the GPU are never held up.  A burst of 20 requests (1 to 8
+// targets each) without a pace / with 50 / 100 / 250 us: 1.80 / 1.71 / 1.69 / 1.70 ms; a Poisson trace at
+// 2000 requests/s: p50 0.365 / 0.374 / 0.382 / 0.440 ms, p99 1.13 / 1.15 / 1.16 / 1.20 ms (1.05 to 1.26
+// requests per wave); at 4000/s p50 0.440 / 0.448 / 0.468 / 0.576 ms, at 8000/s 0.88 / 0.86 / 0.87 / 0.92.
+constexpr std::chrono::microseconds kPace(100);
 constexpr int64_t kFillSeeds = 64;
 
 struct CbArg {
@@ -200,6 +201,7 @@ bool Server::launch(Slot& sl, std::vector<Req*>& take) {
             {
                 std::lock_guard<std::mutex> lock(mu);
                 pending.push_front(take.back());
+                split = true;
             }
             take.pop_back();
             items.pop_back();
@@ -297,29 +299,30 @@ void Server::run() {
         bool paced = false;
         for (Slot& sl : slots) {
             if (sl.busy || pending.empty()) continue;
-            if (max_requests > 1 && launched && !stopping && Clock::now() < t_last + kPace) {
-                int64_t waiting = 0;
-                for (const Req* r : pending) waiting += r->seeds;
-                if (waiting < kFillSeeds * sm_count() && (int)pending.size() < max_requests) {
-                    paced = true;
-                    break;
-                }
-            }
-            std::vector<Req*> take;
+            // the batch: the oldest requests that fit it
+            size_t count = 0;
             int64_t seeds = 0;
             std::vector<int32_t> robots;
-            while (!pending.empty() && (int)take.size() < max_requests) {
-                Req* r = pending.front();
-                if (!take.empty() && seeds + r->seeds > max_seeds) break;
+            while (count < pending.size() && (int)count < max_requests) {
+                const Req* r = pending[count];
+                if (count && seeds + r->seeds > max_seeds) break;
                 if (std::find(robots.begin(), robots.end(), r->robot_id) == robots.end()) {
                     if ((int)robots.size() == kMaxLaunchRobots) break;
                     robots.push_back(r->robot_id);
                 }
-                pending.pop_front();
-                take.push_back(r);
                 seeds += r->seeds;
+                ++count;
             }
-            launched = true;
+            // all of them, with room for more, while others run: wait for company (kPace)
+            const bool any_busy = std::any_of(slots.begin(), slots.end(), [](const Slot& x) { return x.busy; });
+            if (any_busy && !split && !stopping && count == pending.size() && (int)count < max_requests && seeds < max_seeds &&
+                seeds < kFillSeeds * sm_count() && Clock::now() < t_last + kPace) {
+                paced = true;
+                break;
+            }
+            std::vector<Req*> take(pending.begin(), pending.begin() + count);
+            pending.erase(pending.begin(), pending.begin() + count);
+            split = false;
             t_last = Clock::now();
             lock.unlock();
             launch(sl, take);
