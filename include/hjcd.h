@@ -229,10 +229,12 @@ typedef struct hjcd_tune_report {
 
 /* Autotune on a calibration batch (items as for hjcd_solve_batch; their
  * outputs are not written, top_k is taken as 1).  First every launch
- * configuration is timed and the fastest set on the context; then PO-CCD
- * sweep counts {8, 12, 16, 24, 32, 48} x PJ-IK caps {8, 12, 16, 20, 30} are
- * timed and the fastest pair whose success rate is within success_tol of the
- * best swept rate goes to *tuned (base, or the defaults, with those caps).
+ * configuration is timed and the fastest set on the context (a setting that the
+ * batch's kernels do not use, or that they resolve to the same launch, stays as
+ * it was); then PO-CCD sweep counts {8, 12, 16, 24, 32, 48} x PJ-IK caps
+ * {8, 12, 16, 20, 30} are timed and the fastest pair whose success rate is
+ * within success_tol of the best swept rate goes to *tuned (base, or the
+ * defaults, with those caps).
  * Each configuration: one warm-up and the median of `repeats` (0: 3) solves.
  * The paper tunes nothing; it states its iteration caps as parameters. */
 hjcd_status hjcd_autotune(hjcd_ctx* ctx, int n_items, const hjcd_batch_item* items, const hjcd_params* base,

@@ -1077,6 +1077,10 @@ void launch_sample(const RobotParams& R, uint64_t seed, CandMap map, int64_t C, 
                    cudaStream_t st);
 void launch_ccd(const CcdArgs& A, bool trace, cudaStream_t st);
 int launch_lm(const LmArgs& A, bool trace, cudaStream_t st);  // the number of launches
+// What an untraced launch makes of the context's candidates per CTA / warps per CTA: 0 where it takes
+// a kernel that does not use them (no pointer of A but `list` is looked at).
+int ccd_block_used(const CcdArgs& A, int asked);
+int lm_warps_used(const LmArgs& A, int asked);
 void launch_topk_dup(const DupArgs& A, int max_m, cudaStream_t st);
 void launch_rank(const RankArgs& A, int max_b, cudaStream_t st);
 void launch_collide(const CollideArgs& A, cudaStream_t st);

@@ -1093,6 +1093,16 @@ void launch_ccd_b(const CcdArgs& A, cudaStream_t st) {
 
 }  // namespace
 
+// Whether a launch goes to the spread kernel (explained in launch_ccd)
+static bool ccd_spread(const CcdArgs& A, bool trace) {
+    const bool whole = !trace && A.P.cd_variant == 0 && !A.list_in && A.seg_begin == 0 && A.seg_end == 0;
+    return whole && A.C <= (int64_t)sm_count() * 4 * kCoopCands;
+}
+
+int ccd_block_used(const CcdArgs& A, int asked) {
+    return A.C <= 0 || A.P.cd_variant == 2 || ccd_spread(A, false) ? 0 : asked;
+}
+
 void launch_ccd(const CcdArgs& A, bool trace, cudaStream_t st) {
     if (A.C <= 0) return;
     if (A.P.cd_variant == 2) {  // one CTA per target (offset maps only)
@@ -1103,16 +1113,14 @@ void launch_ccd(const CcdArgs& A, bool trace, cudaStream_t st) {
         k_ccd_lock<128><<<A.map.T, 128, smem, st>>>(A);
         return;
     }
-    const bool whole = !trace && A.P.cd_variant == 0 && !A.list_in && A.seg_begin == 0 && A.seg_end == 0;
     // Up to 64 candidates per SM (two resident CTAs of 16 on every SM, twice) the spread kernel's
     // shorter iterations win; past that its extra work does.  Phase time, spread / one thread per candidate, us (7, 20, 24
     // joints): 1000 candidates 55 / 125, 91 / 267, 106 / 311; 4000: 59 / 125, 118 / 269, 135 / 313;
     // 8000: 109 / 126, 224 / 269, 258 / 313; 16000: 198 / 126, 400 / 272, 464 / 314.  Eight warps (the
     // residual's and seven joint warps), twelve for a long chain while a CTA has its SM to itself
     // (20 joints, 1000 candidates: 99 with eight).
-    const int64_t sms = sm_count();
-    if (whole && A.C <= sms * 4 * kCoopCands) {
-        const int warps = A.rs.n_max > 8 && A.C <= sms * kCoopCands ? 12 : 8;
+    if (ccd_spread(A, trace)) {
+        const int warps = A.rs.n_max > 8 && A.C <= (int64_t)sm_count() * kCoopCands ? 12 : 8;
         if (A.in_limits && A.rs.plain) launch_ccd_coop<false>(A, warps, st);
         else launch_ccd_coop<true>(A, warps, st);
         return;

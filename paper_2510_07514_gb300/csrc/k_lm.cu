@@ -1281,13 +1281,13 @@ void launch_lm_t(const LmArgs& A, cudaStream_t st) {
     k_lm<TRACE, WARPS, RED, HAND><<<g, WARPS * 32, smem, st>>>(A);
 }
 
-template <bool TRACE, bool RED, bool HAND>
-void launch_lm_w(const LmArgs& A, cudaStream_t st) {
+// Warps per CTA of a launch of one lane per candidate for which `asked` are set
+int lm_warps_for(const LmArgs& A, int asked) {
     // fewer warps per CTA when the requested count's state does not fit in shared memory
     int optin = 0;
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, current_device());
     const size_t per_warp = sizeof(float) * (size_t)lm_warp_words(A.rs.n_max, A.P.lm_A);
-    int warps = A.warps == 2 || A.warps == 4 || A.warps == 8 ? A.warps : kLmWarps;
+    int warps = asked == 2 || asked == 4 || asked == 8 ? asked : kLmWarps;
     // a batch too small to give every SM a CTA of two warps (a single target, say): two-warp CTAs,
     // spread over more SMs with shorter lock-step stages (latency, not throughput, is at stake)
     if (A.C <= (int64_t)sm_count() * 64) warps = 2;
@@ -1305,18 +1305,40 @@ void launch_lm_w(const LmArgs& A, cudaStream_t st) {
         const int r = resident(w), r0 = resident(warps);
         if (5 * r >= 6 * r0 || (r >= r0 && r0 <= 8)) warps = w;
     }
+    return warps;
+}
+
+template <bool TRACE, bool RED, bool HAND>
+void launch_lm_w(const LmArgs& A, cudaStream_t st) {
+    const int warps = lm_warps_for(A, A.warps);
     if (warps == 2) launch_lm_t<TRACE, 2, RED, HAND>(A, st);
     else if (warps == 4) launch_lm_t<TRACE, 4, RED, HAND>(A, st);
     else launch_lm_t<TRACE, 8, RED, HAND>(A, st);
 }
 
+// Whether a launch goes, in whole or in its first iterations, to the spread kernel, and whether it leaves
+// candidates to a second launch (both explained in launch_lm)
+struct LmRoute {
+    bool spread, hand;
+};
+LmRoute lm_route(const LmArgs& A, bool trace) {
+    const int64_t sms = sm_count();
+    if (trace || A.P.lm_A > kCoopMaxA || A.C > (A.list ? sms * 216 : sms * 4 * kCoopCands)) return {false, false};
+    const bool hand = A.list && A.C > sms * 2 * kCoopCands;
+    return {A.C <= (hand ? sms * 80 : sms * 4 * kCoopCands), hand};
+}
+
 }  // namespace
+
+int lm_warps_used(const LmArgs& A, int asked) {
+    if (A.C <= 0 || lm_route(A, false).spread) return 0;
+    return lm_warps_for(A, asked);
+}
 
 int launch_lm(const LmArgs& B, bool trace, cudaStream_t st) {
     if (B.C <= 0) return 0;
     LmArgs A = B;
     A.hand_at = A.list_in = A.list_lim = 0;
-    const bool coop = !trace && A.P.lm_A <= kCoopMaxA;
     const bool plain = A.in_limits && A.rs.plain;
     const int64_t sms = sm_count();
     auto lanes = [&]() {
@@ -1342,12 +1364,11 @@ int launch_lm(const LmArgs& B, bool trace, cudaStream_t st) {
     // (7, 12, 20 joints, and 6 joints of which a third run to the cap): 5000: 156 / 102, 219 / 137, 291 /
     // 178, 145 / 104; 8000: 168 / 111, 240 / 154, 322 / 203, 158 / 166; 16000: 248 / 150, 305 / 195, 403 /
     // 254, 276 / 287; 32000: 248 / 205, 334 / 285, 406 / 369, 281 / 295; 48000 no gain.
-    if (!coop || A.C > (A.list ? sms * 216 : sms * 4 * kCoopCands)) {
+    const auto [spread, hand] = lm_route(A, trace);
+    if (!spread && !hand) {
         lanes();
         return 1;
     }
-    const bool hand = A.list && A.C > sms * 2 * kCoopCands;
-    const bool spread = A.C <= (hand ? sms * 80 : sms * 4 * kCoopCands);
     if (hand) A.hand_at = spread ? 4 : 6;
     if (spread) {
         const int warps = A.C <= sms * kCoopCands ? 12 : 8;

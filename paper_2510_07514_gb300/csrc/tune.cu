@@ -3,7 +3,9 @@
 //
 // Step 1 times the batch under every launch configuration (PO-CCD candidates
 // per CTA x PJ-IK warps per CTA; results do not depend on it) and keeps the
-// fastest.  Step 2 sweeps the PO-CCD sweep count and the PJ-IK iteration cap
+// fastest of those that differ: settings that the batch's launches resolve
+// to the same kernels count as one, and what a batch does not use stays as
+// it was (a small one takes kernels that use neither).  Step 2 sweeps the PO-CCD sweep count and the PJ-IK iteration cap
 // and keeps the fastest pair whose success rate (a collision-free solution
 // within the request's tolerances) is within success_tol of the best rate
 // seen.  Each configuration: one warm-up solve, then the median of `repeats`
@@ -148,8 +150,26 @@ hjcd_status hjcd_autotune(hjcd_ctx* ctx, int n_items, const hjcd_batch_item* ite
 
     // step 1: launch configuration
     static const int blocks[3] = {64, 128, 256}, warps[3] = {2, 4, 8};
-    int best_b = blk0, best_w = warps0;
-    double best_ms = 1e300;
+    struct Config {
+        int block, warps, block_used, warps_used;
+        double ms;
+    };
+    std::vector<Config> cfg;
+    CcdArgs ca{};
+    LmArgs la{};
+    {
+        WavePlan W;
+        if ((st = plan_wave(ctx, w.data(), n_items, P0, &W))) {
+            cleanup();
+            return st;
+        }
+        ca.C = W.CM;
+        la.C = W.CB;
+        ca.rs.n = la.rs.n = W.NR;
+        ca.rs.n_max = la.rs.n_max = W.n_max;
+        ca.P = la.P = P0;
+        la.list = reinterpret_cast<int32_t*>(dout);  // a wave always gives one
+    }
     for (int b : blocks)
         for (int wp : warps) {
             ctx->ccd_block = b;
@@ -161,12 +181,26 @@ hjcd_status hjcd_autotune(hjcd_ctx* ctx, int n_items, const hjcd_batch_item* ite
                 cleanup();
                 return st;
             }
-            if (tr.ms < best_ms) {
-                best_ms = tr.ms;
-                best_b = b;
-                best_w = wp;
-            }
+            cfg.push_back({b, wp, ccd_block_used(ca, b), lm_warps_used(la, wp), tr.ms});
         }
+    // the settings that come to the same kernels share the median of their times; of the fastest such
+    // group the one that keeps most of the context's settings
+    auto same = [](const Config& x, const Config& y) { return x.block_used == y.block_used && x.warps_used == y.warps_used; };
+    auto kept = [&](const Config& x) { return (x.block == blk0) + (x.warps == warps0); };
+    const Config* best = nullptr;
+    double best_ms = 1e300;
+    for (const Config& x : cfg) {
+        std::vector<double> ms;
+        for (const Config& y : cfg)
+            if (same(x, y)) ms.push_back(y.ms);
+        std::sort(ms.begin(), ms.end());
+        const double m = ms[ms.size() / 2];
+        if (!best || m < best_ms || (same(x, *best) && kept(x) > kept(*best))) {
+            best = &x;
+            best_ms = m;
+        }
+    }
+    const int best_b = best->block, best_w = best->warps;
     ctx->ccd_block = best_b;
     ctx->lm_warps = best_w;
 
