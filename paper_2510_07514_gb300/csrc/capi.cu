@@ -53,8 +53,10 @@ int pointer_reach(const void* p, int device) {
         cudaGetLastError();
         return 0;
     }
-    if (a.type == cudaMemoryTypeManaged) return 2;
-    if (a.type == cudaMemoryTypeDevice) return a.device == device ? 2 : 1;
+    // (a kernel's loads and stores need their natural alignment, a copy does not)
+    const int here = (reinterpret_cast<uintptr_t>(p) & 3u) == 0 ? 2 : 1;
+    if (a.type == cudaMemoryTypeManaged) return here;
+    if (a.type == cudaMemoryTypeDevice) return a.device == device ? here : 1;
     return 0;
 }
 

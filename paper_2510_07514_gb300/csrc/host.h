@@ -103,7 +103,7 @@ struct Carve {
 
 hjcd_status after_launch(hjcd_ctx* ctx, int kernels, const char* what = "kernel");
 int pointer_kind(const void* p);  // 1 device/managed, 0 host, -1 null
-int pointer_reach(const void* p, int device);  // as pointer_kind, but 2 where kernels on `device` can use p themselves
+int pointer_reach(const void* p, int device);  // as pointer_kind, but 2 where kernels on `device` can use p itself
 bool pinned_host(const void* p);
 hjcd_status make_current(hjcd_ctx* ctx);
 hjcd_status ensure_ws(hjcd_ctx* ctx, size_t bytes);
@@ -157,7 +157,7 @@ struct WavePlan {
     std::vector<SceneEnt> scenes;
     std::vector<int> item_t0;
     std::vector<int64_t> item_q0, item_e0;
-    // per item, pointer_reach of its targets, outputs and reference configurations
+    // per item, pointer_reach of its targets, outputs and reference configurations (1: copied by the stream)
     std::vector<char> at_tgt, at_q, at_e, at_c, at_ref;
     bool has_ref = false;
     int64_t q_total = 0, e_total = 0;

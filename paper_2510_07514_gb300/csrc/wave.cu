@@ -147,7 +147,7 @@ hjcd_status plan_wave(hjcd_ctx* ctx, const WaveItem* items, int n_items, const h
     W.o_io = cv.take<TargetIo>(W.T);
     W.o_inl = cv.take<char>(inl_bytes);
     W.head = cv.off;
-    bool copy_tgt = false, copy_ref = false;  // poses or references of another device
+    bool copy_tgt = false, copy_ref = false;  // poses or references of another device, or not on 4 bytes
     for (int i = 0; i < n_items; ++i) {
         copy_tgt = copy_tgt || W.at_tgt[i] == 1;
         copy_ref = copy_ref || W.at_ref[i] == 1;
@@ -280,7 +280,7 @@ hjcd_status run_wave(hjcd_ctx* ctx, const WavePlan& W, const WaveItem* items, co
             std::memcpy(h_ref + t0 * W.n_max, it.q_ref, sizeof(float) * (size_t)it.T * n);
     }
 
-    // ---- what lies in another device's memory ----
+    // ---- what kernels cannot read in place: another device's memory, or not on 4 bytes ----
     for (int i = 0; i < W.n_items; ++i) {
         const WaveItem& it = items[i];
         if (W.at_tgt[i] == 1)
