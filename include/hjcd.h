@@ -275,10 +275,10 @@ hjcd_status hjcd_solve_from_topk(hjcd_ctx* ctx, int32_t robot_id, int32_t scene_
  * paper has no serving layer).  One scheduler thread packs the pending
  * requests, in arrival order, into batches (one launch per phase, as
  * hjcd_solve_batch) and runs each batch on one of max_inflight streams as
- * soon as one is free (while others run, a batch of few seeds with room for more
- * at least a tenth of a millisecond after the last): requests arriving while
- * others run are admitted as streams and memory free up, and their work
- * overlaps on the device.  A
+ * soon as one is free (while others run and requests come close together, a batch
+ * of few seeds with room for more at least a quarter of a millisecond after the
+ * last): requests arriving while others run are admitted as streams and memory
+ * free up, and their work overlaps on the device.  A
  * batch holds at most max_batch_requests requests, max_batch_seeds PO-CCD
  * seeds and memory_budget / max_inflight bytes of device workspace; a request
  * that does not fit that share alone fails with HJCD_ENOMEM.  Zero fields take

@@ -4,12 +4,12 @@
 // the server and returns at once.  One scheduler thread forms batches from
 // the pending requests in arrival order and launches each batch as a packed
 // solve (wave.cu) on one of max_inflight slots -- a stream with its own device
-// workspace and pinned buffers -- as soon as a slot is free (while others run,
-// batches of few seeds a short pace apart: kPace), so requests that arrive
+// workspace and pinned buffers -- as soon as a slot is free (batches of few
+// seeds may wait for company while others run: kPace), so requests that arrive
 // while others run are admitted as slots free up and their work overlaps on
-// the device.  A batch is bounded by max_batch_requests, by max_batch_seeds and by the slot's share of the memory budget (admission by
-// device memory); a request that cannot fit a slot alone fails with
-// HJCD_ENOMEM.  When a batch's copies back to pinned memory complete, a host
+// the device.  A batch is bounded by max_batch_requests, by max_batch_seeds
+// and by the slot's share of the memory budget (admission by device memory);
+// a request that cannot fit a slot alone fails with HJCD_ENOMEM.  When a batch's copies back to pinned memory complete, a host
 // callback wakes the scheduler, which copies each request's results into its
 // caller's buffers and marks it done.
 #include <algorithm>
@@ -81,6 +81,10 @@ struct Server {
     std::vector<Slot> slots;
     Clock::time_point t_last;  // the last batch's launch
     bool split = false;        // the last batch left requests behind for lack of memory
+    Clock::time_point t_arrival;  // the last request's
+    Clock::duration gap{}, gap_mean{};  // between the last two; of the recent ones (kPace says how)
+
+    void arrived(Clock::time_point now);
     std::string fatal;  // first CUDA failure of the scheduler
 
     void run();
@@ -91,15 +95,27 @@ struct Server {
 namespace {
 
 // While a batch is on the device, the next one follows its launch by at least kPace if all that waits
-// would fit that one batch with room for more and is fewer than kFillSeeds seeds per SM: requests
-// that arrive closely together then share one launch sequence, whose time is mostly the latency of its
-// longest candidate, instead of each taking a slot of its own.  An idle device, requests that cannot
-// share a batch and a queue that can fill the GPU are never held up.  A burst of 20 requests (1 to 8
-// targets each) without a pace / with 50 / 100 / 250 us: 1.80 / 1.71 / 1.69 / 1.70 ms; a Poisson trace at
-// 2000 requests/s: p50 0.365 / 0.374 / 0.382 / 0.440 ms, p99 1.13 / 1.15 / 1.16 / 1.20 ms (1.05 to 1.26
-// requests per wave); at 4000/s p50 0.440 / 0.448 / 0.468 / 0.576 ms, at 8000/s 0.88 / 0.86 / 0.87 / 0.92.
-constexpr std::chrono::microseconds kPace(100);
+// would fit that one batch with room for more, is fewer than kFillSeeds seeds per SM, and company is
+// likely: requests have lately arrived less than kPace apart on average (each counts a quarter, a gap
+// at most kGapMost), or the last two within kBurst.  They then share one launch sequence, whose time is
+// mostly the latency of its longest candidate, instead of each taking a slot of its own.  An idle device,
+// requests that cannot share a batch, those far apart and a queue that can fill the GPU are never held up.
+// A burst of 20 requests (1 to 8 targets each) without a pace / with this: 1.80 / 1.69 ms; a Poisson trace
+// at 1000 requests/s p50 0.350 / 0.346 ms, at 2000 0.372 / 0.376 (1.09 requests per batch), at 4000 0.441 /
+// 0.556, at 8000 0.87 / 0.95 (3.6); p99 at 4000 1.52 / 1.56, at 8000 2.14 / 2.20.
+constexpr std::chrono::microseconds kPace(250), kBurst(30), kGapMost(1000);
 constexpr int64_t kFillSeeds = 64;
+
+}  // namespace
+
+void Server::arrived(Clock::time_point now) {
+    if (t_arrival == Clock::time_point{}) gap_mean = kGapMost;
+    gap = std::min<Clock::duration>(now - t_arrival, kGapMost);
+    gap_mean += (gap - gap_mean) / 4;
+    t_arrival = now;
+}
+
+namespace {
 
 struct CbArg {
     Server* sv;
@@ -315,8 +331,9 @@ void Server::run() {
             }
             // all of them, with room for more, while others run: wait for company (kPace)
             const bool any_busy = std::any_of(slots.begin(), slots.end(), [](const Slot& x) { return x.busy; });
-            if (any_busy && !split && !stopping && count == pending.size() && (int)count < max_requests && seeds < max_seeds &&
-                seeds < kFillSeeds * sm_count() && Clock::now() < t_last + kPace) {
+            const bool company = gap_mean < kPace || gap < kBurst;
+            if (any_busy && company && !split && !stopping && count == pending.size() && (int)count < max_requests &&
+                seeds < max_seeds && seeds < kFillSeeds * sm_count() && Clock::now() < t_last + kPace) {
                 paced = true;
                 break;
             }
@@ -476,6 +493,7 @@ hjcd_status hjcd_submit(hjcd_ctx* ctx, const hjcd_batch_item* req, int64_t* requ
         if (sv->stopping) return fail(ctx, HJCD_EINVAL, "the server is stopping");
         r->id = sv->next_id++;
         *request_id = r->id;
+        sv->arrived(Clock::now());
         sv->pending.push_back(r.get());
         sv->reqs.emplace(r->id, std::move(r));
     }
