@@ -1093,10 +1093,11 @@ void launch_ccd_b(const CcdArgs& A, cudaStream_t st) {
 
 }  // namespace
 
+constexpr int kCoopShort = 4;  // joints up to which the spread kernel gains little
 // Whether a launch goes to the spread kernel (explained in launch_ccd)
 static bool ccd_spread(const CcdArgs& A, bool trace) {
     const bool whole = !trace && A.P.cd_variant == 0 && !A.list_in && A.seg_begin == 0 && A.seg_end == 0;
-    return whole && A.C <= (int64_t)sm_count() * 4 * kCoopCands;
+    return whole && A.C <= (int64_t)sm_count() * (A.rs.n_max <= kCoopShort ? 2 : 4) * kCoopCands;
 }
 
 int ccd_block_used(const CcdArgs& A, int asked) {
@@ -1114,8 +1115,10 @@ void launch_ccd(const CcdArgs& A, bool trace, cudaStream_t st) {
         return;
     }
     // Up to 64 candidates per SM (two resident CTAs of 16 on every SM, twice) the spread kernel's
-    // shorter iterations win; past that its extra work does.  Phase time, spread / one thread per candidate, us (7, 20, 24
-    // joints): 1000 candidates 55 / 125, 91 / 267, 106 / 311; 4000: 59 / 125, 118 / 269, 135 / 313;
+    // shorter iterations win; past that its extra work does, and for a chain of up to four joints, which
+    // leaves little to spread, past 32 (one to four joints, 9000 candidates: 101 / 61, 104 / 72, 107 / 85,
+    // 109 / 96 us; 4800: 55 / 61 to 57 / 96; five joints 112 / 110).  Phase time, spread / one thread per
+    // candidate, us (7, 20, 24 joints): 1000 candidates 55 / 125, 91 / 267, 106 / 311; 4000: 59 / 125, 118 / 269, 135 / 313;
     // 8000: 109 / 126, 224 / 269, 258 / 313; 16000: 198 / 126, 400 / 272, 464 / 314.  Eight warps (the
     // residual's and seven joint warps), twelve for a long chain while a CTA has its SM to itself
     // (20 joints, 1000 candidates: 99 with eight).

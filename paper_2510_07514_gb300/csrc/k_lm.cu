@@ -1323,9 +1323,10 @@ struct LmRoute {
 };
 LmRoute lm_route(const LmArgs& A, bool trace) {
     const int64_t sms = sm_count();
-    if (trace || A.P.lm_A > kCoopMaxA || A.C > (A.list ? sms * 216 : sms * 4 * kCoopCands)) return {false, false};
+    const int64_t most = sms * (A.list ? 216 : (A.rs.n_max == 1 ? 2 : 4) * kCoopCands);
+    if (trace || A.P.lm_A > kCoopMaxA || A.C > most) return {false, false};
     const bool hand = A.list && A.C > sms * 2 * kCoopCands;
-    return {A.C <= (hand ? sms * 80 : sms * 4 * kCoopCands), hand};
+    return {!hand || A.C <= sms * 80, hand};
 }
 
 }  // namespace
@@ -1353,8 +1354,10 @@ int launch_lm(const LmArgs& B, bool trace, cudaStream_t st) {
     // shorter iterations win; past that its extra work does.  Phase time of the polish, spread /
     // one lane per candidate, us (7, 20, 24 joints): 1000 candidates 70 / 172, 115 / 328, 129 / 360;
     // 4000: 84 / 200, 164 / 346, 178 / 356; 8000: 166 / 221, 322 / 346, 338 / 356; 16000: 311 / 240,
-    // 594 / 395, 616 / 363 (the last two with loads not yet ahead of the stores, 3 to 6% of its time).  Twelve warps while a CTA has its SM to itself (8: 76, 139, 150), eight
-    // (two CTAs per SM) beyond.
+    // 594 / 395, 616 / 363 (the last two with loads not yet ahead of the stores, 3 to 6% of its time).  A
+    // single joint leaves nothing to spread: up to 32 per SM (9000 candidates 151 / 95, 4800: 84 / 97; two
+    // joints 161 / 176).  Twelve warps while a CTA has its SM to itself (8: 76, 139, 150), eight (two CTAs
+    // per SM) beyond.
     //
     // Where the caller gives a list, batches of up to 216 candidates per SM leave the candidates that
     // need more than a few iterations to a second launch, packed afresh: most candidates converge
