@@ -571,10 +571,10 @@ inline int grid_for(int64_t items, int per_block, int per_sm = 64) {
 // Keys that crowd a bin would cost their square: equal scores (every seed of an invalid target scores
 // infinity, so a padding row of a batch does that), a few distinct ones, or scores squeezed together by
 // keys far away.  The bins therefore span the ordinary keys only (finite and non-negative; not the NaN
-// of the top-K, not the ranking's class 1) where those hold every wanted rank, and a pass that finds more
-// than kCrowd keys in a bin with a wanted rank leaves the order to a radix sort.  The top quarter of 8192
-// scores, 600 targets: spread 445 us, all equal 268 (by their square 9460), 20% NaN 451; all of them in
-// order: 397, 308, 511.  16 targets of 8192 seeds, eight of them padding rows: a solve 5340 -> 684 us.
+// of the top-K, not the ranking's class 1) where those hold every wanted rank, and where the comparisons
+// within the bins that hold wanted ranks would take longer than sorting these bins' keys (crowd_limit), a radix
+// sort does that.  The top quarter of 8192 scores, 600 targets: spread 445 us, all equal 268 (by their
+// square 9460), 20% NaN 451.  16 targets of 8192 seeds, eight of them padding rows: a solve 5340 -> 684 us.
 
 constexpr uint32_t kNoKey32 = 0xffffffffu;  // never ranked
 constexpr int kMaxBins = 2048;
@@ -588,7 +588,9 @@ __device__ __forceinline__ uint32_t score_bits(float s) {
 // grow with the square, and at 256 keys they are the longer way).  COUNT = false leaves that out, for
 // the collision-aware ranking, whose registers it takes past 80 and so a third CTA off each SM.
 constexpr int kCountKeys = 128;
-constexpr int kCrowd = 128;  // more are sorted: 128 in every bin take about as long as the sort
+// Comparisons that take as long as the sort, which costs about 6 us and 1.7 ns a key (measured with one
+// CTA per SM; a comparison takes 36 ps)
+__device__ __forceinline__ uint32_t crowd_limit(int M) { return 160000u + 48u * (uint32_t)M; }
 constexpr uint32_t kOrdinary = 0x7f800000u;  // keys below are finite non-negative scores (of class 0)
 
 // bins of a pass over M keys
@@ -621,12 +623,12 @@ __device__ __forceinline__ Bucket bucket_of(void* smem, int M) {
     return B;
 }
 
-// The crowded case of bucket_order: a radix sort of the `valid` candidates with a key, by
-// min(key - lo, top) and then index.  Each pass takes a digit; a warp ranks its contiguous part of the
+// The crowded case of bucket_order: a radix sort of the `count` candidates whose key lies in [lo, lo + top]
+// by key and then index.  Each pass takes a digit; a warp ranks its contiguous part of the
 // sequence 32 at a time by matching digits, so the order is stable and the time does not depend on
 // the keys.  (Digits of up to 8 bits, as the warps' counts fit the bins' memory; equal keys take one
 // pass.)  Not inlined: it is rarely taken, and the callers' registers and code stay as they are.
-__device__ __forceinline__ void bucket_sort(const Bucket B, int M, int valid, uint32_t lo, uint32_t top) {
+__device__ __forceinline__ void bucket_sort(const Bucket B, int M, int count, uint32_t lo, uint32_t top) {
     const int tid = threadIdx.x, nth = blockDim.x, lane = tid & 31, warp = tid >> 5, W = nth >> 5;
     int D = 8;
     while ((W << D) > 2 * B.bins || (1 << D) > nth) --D;
@@ -635,14 +637,14 @@ __device__ __forceinline__ void bucket_sort(const Bucket B, int M, int valid, ui
     uint16_t *src = B.slot, *dst = B.order;
     int shift = 0;
     do {
-        const bool first = shift == 0;  // the candidates in index order, those without a key left out
-        const int n = first ? M : valid;
+        const bool first = shift == 0;  // the candidates in index order, the others left out
+        const int n = first ? M : count;
         const int part = ((n + W - 1) / W + 31) & ~31, p0 = min(n, warp * part), p1 = min(n, p0 + part);
         // this lane's candidate at p and its digit (R: none)
         auto digit = [&](int p, int& cand) {
             cand = p < p1 ? (first ? p : (int)src[p]) : 0;
             const uint32_t k = p < p1 ? B.key[cand] : kNoKey32;
-            return k != kNoKey32 ? (int)(min(k - lo, top) >> shift & (uint32_t)(R - 1)) : R;
+            return k != kNoKey32 && k - lo <= top ? (int)((k - lo) >> shift & (uint32_t)(R - 1)) : R;
         };
         __syncthreads();
 #pragma unroll 1
@@ -701,7 +703,7 @@ __device__ __forceinline__ void bucket_sort(const Bucket B, int M, int valid, ui
     __syncthreads();
     if (src != B.order) {
 #pragma unroll 1
-        for (int i = tid; i < valid; i += nth) B.order[i] = src[i];
+        for (int i = tid; i < count; i += nth) B.order[i] = src[i];
         __syncthreads();
     }
 }
@@ -781,18 +783,30 @@ __device__ __forceinline__ int bucket_order(const Bucket& B, int M, int want) {
         if (lane >= o) inc += v;
     }
     if (lane == 31) B.tmp[warp] = inc;
+    if (tid < 3) B.tmp[32 + tid] = 0;
     __syncthreads();
     uint32_t at = inc - sum;
     for (int w = 0; w < warp; ++w) at += B.tmp[w];
-    bool crowded = false;
+    uint32_t pairs = 0, last = 0, end = 0;  // comparisons in the bins with a wanted rank; the last such bin, its end
     for (int i = b0; i < b1; ++i) {
         const uint32_t v = B.bin[i];
         B.bin[i] = at;
-        crowded |= v > kCrowd && (int)at < want;
+        if (v && (int)at < want) {
+            pairs += v * v;
+            last = i;
+            end = at + v;
+        }
         at += v;
     }
-    if (__syncthreads_or(crowded)) {
-        bucket_sort(B, M, valid, lo, hi - lo + 1u);
+    if (end) {
+        atomicAdd(&B.tmp[32], pairs);
+        atomicMax(&B.tmp[33], last);
+        atomicMax(&B.tmp[34], end);
+    }
+    __syncthreads();
+    if (B.tmp[32] > crowd_limit(M)) {
+        last = B.tmp[33];  // (keys past the range share the last bin)
+        bucket_sort(B, M, (int)B.tmp[34], lo, (int)last < bins - 1 ? ((last + 1u) << shift) - 1u : kNoKey32 - 1u - lo);
         return valid;
     }
     // the candidates by bin; a bin's entry then holds its end, which is the next one's start
