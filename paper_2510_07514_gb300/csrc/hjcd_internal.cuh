@@ -883,14 +883,14 @@ struct LmArgs {
     int32_t in_limits;  // 1: every joint vector the launch reads lies within its robot's limits
     // Where a launch leaves the candidates that need more than its first iterations to the next one
     // (null: nowhere): their indices and iteration counts [C] and how many there are (zero at launch).
-    // hand_at (set by launch_lm; 0: never): the iteration after which it does.
+    // hand_at (set by launch_lm; 0: never): the iteration after which it does, at the earliest, hand_lim: how
+    // many unfinished candidates it leaves at most (one lane per candidate), n_done: how many are finished
+    // (zero at launch).
     int32_t* list;
     int32_t* list_k;
     int32_t* n_list;
-    unsigned long long* queue2;  // the queue head of a launch over the list, zero
-    int32_t hand_at;
-    int32_t list_in;  // set by launch_lm; 1: the launch runs the list's candidates, when there are more than list_lim
-    int32_t list_lim;
+    int32_t* n_done;
+    int32_t hand_at, hand_lim;
 };
 
 struct DupArgs {

@@ -227,7 +227,7 @@ struct LmCta {
     int* fl;
     int* pl;
     int* np;
-    int* drained;  // some lane found the queue empty
+    int* hand;  // the CTA leaves its candidates to the next launch
 };
 template <int WARPS>
 __host__ __device__ constexpr int lm_cta_words() { return WARPS + 2 * WARPS * 32 + 2; }
@@ -438,7 +438,8 @@ __device__ __noinline__ void dogleg_prepare(const LmW S, int l, int n, float Rt,
 
 // RED = false: the launch's joint vectors lie within the limits of plain robots (no offsets and
 // no range reduction in the kinematics steps; the same bits)
-// HAND: the launch leaves candidates to a later one (hand_at) or runs those that were left (list_in)
+// HAND: the launch leaves its last candidates to the next one: each CTA, from its hand_at-th iteration
+// on, once the queue is empty and hand_lim candidates of the launch or fewer are unfinished
 template <bool TRACE, int WARPS, bool RED, bool HAND>
 __global__ void __launch_bounds__(WARPS * 32, 16 / WARPS) k_lm(const LmArgs A) {
     extern __shared__ __align__(16) float smem_f[];
@@ -453,7 +454,7 @@ __global__ void __launch_bounds__(WARPS * 32, 16 / WARPS) k_lm(const LmArgs A) {
     auto slot_state = [&](int sl) { return LmW{warps_f + (sl >> 5) * words, A.rs.n_max}; };
     const LmCta<WARPS> CL = lm_cta<WARPS>(warps_f + WARPS * words);
     if (HAND) {
-        if (threadIdx.x == 0) CL.drained[0] = 0;
+        if (threadIdx.x == 0) CL.hand[0] = 0;
         __syncthreads();
     }
 
@@ -461,29 +462,29 @@ __global__ void __launch_bounds__(WARPS * 32, 16 / WARPS) k_lm(const LmArgs A) {
     const float Rt = P.lm_trust_R;
     unsigned long long n_it = 0, n_fk = 0, n_sc = 0;
 
-    const bool list = HAND && A.list_in;
-    const int64_t items = list ? (int64_t)*A.n_list : A.C;
-    if (list && items <= A.list_lim) return;  // few: the spread kernel's
     bool has = false;
     int rounds = 0;
-    int64_t qi = 0, c = 0;  // place in the queue, candidate
+    int64_t c = 0;
     int32_t t = 0, s = 0, kk = 0, cap = 0;
     TargetDesc T{};
 
     for (;;) {
         // refill idle lanes from the global queue (one atomic per warp)
         const unsigned need = __ballot_sync(0xffffffffu, !has);
+        if (HAND) {  // those whose candidate is finished
+            const unsigned fin = __ballot_sync(0xffffffffu, !has && rounds > 0 && c < A.C);
+            if (fin && lane == 0) atomicAdd(A.n_done, __popc(fin));
+        }
         if (need) {
             const int leader = __ffs(need) - 1;
             long long base = 0;
-            if (lane == leader) base = (long long)atomicAdd(list ? A.queue2 : A.queue, (unsigned long long)__popc(need));
+            if (lane == leader) base = (long long)atomicAdd(A.queue, (unsigned long long)__popc(need));
             base = __shfl_sync(0xffffffffu, base, leader);
             if (!has) {
-                qi = base + __popc(need & ((1u << lane) - 1u));
-                c = list && qi < items ? (int64_t)A.list[qi] : qi;
-                if (qi < items && A.map.lookup(c, t, s)) {
+                c = base + __popc(need & ((1u << lane) - 1u));
+                if (c < A.C && A.map.lookup(c, t, s)) {
                     T = A.tg[t];
-                    kk = list ? A.list_k[qi] : 0;
+                    kk = 0;
                     cap = A.n_iters >= 0 ? A.n_iters : T.lm_iters;
                     if (T.eps_pos > 0.0f) {
                         has = true;
@@ -619,10 +620,12 @@ __global__ void __launch_bounds__(WARPS * 32, 16 / WARPS) k_lm(const LmArgs A) {
         // (the same barrier ends the loop once no lane holds a candidate and the queue is drained)
         const unsigned fail = __ballot_sync(0xffffffffu, failed);
         if (lane == 0) CL.wm[warp] = fail;
-        // (a lane whose candidate just finished still holds a place below the end and asks again)
-        if (HAND && qi >= items) CL.drained[0] = 1;
-        if (!__syncthreads_or(has || qi < items)) break;
-        const bool drained = HAND && CL.drained[0] != 0;  // some lane asked in vain: no candidate is left in the queue
+        // (a lane whose candidate just finished still holds an index below C and asks again)
+        if (HAND && threadIdx.x == 0 && rounds + 1 >= A.hand_at)
+            CL.hand[0] = *(volatile const unsigned long long*)A.queue >= (unsigned long long)A.C &&
+                         A.C - *(volatile const int32_t*)A.n_done <= A.hand_lim;
+        if (!__syncthreads_or(has || c < A.C)) break;
+        const bool hand = HAND && CL.hand[0] != 0;
         int nf = 0, before = 0;
 #pragma unroll
         for (int w = 0; w < WARPS; ++w) {
@@ -746,7 +749,8 @@ __global__ void __launch_bounds__(WARPS * 32, 16 / WARPS) k_lm(const LmArgs A) {
             ++n_it;
         }
         __syncwarp();
-        if (HAND && A.hand_at > 0 && ++rounds >= A.hand_at && drained) {
+        if (HAND) ++rounds;
+        if (hand) {
             // the candidates that are left, packed afresh, take less time in the kernel that spreads a
             // candidate over a CTA
             const unsigned m = __ballot_sync(0xffffffffu, has);
@@ -909,7 +913,6 @@ __global__ void __launch_bounds__(kCoopLmWarps * 32, 1) k_lm_coop(const LmArgs A
     entry(u, a0, b0);  // (u < 32)
     entry(min(u + U, 41), a1, b1);
     const int64_t items = LIST ? (int64_t)*A.n_list : A.C;
-    if (LIST && items > A.list_lim) return;  // too many: the other kernel's
     for (int64_t base = kCoopCands * (int64_t)blockIdx.x; base < items; base += kCoopCands * (int64_t)gridDim.x) {
         __syncthreads();  // the last group's state is no longer read
         int32_t t = 0, s = 0;
@@ -1316,6 +1319,7 @@ void launch_lm_w(const LmArgs& A, cudaStream_t st) {
     else launch_lm_t<TRACE, 8, RED, HAND>(A, st);
 }
 
+constexpr int kCoopShort = 3;  // joints of a chain that one lane polishes quickly
 // Whether a launch goes, in whole or in its first iterations, to the spread kernel, and whether it leaves
 // candidates to a second launch (both explained in launch_lm)
 struct LmRoute {
@@ -1326,7 +1330,7 @@ LmRoute lm_route(const LmArgs& A, bool trace) {
     const int64_t most = sms * (A.list ? 216 : (A.rs.n_max == 1 ? 2 : 4) * kCoopCands);
     if (trace || A.P.lm_A > kCoopMaxA || A.C > most) return {false, false};
     const bool hand = A.list && A.C > sms * 2 * kCoopCands;
-    return {!hand || A.C <= sms * 80, hand};
+    return {!hand || (A.C <= sms * 80 && A.rs.n_max > kCoopShort), hand};
 }
 
 }  // namespace
@@ -1339,11 +1343,11 @@ int lm_warps_used(const LmArgs& A, int asked) {
 int launch_lm(const LmArgs& B, bool trace, cudaStream_t st) {
     if (B.C <= 0) return 0;
     LmArgs A = B;
-    A.hand_at = A.list_in = A.list_lim = 0;
+    A.hand_at = A.hand_lim = 0;
     const bool plain = A.in_limits && A.rs.plain;
     const int64_t sms = sm_count();
     auto lanes = [&]() {
-        const bool hand = A.hand_at > 0 || A.list_in;
+        const bool hand = A.hand_at > 0;
         if (trace) launch_lm_w<true, true, false>(A, st);
         else if (hand && plain) launch_lm_w<false, false, true>(A, st);
         else if (hand) launch_lm_w<false, true, true>(A, st);
@@ -1360,19 +1364,25 @@ int launch_lm(const LmArgs& B, bool trace, cudaStream_t st) {
     // per SM) beyond.
     //
     // Where the caller gives a list, batches of up to 216 candidates per SM leave the candidates that
-    // need more than a few iterations to a second launch, packed afresh: most candidates converge
-    // in those, and the rest (a fifth of Panda's run to the cap of 20) fit the spread kernel.  Up to 80 per
-    // SM four iterations of the spread kernel, beyond six of one lane per candidate; more than 64 per
-    // SM left (a chain that rarely reaches its targets) go on with one lane each.  One launch / two, us
-    // (7, 12, 20 joints, and 6 joints of which a third run to the cap): 5000: 156 / 102, 219 / 137, 291 /
-    // 178, 145 / 104; 8000: 168 / 111, 240 / 154, 322 / 203, 158 / 166; 16000: 248 / 150, 305 / 195, 403 /
-    // 254, 276 / 287; 32000: 248 / 205, 334 / 285, 406 / 369, 281 / 295; 48000 no gain.
+    // need more than a few iterations to a second launch of the spread kernel, packed afresh: most candidates
+    // converge in those, and the rest (a fifth of Panda's run to the cap of 20) fit it.  Up to 80 per SM four
+    // iterations of the spread kernel; beyond, and for a chain of up to three joints, six of one lane per
+    // candidate, and on until no more than 64 per SM are unfinished: a chain that rarely reaches its targets
+    // may never get there, and then one launch does it all.  One launch / two, us, the quarter of the seeds
+    // duplicated: 7 joints 8000: 252 / 106, 16000: 250 / 141, 32000: 248 / 207; 12 joints 285 / 149, 291 / 180,
+    // 293 / 252; 20 joints 381 / 203, 389 / 235, 406 / 373; 6 joints of which a third run to the cap 270 / 156,
+    // 293 / 266, 283 / 283.  Every seed polished (a ratio of 1): 7 joints 305 / 160, 324 / 270, 338 / 336; 6 joints
+    // 289 / 158, 328 / 338, 330 / 340.  (Handing over at six iterations whatever was left, and only in CTAs
+    // with a lane that had asked the queue in vain, the last two took 534 and 503.)  48000 no gain.
     const auto [spread, hand] = lm_route(A, trace);
     if (!spread && !hand) {
         lanes();
         return 1;
     }
-    if (hand) A.hand_at = spread ? 4 : 6;
+    if (hand) {
+        A.hand_at = spread ? 4 : 6;
+        A.hand_lim = (int32_t)(sms * 4 * kCoopCands);
+    }
     if (spread) {
         const int warps = A.C <= sms * kCoopCands ? 12 : 8;
         if (plain) launch_lm_coop<false, false>(A, warps, st);
@@ -1382,13 +1392,9 @@ int launch_lm(const LmArgs& B, bool trace, cudaStream_t st) {
     }
     if (!hand) return 1;
     A.hand_at = 0;
-    A.list_lim = spread ? 0x7fffffff : (int)(sms * 4 * kCoopCands);
     if (plain) launch_lm_coop<false, true>(A, 8, st);
     else launch_lm_coop<true, true>(A, 8, st);
-    if (spread) return 2;
-    A.list_in = 1;
-    lanes();
-    return 3;
+    return 2;
 }
 
 }  // namespace hjcd

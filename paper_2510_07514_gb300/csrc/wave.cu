@@ -169,7 +169,7 @@ hjcd_status plan_wave(hjcd_ctx* ctx, const WaveItem* items, int n_items, const h
     W.o_ul = cv.take<int32_t>(W.T);           // targets left to the second collision pass
     W.o_sg = cv.take<int32_t>(2 * (size_t)W.CM);  // PO-CCD candidates handed between segments
     // queue head, PJ-IK's count of o_sg, count of o_ul, PO-CCD's counts of o_sg, its segments' queue heads;
-    // PJ-IK's second queue head
+    // PJ-IK's count of finished candidates
     W.o_qf = cv.take<unsigned long long>(7);
     W.bytes = cv.off;
 
@@ -390,7 +390,7 @@ hjcd_status run_wave(hjcd_ctx* ctx, const WavePlan& W, const WaveItem* items, co
     la.list = reinterpret_cast<int32_t*>(ws + W.o_sg);  // PO-CCD is done with its lists
     la.list_k = la.list + W.CM;
     la.n_list = reinterpret_cast<int32_t*>(ws + W.o_qf + 8);
-    la.queue2 = queue + 6;
+    la.n_done = reinterpret_cast<int32_t*>(queue + 6);
     if ((st = after_launch(ctx, launch_lm(la, false, s), "k_lm"))) return st;
     if (ev) HJCD_CUDA(ctx, cudaEventRecord(ev[3], s));
 

@@ -65,3 +65,36 @@ def test_a_smaller_batch_takes_no_longer(ctx, stage, which):
     above = run(most)
     for per_sm in (32, 48, 64):
         assert run(per_sm * sms) <= 1.08 * above + 2, per_sm  # (the clock, and the candidates' own spread)
+
+
+@pytest.mark.parametrize("ratio", [1, 4])
+@pytest.mark.parametrize("which", ["random0", "random3", "chain7", "chain12"])
+def test_a_smaller_polish_takes_no_longer(ctx, which, ratio):
+    """The polish of a mid-size batch leaves its last candidates to a second launch; of a chain that often
+    runs to the cap, or with every seed polished, that must not take longer than the one launch of a
+    batch past those sizes (216 candidates per SM)."""
+    rob = inputs.cfg3_chains()[int(which[6:])] if which.startswith("random") else inputs.dof_scaling_robot(int(which[5:]))
+    rob.sph_body, rob.sph_xyzr = rob.sph_body[:0], rob.sph_xyzr[:0]
+    rid = ctx.add_robot(rob)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    most = 216 * sms // 1000 + 2
+    tg = ctx.fk(rid, torch.as_tensor(inputs.joint_samples(np.random.default_rng(16), rob, most).T.copy(), dtype=torch.float32,
+                                     device="cuda"))
+    params = api.make_params(dup_ratio=ratio)
+
+    def polish_us(T):
+        part = tg[:T].contiguous()
+        ctx.solve(rid, -1, part, 1000, 1, 5, rob.n, params=params)
+        us = []
+        for _ in range(7):
+            ctx.solve(rid, -1, part, 1000, 1, 5, rob.n, params=params)
+            us.append(1e3 * hjcd.hjcd_phase_times(ctx.h)[2])
+        return float(np.median(us))
+
+    hjcd.hjcd_set_profiling(ctx.h, 1)
+    try:
+        above = polish_us(most)
+        for T in (8, 12, 16, 20, 24, most - 2):
+            assert polish_us(T) <= 1.08 * above + 5, T
+    finally:
+        hjcd.hjcd_set_profiling(ctx.h, 0)
