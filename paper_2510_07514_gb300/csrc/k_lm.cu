@@ -1257,7 +1257,12 @@ void launch_lm_coop_n(const LmArgs& A, int warps, cudaStream_t st) {
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lm_coop<RED, N, LIST>, 32 * warps, smem);
     const int g = (int)std::min<int64_t>((A.C + kCoopCands - 1) / kCoopCands, (int64_t)sm_count() * std::max(per_sm, 1));
-    launch_next<LmArgs>(k_lm_coop<RED, N, LIST>, g, 32 * warps, smem, st, A);
+    // Set up while the kernel before still runs -- but where CTAs outnumber the SMs, they are then placed
+    // among that kernel's, unevenly, which the long iterations of long chains show: 24 joints, 5000 / 8000 /
+    // 10000 candidates, a solve 453 / 494 / 586 us so, 428 / 469 / 549 launched after it; 18 joints 387 / 419 / 484
+    // and 369 / 402 / 479; 12 joints 297 / 318 / 358 and 285 / 320 / 361; 7 joints 223 and 225 us at 7000.
+    if (g > sm_count() && A.rs.n_max > 8) k_lm_coop<RED, N, LIST><<<g, 32 * warps, smem, st>>>(A);
+    else launch_next<LmArgs>(k_lm_coop<RED, N, LIST>, g, 32 * warps, smem, st, A);
 }
 
 template <bool RED, bool LIST>
