@@ -685,8 +685,8 @@ void launch_collide_s(const CollideArgs& A, int n_obj4, cudaStream_t st) {
 // mostly the walk over near obstacles, whose counts differ between lanes.  With a whole warp on each
 // candidate that has such a pair, a chain whose bodies crowd one another gained nothing (200k
 // candidates without obstacles, link sphere tests by warp / by lane, us: Panda 111 / 86, 12 joints
-// 583 / 433, 20 joints 2115 / 933; a warp per candidate from the start 228, 612 and 1258).
-// 400k Panda configurations, 60 link spheres, 220 obstacles (27% free): 307 us, where a warp per
+// 583 / 430, 20 joints 2115 / 922; a warp per candidate from the start 228, 612 and 1258).
+// 400k Panda configurations, 60 link spheres, 220 obstacles (27% free): 309 us, where a warp per
 // candidate takes 835 us.
 constexpr int kCells = 6;           // per axis
 constexpr int kLaneList = 12;       // overlapping obstacles a lane holds before it tests them
@@ -718,6 +718,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, PER_SM) k_collide_lane(co
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ float s_lo[3], s_inv[3];
     __shared__ uint32_t s_pair[kMaxBodies];  // bit a of entry b: bodies a < b are checked for self-collision
+    __shared__ unsigned long long s_cnt[3];  // sphere tests, box tests, candidates
     __shared__ int s_all;  // the box of the obstacles is not finite: no cells, every obstacle is near
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const SceneDev sc0 = A.n_scenes > 0 ? A.scenes[0] : SceneDev{nullptr, 0, 0};
@@ -749,6 +750,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, PER_SM) k_collide_lane(co
         lrange[i] = __ldg(rd.range + i);
     }
     if (tid < nb) s_pair[tid] = 0;
+    if (tid < 3) s_cnt[tid] = 0;
     __syncthreads();
     for (int i = tid; i < n_pairs; i += blockDim.x) {
         const int2 pr = __ldg(rd.pairs + i);
@@ -823,7 +825,6 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, PER_SM) k_collide_lane(co
     }
     __syncthreads();
 
-    unsigned long long tests = 0, btests = 0, ncand = 0;
     const bool all = s_all != 0;
     const int64_t nwarps = (int64_t)gridDim.x * kWarpsPerBlock;
     for (int64_t c0 = 32 * ((int64_t)blockIdx.x * kWarpsPerBlock + warp); c0 < A.C; c0 += 32 * nwarps) {
@@ -962,22 +963,22 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, PER_SM) k_collide_lane(co
             }
             body(b, F);
         }
-        if (have) {
-            A.hit[c] = hit ? 1 : 0;
-            ++ncand;
+        if (have) A.hit[c] = hit ? 1 : 0;
+        if (A.cnt) {  // (in shared memory: as 64-bit sums of a thread they would cost the walks registers)
+            t_s = __reduce_add_sync(0xffffffffu, t_s);
+            t_b = __reduce_add_sync(0xffffffffu, t_b);
+            if (lane == 0) {
+                atomicAdd(&s_cnt[0], (unsigned long long)t_s);
+                atomicAdd(&s_cnt[1], (unsigned long long)t_b);
+                atomicAdd(&s_cnt[2], (unsigned long long)min((int64_t)32, A.C - c0));
+            }
         }
-        tests += t_s;
-        btests += t_b;
     }
-    if (A.cnt) {
-        tests = warp_sum(tests);
-        btests = warp_sum(btests);
-        ncand = warp_sum(ncand);
-        if (lane == 0) {
-            atomicAdd(&A.cnt->v[3], tests);
-            atomicAdd(&A.cnt->v[6], btests);
-            atomicAdd(&A.cnt->v[4], ncand);
-        }
+    __syncthreads();
+    if (A.cnt && tid == 0) {
+        atomicAdd(&A.cnt->v[3], s_cnt[0]);
+        atomicAdd(&A.cnt->v[6], s_cnt[1]);
+        atomicAdd(&A.cnt->v[4], s_cnt[2]);
     }
 }
 
@@ -996,9 +997,9 @@ bool launch_collide_lane(const CollideArgs& A, cudaStream_t st) {
     const size_t smem = lane_layout(L.warp, A.rs.ns_max, A.u_n + 2, words).total;
     if (smem > 220 * 1024) return false;
     constexpr int kThreads = kWarpsPerBlock * 32;
-    // Four CTAs per SM (64 registers, a few spilled) for a short chain and more candidates than three
-    // hold at once, else three (80): 400k Panda configurations among 220 obstacles 351 -> 343 us, 200k of 6
-    // joints among 110 218 -> 210; 100k of them 140 -> 145, 200k of 20 joints without obstacles 940 -> 1031.
+    // Four CTAs per SM (64 registers) for a short chain and more candidates than three hold at once, else
+    // three (80): 400k Panda configurations among 220 obstacles 353 -> 343 us, 200k of 6 joints among 110 218 ->
+    // 210; 200k of 20 joints without obstacles 923 -> 1006, 65536 of 12 joints 181 -> 203.
     if (A.u_n <= kLaneLong && A.C > (int64_t)sm_count() * 3 * kThreads) {
         const int per_sm = lane_ctas<4>(smem);
         if (per_sm > 3) {
