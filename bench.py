@@ -724,8 +724,8 @@ def serving_leg(ctx, args, dev):
 
     The served path runs the whole trace at 2000 requests/s.  The plain path is
     swept: halved rates on short runs until its p99 is no worse than the served
-    p99 (the bracket), then rates 1.25x apart across the bracket with at least
-    2000 requests each, repeated on other stretches of the trace; in each repeat
+    p99 (the bracket), then rates 1.25x apart from just below the bracket across
+    it with at least 2000 requests each, repeated on other stretches of the trace; in each repeat
     the rate (and throughput) at which the plain p99 equals the served p99 is
     interpolated, and served/plain solves/s at equal p99 is its ratio.  Both
     paths are also run at 2x and 4x the offered rate (their ceilings)."""
@@ -778,7 +778,7 @@ def serving_leg(ctx, args, dev):
         start = (rep * n_req) % max(1, len(idx) - n_req)
         sub = idx[start:start + n_req]
         pts, runs = [], []
-        for i in range(1, 5):  # the bracket's low point met the target on a short run
+        for i in range(-1, 5):  # from below the bracket's low point, which met the target on a short run
             sc = scale * 1.25 ** i
             r = _serve_run(ctx, reqs, trace, sub, sc, plain_kw)
             r["rate_scale"] = sc

@@ -2,11 +2,12 @@
 //
 // The batch is planned and given its own device workspace and pinned image;
 // one ordinary run (which also sets the kernels' attributes) precedes the
-// capture of the same launch sequence on a private stream.  A replay copies
-// the pinned image (robot and scene tables, target rows, offsets) and the
-// targets from the callers' device buffers, runs every phase and copies each
-// request's results to its device buffers, so changing the targets between
-// replays re-solves the new poses with everything else fixed.
+// capture of the same launch sequence on a private stream.  A replay's first
+// kernel reads the pinned image (robot and scene tables, target rows, offsets)
+// and the targets from the callers' device buffers, the phases run, and the
+// last kernel writes each request's results into its device buffers, so
+// changing the targets between replays re-solves the new poses with everything
+// else fixed.
 #include "host.h"
 
 struct hjcd_graph {

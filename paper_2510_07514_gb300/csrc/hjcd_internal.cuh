@@ -910,7 +910,8 @@ struct DupArgs {
 };
 
 // Where a wave's target comes from and where its results go: its pose and reference configuration
-// (device or pinned host memory; null: no reference) and its blocks of the outputs (device memory).
+// (device or pinned host memory; null: no reference) and its blocks of the outputs (the caller's device
+// memory, the workspace, or the wave's pinned buffer).
 struct TargetIo {
     const float* pose;  // [7]
     const float* ref;   // [n]

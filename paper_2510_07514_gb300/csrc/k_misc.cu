@@ -53,8 +53,9 @@ __device__ __forceinline__ void fk_pose(const RobotParams& R, const Frame2& F, i
 // Bound by the issue of the chain's arithmetic until two candidates share a thread as packed pairs
 // (a joint's constants are then broadcast once for two candidates and no component is left over for
 // a scalar instruction); the angles are loaded eight joints at a time and a warp's 64 poses go out
-// through shared memory as contiguous 16-byte stores.  1M Panda poses (56 MB): 26.6 us with one
-// candidate per thread, an angle load per step and 28-byte strides, 18.4 us now.
+// through shared memory as contiguous 16-byte stores.  1M Panda poses (56 MB, which stay in the L2 from
+// pass to pass): 26.6 us with one candidate per thread, an angle load per step and 28-byte strides, 18.4
+// us now; with the L2 flushed before each pass 30.7 -> 20.4 us.
 __global__ void __launch_bounds__(kFkThreads) k_fk(const RobotParams R, int64_t C, const float* th_in, int64_t ld,
                                                    float* out, int wide) {
     __shared__ __align__(16) float tile[2 * kFkThreads * 7];
