@@ -92,6 +92,15 @@ __device__ __forceinline__ float4 to_world(const Frame& F, float4 s) {
     return make_float4(w.x, w.y, w.z, s.w);
 }
 
+// to_world by the frame of lane src
+__device__ __forceinline__ float4 to_world_of(const Frame& F, int src, float4 s) {
+    auto of = [&](const V3 v) {
+        return v3(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src), __shfl_sync(0xffffffffu, v.z, src));
+    };
+    const V3 w = fma3(s.z, of(F.c2), fma3(s.y, of(F.c1), fma3(s.x, of(F.c0), of(F.p))));
+    return make_float4(w.x, w.y, w.z, s.w);
+}
+
 __device__ __forceinline__ bool sph_sph(float4 a, float4 b) {
     const float dx = a.x - b.x, dy = a.y - b.y, dz = a.z - b.z, rr = a.w + b.w;
     return fmaf(dx, dx, fmaf(dy, dy, dz * dz)) < rr * rr;
@@ -680,21 +689,22 @@ void launch_collide_s(const CollideArgs& A, int n_obj4, cudaStream_t st) {
 // lane's list and are then tested against the body's link spheres.  Pairs of bodies are tested by lane
 // as well: bounding sphere against bounding sphere, the later body's link spheres against the earlier
 // one's bounding sphere, and where both overlap link sphere against link sphere, for which the warp
-// walks the chain again up to the earlier body (its frames would not fit shared memory).  The tests
-// that decide are the other kernel's, on the same spheres, so the verdicts are equal.  Bound by issue,
-// mostly the walk over near obstacles, whose counts differ between lanes.  With a whole warp on each
-// candidate that has such a pair, a chain whose bodies crowd one another gained nothing (200k
-// candidates without obstacles, link sphere tests by warp / by lane, us: Panda 111 / 86, 12 joints
-// 583 / 430, 20 joints 2115 / 922; a warp per candidate from the start 228, 612 and 1258).
-// 400k Panda configurations, 60 link spheres, 220 obstacles (27% free): 309 us, where a warp per
-// candidate takes 835 us.
+// walks the chain again up to the earlier body (its frames would not fit shared memory): by the lanes
+// that have the pair, or, where those are few, by the whole warp for one after another.  The tests that
+// decide are the other kernel's, on the same spheres, so the verdicts are equal.  Bound by issue, mostly
+// the walk over near obstacles, whose counts differ between lanes.  200k candidates without obstacles, us:
+// a warp per candidate 228 (Panda), 612 (12 joints), 1258 (20 joints); here with the warp routine's whole self
+// test for each candidate with such a pair 111, 583, 2115; with the pairs tested by lane 86, 428, 922; as it
+// is 76, 301, 623.  400k Panda configurations, 60 link spheres, 220 obstacles (27% free): 294 us, where a
+// warp per candidate takes 835 us.
 constexpr int kCells = 6;           // per axis
 constexpr int kLaneList = 12;       // overlapping obstacles a lane holds before it tests them
-constexpr int64_t kLaneMinCands = 32768, kLaneMinCandsLong = 49152;
-constexpr int kLaneLong = 8, kLaneFewObjs = 64;  // joints above and obstacles below which the latter counts
+constexpr int64_t kLaneMinCands = 32768;
+constexpr int kLaneShort = 8;       // joints up to which four CTAs per SM are taken
 constexpr int kLaneMaxWords = 16;   // obstacles: 32 per word of a cell's mask, spheres and boxes in words of their own
 static_assert(kCells * kCells * kCells <= kWarpsPerBlock * 32, "a cell per thread");
 constexpr float kSmallBody = 0.6f;  // bounding radii up to this part of the largest have masks of their own
+constexpr int kFewLanes = 4;  // candidates of a warp whose pair of bodies the whole warp tests, one after another
 constexpr float kFewUlps = 4e-7f, kSomeUlps = 1e-6f;  // of a coordinate: the margins for its rounding
 
 struct LaneLayout {
@@ -933,8 +943,25 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, PER_SM) k_collide_lane(co
             for (int a = 0; left; ++a) {
                 if (a > 0) fk_step(R, a - 1, have ? A.th[(a - 1) * A.ld + c] : 0.0f, G);
                 if (!(left >> a & 1u)) continue;
-                if (pairs >> a & 1u) {
-                    const int2 ra = lrange[a];
+                const int2 ra = lrange[a];
+                unsigned who = __ballot_sync(0xffffffffu, pairs >> a & 1u);
+                if (__popc(who) <= kFewLanes) {  // the warp tests one lane's spheres at a time
+                    const int items = ra.y * rg.y;
+                    const float per = __fdividef(1.0f, (float)rg.y);
+                    for (; who; who &= who - 1u) {
+                        const int src = __ffs(who) - 1;
+                        bool h = false;
+                        for (int w0 = 0; w0 < items; w0 += 32) {
+                            const int w = min(w0 + lane, items - 1), k = (int)(((float)w + 0.5f) * per);
+                            h |= sph_sph(to_world_of(G, src, lsph[ra.x + k]), to_world_of(F, src, lsph[rg.x + w - k * rg.y]));
+                        }
+                        h = __any_sync(0xffffffffu, h);
+                        if (lane == src) {
+                            hit = h;
+                            t_s += items;
+                        }
+                    }
+                } else if (pairs >> a & 1u) {
                     const float4 ca = widen(bound(a));
 #pragma unroll 1
                     for (int i = rg.x; i < rg.x + rg.y && !hit; ++i) {
@@ -997,10 +1024,11 @@ bool launch_collide_lane(const CollideArgs& A, cudaStream_t st) {
     const size_t smem = lane_layout(L.warp, A.rs.ns_max, A.u_n + 2, words).total;
     if (smem > 220 * 1024) return false;
     constexpr int kThreads = kWarpsPerBlock * 32;
-    // Four CTAs per SM (64 registers) for a short chain and more candidates than three hold at once, else
-    // three (80): 400k Panda configurations among 220 obstacles 353 -> 343 us, 200k of 6 joints among 110 218 ->
-    // 210; 200k of 20 joints without obstacles 923 -> 1006, 65536 of 12 joints 181 -> 203.
-    if (A.u_n <= kLaneLong && A.C > (int64_t)sm_count() * 3 * kThreads) {
+    // Four CTAs per SM (64 registers, a few spilled) for a short chain and more candidates than three hold
+    // at once, else three (80): 400k Panda configurations among 220 obstacles 353 -> 343 us, 200k of 6 joints
+    // among 110 218 -> 210; 200k of 20 joints without obstacles 923 -> 1006, 65536 of 12 joints 181 -> 203
+    // (before the warp took part in the pairs' tests).
+    if (A.u_n <= kLaneShort && A.C > (int64_t)sm_count() * 3 * kThreads) {
         const int per_sm = lane_ctas<4>(smem);
         if (per_sm > 3) {
             k_collide_lane<4><<<grid_for(A.C, kThreads, per_sm), kThreads, smem, st>>>(A);
@@ -1083,14 +1111,11 @@ void launch_collide(const CollideArgs& A, cudaStream_t st) {
     const bool uni = A.uniform && A.rs.n == 1 && A.n_scenes <= 1 && A.max_obj4 <= kMaxStagedObj4;
     const int n4 = A.n_scenes == 1 ? A.max_obj4 : 0;
     // From 32768 candidates on, a candidate per lane: below, its 32 candidates per warp leave the GPU
-    // underfilled; from 49152 on for a long chain among few obstacles, whose time is the pairs' tests and
-    // their latency.  us, by lane / by warp: Panda with 60 spheres, 32768 candidates: no obstacles 53 / 66,
-    // 110: 80 / 100; 6 joints, 73 spheres: 54 / 90, 92 / 146; 12 joints, 127 spheres: 154 / 134, 20 obstacles
-    // 166 / 149, 110: 167 / 193; 20 joints, 197 spheres: 307 / 265, 295 / 286, 251 / 323, and at 49152
-    // 12 joints 179 / 180, 20 joints 385 / 367, 110 obstacles 269 / 454.
+    // underfilled.  us, by lane / by warp, 32768 candidates: Panda with 60 spheres, no obstacles 54 / 74, 110
+    // obstacles 78 / 99; 6 joints, 73 spheres 55 / 92, 92 / 147; 12 joints, 127 spheres 100 / 134, 138 / 196; 20
+    // joints, 197 spheres 198 / 266, 194 / 324.  (Panda among 220 obstacles, 16000: 100 / 74.)
     const int words = (A.u_osph + 31) / 32 + (A.u_obox + 31) / 32;
-    const int64_t from = A.u_n > kLaneLong && A.u_osph + A.u_obox < kLaneFewObjs ? kLaneMinCandsLong : kLaneMinCands;
-    if (uni && !A.has_grid && !A.list && words <= kLaneMaxWords && A.C >= from && launch_collide_lane(A, st)) return;
+    if (uni && !A.has_grid && !A.list && words <= kLaneMaxWords && A.C >= kLaneMinCands && launch_collide_lane(A, st)) return;
     if (uni && A.has_grid) launch_collide_s<true, true>(A, n4, st);
     else if (uni) launch_collide_s<true, false>(A, n4, st);
     else if (A.has_grid) launch_collide_s<false, true>(A, 0, st);

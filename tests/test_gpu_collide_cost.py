@@ -1,5 +1,5 @@
-"""The collision filter's time over its two kernels: a candidate has a lane in large sets (from 32768 or
-49152 candidates on) and a warp below.  The change must not make a set cost more than its size, whatever
+"""The collision filter's time over its two kernels: a candidate has a lane in large sets (from 32768
+candidates on) and a warp below.  The change must not make a set cost more than its size, whatever
 the robot: chains whose bodies crowd one another leave many body pairs to the link spheres' tests."""
 import numpy as np
 import pytest
